@@ -482,7 +482,7 @@ int pprviz_layout_metrics(pprviz_ctx *ctx, const void *x, int32_t k, const pprvi
  *             energy and the status word. No context is needed: the call runs
  *             on the current device, in its primary context (the one the CUDA
  *             runtime API uses).
- * Scratch: a fixed device array inside the library (about 528 KiB, held by
+ * Scratch: a fixed device array inside the library (about 517 KiB, held by
  * every GPU that loads the library until the process exits), so k is limited
  * to 65,536. The first call on a device looks up the array's device address
  * in that device's primary context (once per device, with that device

@@ -33,9 +33,6 @@ namespace pprviz {
 
 constexpr int ST = 128;       // symmetric pass tile edge
 constexpr int SRPI = 8;       // rows per warp per sub-iteration in the symmetric pass
-constexpr int LWARPS = 8;     // warps per block in the energy pass
-constexpr int RPW = 4;        // rows per warp in the energy pass
-constexpr int XCH = 1024;     // coordinates staged per shared-memory chunk (energy)
 
 template <typename T> struct T2;
 template <> struct T2<float> { using type = float2; };
@@ -714,84 +711,227 @@ __global__ void k_finish(int32_t k, const typename T2<T>::type *__restrict__ X, 
 //   energy += e^2 (halved at the end: Eq. (7) sums i < j)
 //   grad_x_i += -2 e u / d (x_i - x_j)      (0 when d = 0)
 //   grad_pdist_ij = e d u^2
-// Each block writes its FP64 energy partial; k_reduce_energy adds them in order.
+//
+// A block owns ERPB rows at a time (block-stride over row groups, at most
+// EBLOCKS blocks) and its 256 threads share the columns, so a view of a few
+// thousand nodes already fills the GPU; the coordinates (8 k bytes) come from
+// L1. The pass is meant to be bound by reading Delta (and writing
+// grad_pdist). What it must not spend is GB300's FP64 pipe (2 operations per
+// cycle and SM): one FP64 add and one conversion per pair alone cost five
+// times the read. In FP32 the squares e^2 are therefore summed as a float and
+// its exact rounding errors (TwoSum, Knuth), two rows at a time with the
+// paired FP32 instructions, and converted once per thread; the sum is as
+// exact as the FP64 sum it replaces (~2^-46). 1/Delta and 1/d come from the
+// special-function unit, each followed by one Newton step (Newton's iteration
+// for a^-1 and a^-1/2), which leaves them within about an ulp. Pairs outside
+// the range in which those steps are safe (coincident or extremely close
+// points, huge or tiny values, infinities, NaN, the diagonal) and a last
+// group of fewer than ERPB rows take the plain formulas.
+// Measured at k = 8,192 on one GB300 (read 268 MB, write 268 MB with
+// grad_pdist), before -> now: energy alone 572 -> 95 us, both gradients
+// 692 -> 142 us. It now issues ~30 instructions per pair, most of them on
+// the FMA pipe, and waits on loads for the rest.
 // ---------------------------------------------------------------------------
+constexpr int ERPB = 4;                 // rows of a row group
+constexpr int ETHREADS = 256;           // threads per block
+constexpr int EBLOCKS = 608;            // blocks (and FP64 partials) at most: four per SM, so that the FP64
+                                        // reduction at a block's end runs once per several row groups
+inline unsigned energy_blocks(int64_t k) {
+  return (unsigned)std::min<int64_t>((k + ERPB - 1) / ERPB, EBLOCKS);
+}
+
+// per-thread energy sums: a paired float sum with its rounding errors (FP32
+// pairs on the fast path) and an FP64 sum (everything else)
+template <typename T>
+struct EAcc {
+  float2 s = make_float2(0.0f, 0.0f), c = make_float2(0.0f, 0.0f);
+  double d = 0.0;
+  __device__ __forceinline__ void add2(float2 q) {  // TwoSum, both halves
+    const float2 n = make_float2(-1.0f, -1.0f);
+    const float2 t = __fadd2_rn(s, q);
+    const float2 bb = __ffma2_rn(n, s, t);                       // t - s
+    const float2 e0 = __ffma2_rn(n, __ffma2_rn(n, bb, t), s);    // s - (t - bb)
+    const float2 e1 = __ffma2_rn(n, bb, q);                      // q - bb
+    c = __fadd2_rn(c, __fadd2_rn(e0, e1));
+    s = t;
+  }
+  __device__ __forceinline__ double total() const {
+    return d + (((double)s.x + (double)s.y) + ((double)c.x + (double)c.y));
+  }
+};
+
+// one pair by the plain formulas; row i, column j
 template <typename T, bool GX, bool GD>
-__global__ void __launch_bounds__(LWARPS * 32)
+__device__ __forceinline__ void energy_pair(int64_t i, int64_t j, int64_t k, T del, T dx, T dy, T scale, double &eacc,
+                                            T &gxx, T &gxy, T *__restrict__ gD, int &bad) {
+  if (i == j) {
+    if (GD) gD[i * k + j] = T(0);
+    return;
+  }
+  if (!(del > T(0))) bad = 1;
+  const T d = sqrt(dx * dx + dy * dy);
+  const T u = T(1) / del;
+  const T e = T(1) - d * u;
+  eacc += (double)(e * e);
+  if (GX && d > T(0)) {
+    const T coef = T(-2) * e * u / d;
+    gxx += coef * dx;
+    gxy += coef * dy;
+  }
+  if (GD) gD[i * k + j] = scale * e * d * u * u;
+}
+
+// All of a, b, c, d in [2^lo, 2^hi], as bit patterns of positive floats (zero,
+// negative and NaN values fall outside).
+__device__ __forceinline__ bool all_in_range(const float (&v)[4], int lo, int hi) {
+  const int a = __float_as_int(v[0]), b = __float_as_int(v[1]), c = __float_as_int(v[2]), d = __float_as_int(v[3]);
+  return min(min(a, b), min(c, d)) >= ((127 + lo) << 23) && max(max(a, b), max(c, d)) <= ((127 + hi) << 23);
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+template <typename T, bool GX, bool GD>
+__global__ void __launch_bounds__(ETHREADS, std::is_same<T, float>::value ? 4 : 2)
 k_energy(int32_t k, const T *__restrict__ Delta, const typename T2<T>::type *__restrict__ X, T scale,
          double *__restrict__ eparts, T *__restrict__ gx, T *__restrict__ gD, int *__restrict__ flag) {
   using V2 = typename T2<T>::type;
-  __shared__ V2 sv[XCH];
-  __shared__ double se[LWARPS];
+  constexpr int WARPS = ETHREADS / 32;
+  constexpr int QCH = 32;  // columns per thread between two runs of the plain formulas (bits of `plain`)
+  __shared__ double se[WARPS];
+  __shared__ T sg[WARPS][2 * ERPB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int64_t rows[RPW];
-  T xi[RPW], yi[RPW], gxx[RPW], gxy[RPW];
-  double eacc = 0.0;
+  EAcc<T> acc;
   int bad = 0;
+  for (int64_t r0 = (int64_t)blockIdx.x * ERPB; r0 < k; r0 += (int64_t)gridDim.x * ERPB) {
+    const int nr = (int)min((int64_t)ERPB, k - r0);
+    const T *D0 = Delta + r0 * k;
+    V2 xi[ERPB];
+    T gxx[ERPB], gxy[ERPB];
 #pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    rows[r] = ((int64_t)blockIdx.x * LWARPS + warp) * RPW + r;
-    gxx[r] = T(0);
-    gxy[r] = T(0);
-    xi[r] = T(0);
-    yi[r] = T(0);
-    if (rows[r] < k) {
-      xi[r] = X[rows[r]].x;
-      yi[r] = X[rows[r]].y;
+    for (int r = 0; r < ERPB; ++r) {
+      xi[r] = X[min((int)r0 + r, k - 1)];
+      gxx[r] = gxy[r] = T(0);
     }
-  }
-  for (int64_t c0 = 0; c0 < k; c0 += XCH) {
-    const int cn = (int)min((int64_t)XCH, (int64_t)k - c0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cn; t += blockDim.x) sv[t] = X[c0 + t];
-    __syncthreads();
-    for (int t = lane; t < cn; t += 32) {
-      const V2 xj = sv[t];
-      const int64_t j = c0 + t;
+    for (int64_t c0 = threadIdx.x; c0 < k; c0 += QCH * ETHREADS) {
+      const int nq = (int)min((int64_t)QCH, (k - c0 + ETHREADS - 1) / ETHREADS);
+      uint32_t plain = nq == QCH ? 0xffffffffu : (1u << nq) - 1u;  // columns left to the plain formulas
+      if constexpr (std::is_same<T, float>::value) {
+        if (nr == ERPB) {
+          const float2 n = make_float2(-1.0f, -1.0f), one = make_float2(1.0f, 1.0f), half = make_float2(0.5f, 0.5f);
+          const T *Dc = D0 + c0;
+          const V2 *Xc = X + c0;
+          const int jd = (int)(r0 - c0);  // columns jd .. jd + 3 (from c0) hold the diagonal
+          // the next column's loads are in flight while a column is computed
+          float nd[ERPB];
+          V2 nx = Xc[0];
 #pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        const int64_t i = rows[r];
-        if (i >= k) continue;
-        if (i == j) {
-          if (GD) gD[i * k + j] = T(0);
-          continue;
+          for (int r = 0; r < ERPB; ++r) nd[r] = __ldcs(Dc + (int64_t)r * k);
+#pragma unroll 2
+          for (int q = 0; q < nq; ++q) {
+            float del[ERPB], d2a[ERPB];
+            const V2 xj = nx;
+#pragma unroll
+            for (int r = 0; r < ERPB; ++r) del[r] = nd[r];
+            if (q + 1 < nq) {
+              nx = Xc[(q + 1) * ETHREADS];
+#pragma unroll
+              for (int r = 0; r < ERPB; ++r) nd[r] = __ldcs(Dc + (int64_t)r * k + (q + 1) * ETHREADS);
+            }
+            float2 dx[ERPB / 2], dy[ERPB / 2], d2[ERPB / 2];
+            const float2 xj2 = make_float2(xj.x, xj.x), yj2 = make_float2(xj.y, xj.y);
+#pragma unroll
+            for (int p = 0; p < ERPB / 2; ++p) {  // rows 2p, 2p + 1
+              dx[p] = __ffma2_rn(n, xj2, make_float2(xi[2 * p].x, xi[2 * p + 1].x));
+              dy[p] = __ffma2_rn(n, yj2, make_float2(xi[2 * p].y, xi[2 * p + 1].y));
+              d2[p] = __ffma2_rn(dx[p], dx[p], __fmul2_rn(dy[p], dy[p]));
+              d2a[2 * p] = d2[p].x;
+              d2a[2 * p + 1] = d2[p].y;
+            }
+            if (!all_in_range(d2a, -80, 40) || !all_in_range(del, -20, 60) ||
+                (unsigned)(q * ETHREADS - jd) < (unsigned)ERPB)
+              continue;
+            plain &= ~(1u << q);
+#pragma unroll
+            for (int p = 0; p < ERPB / 2; ++p) {
+              const float2 dl = make_float2(del[2 * p], del[2 * p + 1]);
+              const float2 u0 = make_float2(rcp_approx(dl.x), rcp_approx(dl.y));
+              const float2 y0 = make_float2(rsqrt_approx(d2[p].x), rsqrt_approx(d2[p].y));
+              // u0 + u0 (1 - Delta u0)
+              const float2 u = __ffma2_rn(__ffma2_rn(__fmul2_rn(n, dl), u0, one), u0, u0);
+              const float2 s0 = __fmul2_rn(d2[p], y0);
+              // d = s0 + (d2 - s0^2) / (2 s0), 1 / s0 ~ y0
+              const float2 res = __ffma2_rn(__fmul2_rn(n, s0), s0, d2[p]);
+              const float2 d = __ffma2_rn(__fmul2_rn(half, y0), res, s0);
+              const float2 e = __ffma2_rn(__fmul2_rn(n, d), u, one);
+              acc.add2(__fmul2_rn(e, e));
+              if (GX) {
+                // 1 / d = y0 + y0 (1 - d y0)
+                const float2 y = __ffma2_rn(__ffma2_rn(__fmul2_rn(n, d), y0, one), y0, y0);
+                const float2 cf = __fmul2_rn(__fmul2_rn(make_float2(-2.0f, -2.0f), e), __fmul2_rn(u, y));
+                const float2 gX = __ffma2_rn(cf, dx[p], make_float2(gxx[2 * p], gxx[2 * p + 1]));
+                const float2 gY = __ffma2_rn(cf, dy[p], make_float2(gxy[2 * p], gxy[2 * p + 1]));
+                gxx[2 * p] = gX.x;
+                gxx[2 * p + 1] = gX.y;
+                gxy[2 * p] = gY.x;
+                gxy[2 * p + 1] = gY.y;
+              }
+              if (GD) {  // ((scale e) d u) u, the order of the plain formula
+                const float2 g = __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(make_float2(scale, scale), e), d), u), u);
+                T *o = gD + (r0 + 2 * p) * k + c0 + q * ETHREADS;
+                __stcs(o, g.x);
+                __stcs(o + k, g.y);
+              }
+            }
+          }
         }
-        const T del = Delta[i * k + j];
-        if (!(del > T(0))) bad = 1;
-        const T dx = xi[r] - xj.x, dy = yi[r] - xj.y;
-        const T d = sqrt(dx * dx + dy * dy);
-        const T u = T(1) / del;
-        const T e = T(1) - d * u;
-        eacc += (double)(e * e);
-        if (GX && d > T(0)) {
-          const T coef = T(-2) * e * u / d;
-          gxx[r] += coef * dx;
-          gxy[r] += coef * dy;
-        }
-        if (GD) gD[i * k + j] = scale * e * d * u * u;
       }
-    }
-  }
-  if (GX) {
+      while (plain) {
+        const int q = __ffs((int)plain) - 1;
+        plain &= plain - 1u;
+        const int64_t j = c0 + q * ETHREADS;
+        const V2 xj = X[j];
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      T vx = gxx[r], vy = gxy[r];
-      for (int o = 16; o > 0; o >>= 1) {
-        vx += __shfl_xor_sync(0xffffffffu, vx, o);
-        vy += __shfl_xor_sync(0xffffffffu, vy, o);
-      }
-      if (lane == 0 && rows[r] < k) {
-        gx[2 * rows[r]] = scale * vx;
-        gx[2 * rows[r] + 1] = scale * vy;
+        for (int r = 0; r < ERPB; ++r)
+          if (r < nr)
+            energy_pair<T, GX, GD>(r0 + r, j, k, D0[(int64_t)r * k + j], xi[r].x - xj.x, xi[r].y - xj.y, scale, acc.d,
+                                   gxx[r], gxy[r], gD, bad);
       }
     }
+    if (GX) {
+      T v[2 * ERPB];
+#pragma unroll
+      for (int r = 0; r < ERPB; ++r) {
+        v[2 * r] = gxx[r];
+        v[2 * r + 1] = gxy[r];
+      }
+      const T tot = lanes_transpose_sum<2 * ERPB, T>(v, lane);
+      constexpr int REP = 32 / (2 * ERPB);
+      if (lane % REP == 0) sg[warp][lane / REP] = tot;
+      __syncthreads();
+      if (threadIdx.x < 2 * ERPB && r0 + (threadIdx.x >> 1) < k) {
+        T s = T(0);
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) s += sg[w][threadIdx.x];
+        gx[2 * r0 + threadIdx.x] = scale * s;
+      }
+      __syncthreads();  // before the next group's sums
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) eacc += __shfl_xor_sync(0xffffffffu, eacc, o);
-  if (lane == 0) se[warp] = eacc;
+  double e = acc.total();
+  for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (lane == 0) se[warp] = e;
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < LWARPS; ++w) s += se[w];
+    for (int w = 0; w < WARPS; ++w) s += se[w];
     eparts[blockIdx.x] = s;
   }
   if (bad) atomicOr(flag, 1);
@@ -1090,7 +1230,7 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   ctx->stats.bytes_ly = half * iters;
   ctx->stats.bytes_apply = half * iters;
   if (stress_h) {
-    const unsigned eb = (unsigned)((k + LWARPS * RPW - 1) / (LWARPS * RPW));
+    const unsigned eb = energy_blocks(k);
     PPRVIZ_TRY(ws_ensure(ctx, WS_OUT1, sizeof(double) * (eb + 1)));
     double *ep = ctx->ws[WS_OUT1].as<double>();
     // stress of the final layout on the input pdist (Eq. (7)), in the path's arithmetic
@@ -1102,7 +1242,7 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
       PPRVIZ_LAUNCHED(ctx);
       Dt = Dw;
     }
-    { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_energy<T, false, false><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, Dt, Xc, T(1), ep, nullptr, nullptr, flag); }
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_energy<T, false, false><<<eb, ETHREADS, 0, ctx->stream>>>(k, Dt, Xc, T(1), ep, nullptr, nullptr, flag); }
     PPRVIZ_LAUNCHED(ctx);
     { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_reduce_energy<<<1, 256, 0, ctx->stream>>>((int)eb, ep, ep + eb); }
     PPRVIZ_LAUNCHED(ctx);
@@ -1267,7 +1407,7 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
   // centre and emit each view; stress per view on its input pdist
   int64_t maxk = 0;
   for (int32_t v = 0; v < nviews; ++v) maxk = std::max<int64_t>(maxk, bv[v].k);
-  const unsigned eb_max = (unsigned)((maxk + LWARPS * RPW - 1) / (LWARPS * RPW));
+  const unsigned eb_max = energy_blocks(maxk);
   PPRVIZ_TRY(ws_ensure(ctx, WS_E, sizeof(V2) * (size_t)maxk + 64));
   PPRVIZ_TRY(ws_ensure(ctx, WS_OUT1, sizeof(double) * ((size_t)eb_max + 1) * nviews));
   V2 *Xc = ctx->ws[WS_E].as<V2>();
@@ -1276,12 +1416,12 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
   xo = 0;
   for (int32_t v = 0; v < nviews; ++v) {
     const int32_t k = bv[v].k;
-    const unsigned eb = (unsigned)((k + LWARPS * RPW - 1) / (LWARPS * RPW));
+    const unsigned eb = energy_blocks(k);
     double *epv = ep + (size_t)v * (eb_max + 1);
     { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_finish<float, float><<<1, 1024, 0, ctx->stream>>>(k, X + bv[v].vec_off, x_out_d + 2 * xo, Xc); }
     PPRVIZ_LAUNCHED(ctx);
     if (stress_h) {
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_energy<float, false, false><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, pdist_d + sq, Xc, 1.0f, epv, nullptr, nullptr, flag); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_energy<float, false, false><<<eb, ETHREADS, 0, ctx->stream>>>(k, pdist_d + sq, Xc, 1.0f, epv, nullptr, nullptr, flag); }
       PPRVIZ_LAUNCHED(ctx);
       { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_reduce_energy<<<1, 256, 0, ctx->stream>>>((int)eb, epv, epv + eb_max); }
       PPRVIZ_LAUNCHED(ctx);
@@ -1302,34 +1442,32 @@ template <typename T>
 static int energy_typed(pprviz_ctx *ctx, const T *pdist, int32_t k, const T *x, double scale, double *e_h,
                         T *gx, T *gD) {
   using V2 = typename T2<T>::type;
-  const unsigned eb = (unsigned)((k + LWARPS * RPW - 1) / (LWARPS * RPW));
+  const unsigned eb = energy_blocks(k);
   PPRVIZ_TRY(ws_ensure(ctx, WS_E, sizeof(V2) * (size_t)k + 64));
-  PPRVIZ_TRY(ws_ensure(ctx, WS_OUT1, sizeof(double) * (eb + 1)));
-  PPRVIZ_TRY(ws_ensure(ctx, WS_FLAG, 64));
+  // block partials, then the energy and the status word (read back together)
+  PPRVIZ_TRY(ws_ensure(ctx, WS_OUT1, sizeof(double) * (eb + 2)));
   V2 *X = ctx->ws[WS_E].as<V2>();
   double *ep = ctx->ws[WS_OUT1].as<double>();
-  int *flag = ctx->ws[WS_FLAG].as<int>();
+  int *flag = reinterpret_cast<int *>(ep + eb + 1);
   PPRVIZ_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
   { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_load_x<T, T><<<(unsigned)((k + 255) / 256), 256, 0, ctx->stream>>>(k, k, x, X); }
   PPRVIZ_LAUNCHED(ctx);
   const T s = (T)scale;
   {
     PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY);
-    if (gx && gD) k_energy<T, true, true><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
-    else if (gx) k_energy<T, true, false><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
-    else if (gD) k_energy<T, false, true><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
-    else k_energy<T, false, false><<<eb, LWARPS * 32, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
+    if (gx && gD) k_energy<T, true, true><<<eb, ETHREADS, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
+    else if (gx) k_energy<T, true, false><<<eb, ETHREADS, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
+    else if (gD) k_energy<T, false, true><<<eb, ETHREADS, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
+    else k_energy<T, false, false><<<eb, ETHREADS, 0, ctx->stream>>>(k, pdist, X, s, ep, gx, gD, flag);
   }
   PPRVIZ_LAUNCHED(ctx);
   { PPRVIZ_PROF(ctx, PPRVIZ_K_ENERGY); k_reduce_energy<<<1, 256, 0, ctx->stream>>>((int)eb, ep, ep + eb); }
   PPRVIZ_LAUNCHED(ctx);
-  double e = 0.0;
-  int hf = 0;
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&e, ep + eb, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  struct { double e; int flag, pad; } h = {0.0, 0, 0};
+  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&h, ep + eb, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
   PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  if (hf) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "pdist has a non-positive off-diagonal entry");
-  if (e_h) *e_h = e;
+  if (h.flag) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "pdist has a non-positive off-diagonal entry");
+  if (e_h) *e_h = h.e;
   return PPRVIZ_OK;
 }
 
@@ -1355,9 +1493,9 @@ int energy_run(pprviz_ctx *ctx, const void *pdist_d, int32_t k, const void *x_d,
 // until the process exits. The caller provides inputs and outputs.
 // ---------------------------------------------------------------------------
 constexpr int kNoAllocMaxK = 65536;
-constexpr int kNoAllocBlocks = (kNoAllocMaxK + LWARPS * RPW - 1) / (LWARPS * RPW);
+constexpr int kNoAllocBlocks = EBLOCKS;
 constexpr size_t kNoAllocXBytes = sizeof(float2) * kNoAllocMaxK;             // 512 KiB
-constexpr size_t kNoAllocEBytes = sizeof(double) * (kNoAllocBlocks + 1);     // 16 KiB + 8 B
+constexpr size_t kNoAllocEBytes = sizeof(double) * (kNoAllocBlocks + 1);     // ~5 KiB
 constexpr size_t kNoAllocBytes = kNoAllocXBytes + kNoAllocEBytes + 256;       // + status word
 
 static __device__ __align__(256) unsigned char g_energy_scratch[kNoAllocBytes];
@@ -1406,19 +1544,19 @@ extern "C" int pprviz_energy_noalloc(const float *pdist, int32_t k, const float 
   float2 *X = reinterpret_cast<float2 *>(base);
   double *eparts = reinterpret_cast<double *>(static_cast<unsigned char *>(base) + kNoAllocXBytes);
   int *flag = reinterpret_cast<int *>(static_cast<unsigned char *>(base) + kNoAllocXBytes + kNoAllocEBytes);
-  const unsigned eb = (unsigned)((k + LWARPS * RPW - 1) / (LWARPS * RPW));
+  const unsigned eb = energy_blocks(k);
   // the status word keeps the previous call's value: clear it first
   if (cudaMemsetAsync(flag, 0, sizeof(int), stream) != cudaSuccess) return PPRVIZ_E_CUDA;
   k_load_x<float, float><<<(unsigned)((k + 255) / 256), 256, 0, stream>>>(k, k, x, X);
   const float s = (float)grad_scale;
   if (grad_x && grad_pdist)
-    k_energy<float, true, true><<<eb, LWARPS * 32, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
+    k_energy<float, true, true><<<eb, ETHREADS, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
   else if (grad_x)
-    k_energy<float, true, false><<<eb, LWARPS * 32, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
+    k_energy<float, true, false><<<eb, ETHREADS, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
   else if (grad_pdist)
-    k_energy<float, false, true><<<eb, LWARPS * 32, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
+    k_energy<float, false, true><<<eb, ETHREADS, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
   else
-    k_energy<float, false, false><<<eb, LWARPS * 32, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
+    k_energy<float, false, false><<<eb, ETHREADS, 0, stream>>>(k, pdist, X, s, eparts, grad_x, grad_pdist, flag);
   k_reduce_energy<<<1, 256, 0, stream>>>((int)eb, eparts, eparts + eb);
   if (cudaGetLastError() != cudaSuccess) return PPRVIZ_E_CUDA;
   double e = 0.0;
