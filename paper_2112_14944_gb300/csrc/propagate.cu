@@ -89,12 +89,34 @@ __global__ void k_init_delta(int32_t gcount, const int32_t *__restrict__ src, in
   if (s >= 0) y[(int64_t)s * ld + q] = alpha * invdw[s];
 }
 
-// y = rhs / dw (the first iterate of the correction system, x_1 = rhs).
+// (row, first column) of the idx-th 4-vector of an [n][ld] state, ld % 4 == 0;
+// 32-bit division where the index allows it
+__device__ __forceinline__ void vec_row_col(int64_t idx, int64_t ld, int64_t &j, int64_t &q) {
+  const uint32_t ld4 = (uint32_t)(ld >> 2);
+  if (idx < (int64_t)1 << 32) {
+    const uint32_t r = (uint32_t)idx / ld4;
+    j = r;
+    q = (int64_t)((uint32_t)idx - r * ld4) * 4;
+  } else {
+    j = idx / ld4;
+    q = (idx - j * ld4) * 4;
+  }
+}
+
+// y = rhs / dw (the first iterate of the correction system, x_1 = rhs). One
+// thread per 4-vector here and in the other starts (bound by the writes).
 __global__ void k_init_rhs(int64_t n, int64_t ld, const float *__restrict__ rhs,
                            const float *__restrict__ invdw, float *__restrict__ y) {
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * ld) return;
-  y[idx] = rhs[idx] * invdw[idx / ld];
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * (ld >> 2)) return;
+  int64_t j, q;
+  vec_row_col(idx, ld, j, q);
+  float v[4];
+  Vec<float>::load(rhs + 4 * idx, v);
+  const float s = invdw[j];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) v[u] *= s;
+  Vec<float>::store(y + 4 * idx, v);
 }
 
 // Deflated start of a solve for the sources of a group: on the component of
@@ -108,13 +130,29 @@ __global__ void k_init_defl(int64_t n, int64_t ld, const int32_t *__restrict__ c
                             const float *__restrict__ invdw, float alpha, float c, float *__restrict__ y0,
                             float *__restrict__ y1) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * ld) return;
-  const int64_t j = idx / ld, q = idx - j * ld;
-  const int32_t cs = csrc[q];
-  const float v0 = (cs >= 0 && comp[j] == cs) ? (float)kappa[q] : 0.0f;
-  const float b = rhs ? rhs[idx] : ((src[q] == (int32_t)j) ? alpha : 0.0f);
-  y0[idx] = v0;
-  y1[idx] = c * v0 + b * invdw[j];
+  if (idx >= n * (ld >> 2)) return;
+  int64_t j, q;
+  vec_row_col(idx, ld, j, q);
+  const int4 cs = *reinterpret_cast<const int4 *>(csrc + q);
+  const int32_t csu[4] = {cs.x, cs.y, cs.z, cs.w};
+  const int32_t cj = comp[j];
+  const float s = invdw[j];
+  float v0[4], b[4], v1[4];
+  if (rhs) {
+    Vec<float>::load(rhs + 4 * idx, b);
+  } else {
+    const int4 sr = *reinterpret_cast<const int4 *>(src + q);
+    const int32_t sru[4] = {sr.x, sr.y, sr.z, sr.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) b[u] = (sru[u] == (int32_t)j) ? alpha : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    v0[u] = (csu[u] >= 0 && cj == csu[u]) ? (float)kappa[q + u] : 0.0f;
+    v1[u] = c * v0[u] + b[u] * s;
+  }
+  Vec<float>::store(y0 + 4 * idx, v0);
+  Vec<float>::store(y1 + 4 * idx, v1);
 }
 
 __global__ void k_axpy(int64_t count, const float *__restrict__ x, float *__restrict__ y) {
@@ -372,6 +410,124 @@ k_sweep_sp(int64_t nitems, int64_t ld, int nchunks, const int4 *__restrict__ ite
   Vec<float>::store(yout + rowoff, out);
 }
 
+// The same sweep for a narrow group of LD = 4 LPR columns (32 or 64): LPR lanes
+// share a work item, so a warp takes 32 / LPR items at once and a gathered
+// neighbour row is one 128- or 256-byte read. For a state that does not fit in
+// L2 the narrow rows keep four or two times as many of the often-gathered hub
+// rows resident (against re-reading the graph once per group), and for a call
+// with few columns (the children of a supernode) no padding is moved. The
+// items' edge lists run in lockstep, 8 gathers in flight per lane; a missing
+// edge adds zero. Twelve blocks per SM (40 registers) on unweighted 32-wide
+// groups: the time follows the
+// gathers in flight, so loading the row's y_old ahead of them costs more
+// registers than it hides (818 us); cache hints on the gathers, the streams or
+// the stores change nothing. 2M nodes, 20M edges, one sweep: 436 us for 32
+// columns against 2,040 us for 128 in one group (k_sweep_sp), so 1.74 ms per
+// 128 columns; 2.15 GB from DRAM, 4.9 TB/s.
+template <int LPR, bool WEIGHTED, bool RHS>
+__global__ void __launch_bounds__(128, LPR == 8 && !WEIGHTED ? 12 : 9)
+k_sweep_nw(int64_t nitems, const int4 *__restrict__ items, const int2 *__restrict__ srow,
+           const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ w,
+           const float *__restrict__ invdw, const int32_t *__restrict__ src, const float *__restrict__ rhs,
+           const float *__restrict__ ycur, const float *yold, float *yout, float alpha, float c, float om, float om1,
+           float *__restrict__ part, int *__restrict__ cnt) {
+  constexpr int LD = 4 * LPR, IPW = 32 / LPR;
+  const int lane = threadIdx.x & 31, sl = lane % LPR;
+  const int64_t wid = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (wid * IPW >= nitems) return;  // the whole warp
+  const int64_t t = wid * IPW + lane / LPR;
+  const bool live = t < nitems;
+  const int4 it = live ? items[t] : make_int4(0, 0, 0, -1);
+  const int64_t j = it.x;
+  const int off = sl * 4, len = live ? it.z : 0;
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const int64_t b = rp[j] + it.y;
+  const int maxlen = __reduce_max_sync(0xffffffffu, len);
+  int32_t nxc = sl < len ? col[b + sl] : -1;
+  for (int base = 0; base < maxlen; base += LPR) {
+    const int32_t myc = nxc;
+    nxc = base + LPR + sl < len ? col[b + base + LPR + sl] : -1;  // the next round's indices, in flight meanwhile
+    float myw = 1.0f;
+    if (WEIGHTED) myw = base + sl < len ? w[b + base + sl] : 0.0f;
+#pragma unroll
+    for (int t0 = 0; t0 < LPR; t0 += 8) {
+      if (base + t0 >= maxlen) break;
+      float v[8][4], wv[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int32_t i = __shfl_sync(0xffffffffu, myc, t0 + q, LPR);
+        if (WEIGHTED) wv[q] = __shfl_sync(0xffffffffu, myw, t0 + q, LPR);
+        if (i >= 0) {
+          Vec<float>::load(ycur + (int64_t)i * LD + off, v[q]);
+        } else {
+          v[q][0] = v[q][1] = v[q][2] = v[q][3] = 0.0f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (WEIGHTED) {
+          float s2 = 0.0f;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) s2 += wv[q] * v[q][u];
+          acc[u] += s2;
+        } else {
+          acc[u] += ((v[0][u] + v[1][u]) + (v[2][u] + v[3][u])) + ((v[4][u] + v[5][u]) + (v[6][u] + v[7][u]));
+        }
+      }
+    }
+  }
+  bool update = live;
+  const bool split = live && it.w >= 0;
+  if (__any_sync(0xffffffffu, split)) {
+    int last = 0;
+    int2 s = make_int2(0, 0);
+    if (split) {
+      s = srow[it.w];
+      Vec<float>::store(part + (int64_t)(s.x + it.y / kSegEdges) * LD + off, acc);
+      __threadfence();
+    }
+    __syncwarp();
+    if (split && sl == 0) last = atomicAdd(&cnt[it.w], 1) == s.y - 1;
+    last = __shfl_sync(0xffffffffu, last, 0, LPR);
+    if (split) {
+      update = last != 0;
+      if (last) {
+        __threadfence();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = 0.0f;
+        for (int k2 = 0; k2 < s.y; ++k2) {
+          const float4 p4 = __ldcg(reinterpret_cast<const float4 *>(part + (int64_t)(s.x + k2) * LD + off));
+          acc[0] += p4.x; acc[1] += p4.y; acc[2] += p4.z; acc[3] += p4.w;
+        }
+        if (sl == 0) cnt[it.w] = 0;
+      }
+    }
+  }
+  if (!update) return;
+  const int64_t rowoff = j * LD + off;
+  if (len == 0) {  // no edges: the walk stays on j (self-loop of weight 1)
+    float v0[4];
+    Vec<float>::load(ycur + rowoff, v0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] += v0[u];
+  }
+  const float invd = invdw[j];
+  float bq[4];
+  if (RHS) {
+    const float4 r4 = __ldcs(reinterpret_cast<const float4 *>(rhs + rowoff));
+    bq[0] = r4.x; bq[1] = r4.y; bq[2] = r4.z; bq[3] = r4.w;
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) bq[u] = (src[off + u] == (int32_t)j) ? alpha : 0.0f;
+  }
+  const float4 o4 = __ldcs(reinterpret_cast<const float4 *>(yold + rowoff));
+  const float old[4] = {o4.x, o4.y, o4.z, o4.w};
+  float out[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) out[u] = om1 * old[u] + om * ((bq[u] + c * acc[u]) * invd);
+  Vec<float>::store(yout + rowoff, out);
+}
+
 // v[u] = (double)(y_hi[u] + y_lo[u]), u < 4, with 16-byte loads (p is 4-aligned).
 __device__ __forceinline__ void load4(const float *hi, const float *lo, double (&v)[4]) {
   float a[4];
@@ -411,20 +567,25 @@ __device__ __forceinline__ void load4(const double *hi, const float *lo, double 
 // (Sec. 3.2, Eq. (2)): b_jq = alpha d(j) / |F(V_q)| for the leaves j of V_q,
 // given per node by src[j] = its supernode (-1 for none) and bscale[j] =
 // d(j) / |F(V_src[j])| in FP64, so the residual is exact for that b.
-template <typename T, bool WEIGHTED, bool EXACT, bool BATCH, bool LEVEL, bool LO = true>
+// A group of 4 LPR < 128 columns (k_sweep_nw) has LPR lanes per row and 32 / LPR
+// rows per warp; the rows of a warp take their edges side by side.
+template <typename T, bool WEIGHTED, bool EXACT, bool BATCH, bool LEVEL, bool LO = true, int LPR = 32>
 __global__ void __launch_bounds__(kWarps * 32)
 k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
            const float *__restrict__ w, const double *__restrict__ invdw, const float2 *__restrict__ dwff,
            const int32_t *__restrict__ src, const T *__restrict__ yhi, const float *__restrict__ ylo,
            float *__restrict__ rhs_out, double *__restrict__ part_out, double alpha, double c,
            const int2 *__restrict__ brows, int64_t row0, int32_t g0, const double *__restrict__ bscale) {
-  constexpr int VEC = 4;  // 128 sources per warp chunk for both state types
-  __shared__ double red[kWarps][32 * VEC];
-  __shared__ double reds[kWarps][32 * VEC];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
+  constexpr int VEC = 4;  // 4 LPR sources per row chunk for both state types
+  constexpr int CW = LPR * VEC, NSUB = kWarps * 32 / LPR;
+  static_assert(LPR == 32 || !BATCH, "batched views use whole warps");
+  __shared__ double red[NSUB][CW];
+  __shared__ double reds[NSUB][CW];
+  const int lane = threadIdx.x % LPR;
+  const int warp = threadIdx.x / LPR;  // the row's lane group
+  const unsigned rmask = LPR == 32 ? 0xffffffffu : ((1u << LPR) - 1u) << ((threadIdx.x & 31) / LPR * LPR);
   const int64_t chunk = blockIdx.y;
-  const int64_t off = chunk * (32 * VEC) + lane * VEC;
+  const int64_t off = chunk * CW + lane * VEC;
   int32_t sq[VEC];
 #pragma unroll
   for (int u = 0; u < VEC; ++u) sq[u] = (BATCH || LEVEL) ? 0 : src[off + u];
@@ -446,9 +607,9 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
     jend = br.y;
     stride = kWarps;
   } else {
-    jfirst = (int64_t)blockIdx.x * kWarps + warp;
+    jfirst = (int64_t)blockIdx.x * NSUB + warp;
     jend = n;
-    stride = (int64_t)gridDim.x * kWarps;
+    stride = (int64_t)gridDim.x * NSUB;
   }
   for (int64_t j = jfirst; j < jend; j += stride) {
     const int64_t jg = j + row0;  // row of the graph
@@ -467,14 +628,14 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
       // (Knuth) keeps the exact rounding error of every addition of the high
       // parts, FMA the exact error of every weighted product; the
       // compensation is flushed into a float-float accumulator (ah, al) after
-      // every 32 edges. The residual is then formed in float-float arithmetic
+      // every LPR edges. The residual is then formed in float-float arithmetic
       // (TwoProd by FMA, TwoSum), ~2^-48 relative to the row: GB300's FP64
       // rate is too low to spend FP64 operations per (node, source).
       float shi[VEC], sc[VEC], slo[VEC], ah[VEC], al[VEC];
 #pragma unroll
       for (int u = 0; u < VEC; ++u) shi[u] = sc[u] = slo[u] = ah[u] = al[u] = 0.0f;
-      for (int64_t base = b; base < e; base += 32) {
-        const int cnt = (int)min((int64_t)32, e - base);
+      for (int64_t base = b; base < e; base += LPR) {
+        const int cnt = (int)min((int64_t)LPR, e - base);
         int32_t myc = lane < cnt ? col[base + lane] : 0;
         float myw = 1.0f;
         if (WEIGHTED) myw = lane < cnt ? w[base + lane] : 0.0f;
@@ -484,8 +645,8 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
           float h[GB][VEC], l[GB][VEC], wv[GB];
 #pragma unroll
           for (int q = 0; q < GB; ++q) {
-            const int32_t i = __shfl_sync(0xffffffffu, myc, (t0 + q) & 31);
-            wv[q] = WEIGHTED ? __shfl_sync(0xffffffffu, myw, (t0 + q) & 31) : 1.0f;
+            const int32_t i = __shfl_sync(rmask, myc, (t0 + q) & (LPR - 1), LPR);
+            wv[q] = WEIGHTED ? __shfl_sync(rmask, myw, (t0 + q) & (LPR - 1), LPR) : 1.0f;
             if (t0 + q < cnt) {
               const int64_t p = ((int64_t)i - rb) * ld + off;
               Vec<float>::load(reinterpret_cast<const float *>(yhi) + p, h[q]);
@@ -563,8 +724,8 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
       }
       continue;
     } else {
-      for (int64_t base = b; base < e; base += 32) {
-        const int cnt = (int)min((int64_t)32, e - base);
+      for (int64_t base = b; base < e; base += LPR) {
+        const int cnt = (int)min((int64_t)LPR, e - base);
         int32_t myc = lane < cnt ? col[base + lane] : 0;
         float myw = 1.0f;
         if (WEIGHTED) myw = lane < cnt ? w[base + lane] : 0.0f;
@@ -573,8 +734,8 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
           double v[4][VEC], wv[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const int32_t i = __shfl_sync(0xffffffffu, myc, (t0 + q) & 31);
-            wv[q] = WEIGHTED ? (double)__shfl_sync(0xffffffffu, myw, (t0 + q) & 31) : 1.0;
+            const int32_t i = __shfl_sync(rmask, myc, (t0 + q) & (LPR - 1), LPR);
+            wv[q] = WEIGHTED ? (double)__shfl_sync(rmask, myw, (t0 + q) & (LPR - 1), LPR) : 1.0;
             if (t0 + q < cnt) {
               const int64_t p = ((int64_t)i - rb) * ld + off;
               load4(yhi + p, ylo ? ylo + p : nullptr, v[q]);
@@ -610,15 +771,15 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
     reds[warp][lane * VEC + u] = psig[u] + (double)fpsig[u];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < 32 * VEC; t += blockDim.x) {
+  for (int t = threadIdx.x; t < CW; t += blockDim.x) {
     double s = 0.0, ss = 0.0;
 #pragma unroll
-    for (int wv = 0; wv < kWarps; ++wv) {
+    for (int wv = 0; wv < NSUB; ++wv) {
       s += red[wv][t];
       ss += reds[wv][t];
     }
-    part_out[((int64_t)blockIdx.x * 2 + 0) * ld + chunk * (32 * VEC) + t] = s;
-    part_out[((int64_t)blockIdx.x * 2 + 1) * ld + chunk * (32 * VEC) + t] = ss;
+    part_out[((int64_t)blockIdx.x * 2 + 0) * ld + chunk * CW + t] = s;
+    part_out[((int64_t)blockIdx.x * 2 + 1) * ld + chunk * CW + t] = ss;
   }
 }
 
@@ -782,6 +943,16 @@ int64_t choose_group(int64_t n, int32_t k, size_t elem) {
   return g;
 }
 
+// ~3 live [n][ld] FP32 buffers within ~64 MB of L2
+bool state_fits(int64_t n, int64_t ld) { return 12.0 * (double)n * (double)ld <= 64.0 * 1024 * 1024; }
+
+// FP32 CSR path: 32- or 64-wide groups (k_sweep_nw) where the sources fit in one
+int64_t choose_group_f32(int64_t n, int32_t k) {
+  if (k <= 32) return 32;
+  if (k <= 64) return 64;
+  return choose_group(n, k, sizeof(float));
+}
+
 // A wave of batched views (see k_sweep): the state covers the union-graph
 // rows [row0, row0 + nrows), column q is source g0 + q of every row's view;
 // lidx[i] is node i's index within its view. The residual's blocks each cover
@@ -875,10 +1046,10 @@ int launch_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, bool cheb, 
       const int64_t nslots = wv ? wv->nslots : g->sp_nslots;
       const int4 *items = wv ? wv->items : g->sp_items.as<int4>();
       const int2 *srowp = wv ? wv->srow : g->sp_srow.as<int2>();
-      if (nsplit > 0) {
-        const int nchunks = (int)(ld / 128);
+      if (nsplit > 0 || ld < kChunk) {
+        const int nchunks = (int)std::max<int64_t>(1, ld / kChunk);
         PPRVIZ_TRY(ws_ensure(ctx, WS_SPART, sizeof(float) * (size_t)std::max<int64_t>(1, nslots) * (size_t)ld));
-        const size_t cbytes = sizeof(int) * (size_t)nsplit * (size_t)nchunks;
+        const size_t cbytes = sizeof(int) * (size_t)std::max<int64_t>(1, nsplit) * (size_t)nchunks;
         const bool fresh = ctx->ws[WS_SCNT].cap < cbytes || !ctx->ws[WS_SCNT].p;
         PPRVIZ_TRY(ws_ensure(ctx, WS_SCNT, cbytes));
         // the counters return to zero after every sweep; clear them once per call
@@ -893,6 +1064,25 @@ int launch_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, bool cheb, 
         const int64_t row0 = wv ? wv->row0 : 0;
         const int32_t g0 = wv ? wv->g0 : 0;
         PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
+        if (ld < kChunk) {
+          const int ipb = ld == 32 ? 16 : 8;  // work items per block of four warps
+          const unsigned nb = (unsigned)((nitems + ipb - 1) / ipb);
+#define PPRVIZ_SWEEP_NW(L, W, R)                                                                               \
+  k_sweep_nw<L, W, R><<<nb, 128, 0, ctx->stream>>>(                                                             \
+      nitems, items, srowp, pull_rp(g), pull_col(g), w, g->invdw_f.as<float>(), srcp, rhsbuf,                   \
+      (const float *)ycur, (const float *)yold, (float *)yout, a, c, o, o1, ctx->ws[WS_SPART].as<float>(),      \
+      ctx->ws[WS_SCNT].as<int>())
+          if (ld == 32) {
+            if (pull_weighted(g)) { if (rhs) PPRVIZ_SWEEP_NW(8, true, true); else PPRVIZ_SWEEP_NW(8, true, false); }
+            else { if (rhs) PPRVIZ_SWEEP_NW(8, false, true); else PPRVIZ_SWEEP_NW(8, false, false); }
+          } else {
+            if (pull_weighted(g)) { if (rhs) PPRVIZ_SWEEP_NW(16, true, true); else PPRVIZ_SWEEP_NW(16, true, false); }
+            else { if (rhs) PPRVIZ_SWEEP_NW(16, false, true); else PPRVIZ_SWEEP_NW(16, false, false); }
+          }
+#undef PPRVIZ_SWEEP_NW
+          PPRVIZ_LAUNCHED(ctx);
+          return PPRVIZ_OK;
+        }
 #define PPRVIZ_SWEEP_SP(W, R, B)                                                                               \
   k_sweep_sp<W, R, B><<<(unsigned)blocks, 32, 0, ctx->stream>>>(                                                \
       nitems, ld, nchunks, items, srowp, pull_rp(g), pull_col(g), w, g->invdw_f.as<float>(),                    \
@@ -957,10 +1147,14 @@ int launch_residual(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
                     const T *yhi, const float *ylo, float *rhs_out, double *l1, double alpha,
                     const Wave *wv = nullptr, int total_blocks = 1216, const double *bscale = nullptr,
                     int32_t level_g0 = 0) {
-  const int nchunks = (int)(ld / 128);
+  const bool narrow = ld < kChunk;  // 32 or 64 columns: FP32 state, no batch
+  const int nchunks = (int)std::max<int64_t>(1, ld / kChunk);
   int rows_blocks;
   if (wv) {
     rows_blocks = wv->nblocks;
+  } else if (narrow) {
+    const int64_t rows = ld == 32 ? 4 * kWarps : 2 * kWarps;  // rows of a block at a time
+    rows_blocks = (int)std::min<int64_t>((g->n + rows - 1) / rows, 1216);
   } else {
     // `total_blocks` CTAs in all when the group's state fits in L2 (1,216
     // unless tuned); otherwise ~608 per chunk (about the resident CTAs of the
@@ -979,19 +1173,29 @@ int launch_residual(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
   const int64_t row0 = wv ? wv->row0 : 0;
   const int32_t g0 = wv ? wv->g0 : level_g0;
   if (wv) src = wv->lidx;
-#define PPRVIZ_RES(W, B, L, LOW)                                                                             \
-  k_residual<T, W, EXACT, B, L, LOW><<<grid, kWarps * 32, 0, ctx->stream>>>(                                   \
+#define PPRVIZ_RES(W, B, L, LOW) PPRVIZ_RES_L(W, B, L, LOW, 32)
+#define PPRVIZ_RES_L(W, B, L, LOW, LPR)                                                                        \
+  k_residual<T, W, EXACT, B, L, LOW, LPR><<<grid, kWarps * 32, 0, ctx->stream>>>(                                   \
       n, ld, pull_rp(g), pull_col(g), w, g->invdw_d.as<double>(), g->dwff.as<float2>(), src,                   \
       yhi, ylo, rhs_out, part, alpha, 1.0 - alpha, brows, row0, g0, bscale)
   {
     PPRVIZ_PROF(ctx, PPRVIZ_K_RESIDUAL);
-    if (wv) { if (pull_weighted(g)) PPRVIZ_RES(true, true, false, true); else PPRVIZ_RES(false, true, false, true); }
+    if (narrow) {
+      if constexpr (std::is_same<T, float>::value) {
+#define PPRVIZ_RES_N(LPR)                                                                                              \
+  if (bscale) { if (pull_weighted(g)) PPRVIZ_RES_L(true, false, true, true, LPR); else PPRVIZ_RES_L(false, false, true, true, LPR); } \
+  else { if (pull_weighted(g)) PPRVIZ_RES_L(true, false, false, true, LPR); else PPRVIZ_RES_L(false, false, false, true, LPR); }
+        if (ld == 32) { PPRVIZ_RES_N(8) } else { PPRVIZ_RES_N(16) }
+#undef PPRVIZ_RES_N
+      }
+    } else if (wv) { if (pull_weighted(g)) PPRVIZ_RES(true, true, false, true); else PPRVIZ_RES(false, true, false, true); }
     else if (bscale) { if (pull_weighted(g)) PPRVIZ_RES(true, false, true, true); else PPRVIZ_RES(false, false, true, true); }
     else if (pull_weighted(g)) PPRVIZ_RES(true, false, false, true);
     else if (ylo) PPRVIZ_RES(false, false, false, true);
     else PPRVIZ_RES(false, false, false, false);  // no low parts: a lighter instance (fewer registers)
   }
 #undef PPRVIZ_RES
+#undef PPRVIZ_RES_L
   PPRVIZ_LAUNCHED(ctx);
   if (wv) {
     const int64_t warps = (int64_t)wv->nviews * ld;
@@ -1008,9 +1212,10 @@ int launch_residual(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
 // lengths of n, nnz and k, weighted or not), kept in the context so that its
 // cost (a few milliseconds) is paid on the first call of each class:
 //  * the source-group width G: candidates 128, 256, ... up to the width whose
-//    ~3 live [n][G] buffers fill ~64 MB of L2 (choose_group); each runs three
-//    timed Chebyshev sweeps on the graph (after one untimed), and the width
-//    with the least time per source and sweep wins;
+//    ~3 live [n][G] buffers fill ~64 MB of L2 (choose_group), and 32 and 64
+//    where not even 128 columns fit; each runs three timed Chebyshev sweeps on
+//    the graph (after one untimed), and the width with the least time for all
+//    k sources wins;
 //  * then, at that width, the residual's CTA count (608 .. 4,864 in all): three
 //    timed residual passes with a low part each, the fastest wins.
 // The values of the state do not change the work of either kernel, so both
@@ -1025,10 +1230,12 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
   auto bits = [](uint64_t x) { int b = 0; while (x) { ++b; x >>= 1; } return (uint64_t)b; };
   const uint64_t key = (bits((uint64_t)g->n) << 40) | (bits((uint64_t)g->nnz) << 32) | (bits((uint64_t)k) << 8) |
                        (g->weighted ? 1u : 0u) | (g->directed ? 2u : 0u);
+  const int64_t gmax = choose_group_f32(g->n, k);
+  if (gmax < kChunk) return TunedShape{gmax, 1216};  // one narrow group
   for (const auto &e : ctx->tuned_groups)
     if (e.first == key) return TunedShape{e.second >> 16, (int)(e.second & 0xFFFF)};
-  const int64_t gmax = choose_group(g->n, k, sizeof(float));
   std::vector<int64_t> cands;
+  if (gmax == kChunk && !state_fits(g->n, kChunk)) cands = {32, 64};
   for (int64_t c = kChunk; c < gmax; c *= 2) cands.push_back(c);
   cands.push_back(gmax);
   int64_t best = gmax;
@@ -1067,7 +1274,7 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
         st = cuda_err(ctx, ce, "autotuner timing");
         break;
       }
-      const double score = (double)ms / (double)G;
+      const double score = (double)ms * (double)((k + G - 1) / G);
       if (best_score == 0.0 || score < best_score) {
         best_score = score;
         best = G;
@@ -1164,14 +1371,14 @@ int chebyshev_solve(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
         (float)alpha, (float)c, ya, yb); }
     PPRVIZ_LAUNCHED(ctx);
   } else if (csrc) {
-    const int64_t cnt = g->n * ld;
+    const int64_t cnt = g->n * (ld / 4);
     { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_init_defl<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(
         g->n, ld, g->comp.as<int32_t>(), csrc, kappa, src, rhs, g->invdw_f.as<float>(), (float)alpha, (float)c, ya, yb); }
     PPRVIZ_LAUNCHED(ctx);
   } else {
   PPRVIZ_CUDA(ctx, cudaMemsetAsync(ya, 0, bytes, ctx->stream));
   if (rhs) {
-    const int64_t cnt = g->n * ld;
+    const int64_t cnt = g->n * (ld / 4);
     { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_init_rhs<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(g->n, ld, rhs, g->invdw_f.as<float>(), yb); }
     PPRVIZ_LAUNCHED(ctx);
   } else {
@@ -1453,13 +1660,33 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
 // --------------------------------------------------------------------------
 namespace {
 
+// owner[t] = the supernode whose leaf t is, bscale[t] = d(t) / |F(V_owner)|; one
+// block per supernode (the leaf sets are disjoint)
+__global__ void k_level_owner(const int64_t *__restrict__ leaf_ptr, const int32_t *__restrict__ leaf_idx,
+                              const double *__restrict__ deg, int32_t *__restrict__ owner,
+                              double *__restrict__ bscale) {
+  const int64_t a = leaf_ptr[blockIdx.x], e = leaf_ptr[blockIdx.x + 1];
+  const double sz = (double)(e - a);
+  for (int64_t p = a + threadIdx.x; p < e; p += blockDim.x) {
+    const int32_t t = leaf_idx[p];
+    owner[t] = (int32_t)blockIdx.x;
+    bscale[t] = deg[t] / sz;
+  }
+}
+
 // rhs[j][q] = alpha * bscale[j] if node j is a leaf of supernode g0 + q, else 0
 __global__ void k_level_rhs(int64_t n, int64_t ld, int32_t g0, const int32_t *__restrict__ owner,
                             const double *__restrict__ bscale, double alpha, float *__restrict__ rhs) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * ld) return;
-  const int64_t j = idx / ld, q = idx - j * ld;
-  rhs[idx] = (owner[j] == g0 + (int32_t)q) ? (float)(alpha * bscale[j]) : 0.0f;
+  if (idx >= n * (ld >> 2)) return;
+  int64_t j, q;
+  vec_row_col(idx, ld, j, q);
+  const int32_t own = owner[j] - g0 - (int32_t)q;
+  float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (own == u) v[u] = (float)(alpha * bscale[j]);
+  Vec<float>::store(rhs + 4 * idx, v);
 }
 
 // out[(g0 + q) * nsup + r] = sum_{t in F(V_r)} x_q(t) / |F(V_r)|, x = dw (y_hi + y_lo),
@@ -1489,18 +1716,8 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
                      const std::vector<int32_t> &leaf_idx_h, double alpha, double eps, void *out_d, bool out64,
                      double *cert_h) {
   const int64_t n = g->n;
-  // owner of each node and the FP64 right-hand-side scale d(j) / |F(V_owner)|
-  std::vector<int32_t> owner((size_t)n, -1);
-  std::vector<double> bscale((size_t)n, 0.0);
-  for (int32_t v = 0; v < nsup; ++v) {
-    const double sz = (double)(leaf_ptr_h[v + 1] - leaf_ptr_h[v]);
-    for (int64_t p = leaf_ptr_h[v]; p < leaf_ptr_h[v + 1]; ++p) {
-      const int32_t t = leaf_idx_h[p];
-      owner[t] = v;
-      bscale[t] = g->h_deg[t] / sz;
-    }
-  }
-  const int64_t ld = choose_group(n, nsup, sizeof(float));
+  int64_t ld = choose_group_f32(n, nsup);
+  if (ld == kChunk && !state_fits(n, ld)) ld = 32;  // a state beyond L2: narrow groups (see k_sweep_nw)
   const size_t sbytes = sizeof(float) * (size_t)(n * ld);
   PPRVIZ_TRY(ws_ensure(ctx, WS_Y0, sbytes));
   PPRVIZ_TRY(ws_ensure(ctx, WS_Y1, sbytes));
@@ -1513,10 +1730,14 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
   int32_t *owner_d = ctx->ws[WS_SRC].as<int32_t>();
   double *bscale_d = ctx->ws[WS_KAPPA].as<double>();
   double *l1 = ctx->ws[WS_CERT].as<double>();
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(owner_d, owner.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice,
-                                   ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(bscale_d, bscale.data(), sizeof(double) * (size_t)n, cudaMemcpyHostToDevice,
-                                   ctx->stream));
+  // owner of each node and the FP64 right-hand-side scale d(j) / |F(V_owner)|
+  PPRVIZ_CUDA(ctx, cudaMemsetAsync(owner_d, 0xFF, sizeof(int32_t) * (size_t)n, ctx->stream));
+  PPRVIZ_CUDA(ctx, cudaMemsetAsync(bscale_d, 0, sizeof(double) * (size_t)n, ctx->stream));
+  {
+    PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER);
+    k_level_owner<<<(unsigned)nsup, 128, 0, ctx->stream>>>(leaf_ptr_d, leaf_idx_d, g->deg.as<double>(), owner_d, bscale_d);
+  }
+  PPRVIZ_LAUNCHED(ctx);
   pprviz_stats &st = ctx->stats;
   st.source_group = (int32_t)ld;
   const double c = 1.0 - alpha;
@@ -1534,7 +1755,7 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
     float *rhs = ctx->ws[WS_RHS].as<float>();
     {
       PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER);
-      k_level_rhs<<<(unsigned)((n * ld + 255) / 256), 256, 0, ctx->stream>>>(n, ld, g0, owner_d, bscale_d, alpha, rhs);
+      k_level_rhs<<<(unsigned)((n * (ld / 4) + 255) / 256), 256, 0, ctx->stream>>>(n, ld, g0, owner_d, bscale_d, alpha, rhs);
     }
     PPRVIZ_LAUNCHED(ctx);
     // undeflated Chebyshev on the whole interval [1 - c, 1 + c] (a leaf set

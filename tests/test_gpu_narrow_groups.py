@@ -1,0 +1,73 @@
+"""Source groups of 32 and 64 columns (few sources, or a state beyond L2)
+against the 128-wide groups of an all-nodes call: every DPPR entry of the two
+lies within the sum of its certificates, on hub rows split into segments,
+isolated nodes, weights and directed graphs."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+ALPHA = 0.15
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2112_14944_gb300 as P
+    c = P.Context(0)
+    yield c
+    c.close()
+
+
+def graph(kind):
+    if kind == "hubs":
+        return synth.chung_lu(901, 12, 2.2, seed=3)  # rows of more than 64 edges, some isolated nodes
+    if kind == "weighted":
+        return synth.dense_clustered(300, blocks=4, density=0.04, seed=2)
+    return synth.directed_from(synth.chung_lu(901, 12, 2.2, seed=3), seed=5)
+
+
+_wide = {}
+
+
+def wide(ctx, kind, eps):
+    """(uploaded graph, DPPR of all nodes, certificates) with 128-wide groups."""
+    import paper_2112_14944_gb300 as P
+    if (kind, eps) not in _wide:
+        G = ctx.upload_graph(graph(kind))
+        view = np.arange(G.n, dtype=np.int32)
+        D, _, cert, st = ctx.dppr(G, view, ALPHA, eps, P.FP32_CSR, out64=True)
+        assert st == 0 and ctx.stats()["source_group"] >= 128
+        _wide[kind, eps] = G, D, cert
+    return _wide[kind, eps]
+
+
+@pytest.mark.parametrize("eps", [1e-6, 1e-10])
+@pytest.mark.parametrize("k", [1, 31, 32, 33, 64, 65])
+@pytest.mark.parametrize("kind", ["hubs", "weighted", "directed"])
+def test_narrow_groups_match_wide(ctx, kind, k, eps):
+    import paper_2112_14944_gb300 as P
+    G, D, cert = wide(ctx, kind, eps)
+    view = synth.sample_view(G.n, k, seed=k)
+    Dn, _, cn, st = ctx.dppr(G, view, ALPHA, eps, P.FP32_CSR, out64=True)
+    assert st == 0 and cn.max() <= eps
+    assert ctx.stats()["source_group"] == (32 if k <= 32 else 64 if k <= 64 else 128)
+    ref = D[np.ix_(view, view)]
+    # the outputs are float-float products rounded below 2^-40 of an entry
+    assert (np.abs(Dn - ref) <= (cn + cert[view])[:, None] + 2.0 ** -40 * np.abs(ref)).all()
+
+
+@pytest.mark.parametrize("children", [1, 32, 40, 64, 70])
+@pytest.mark.parametrize("kind", ["hubs", "directed"])
+def test_narrow_level_groups(ctx, kind, children):
+    """Level-l DPPR of leaf sets of uneven size: averages of the node rows (Eq. (2))."""
+    G, D, cert = wide(ctx, kind, 1e-10)
+    sizes = 1 + np.arange(children) % 5
+    ptr, idx = synth.random_leaf_sets(G.n, sizes, seed=children)
+    sets = [idx[ptr[i]:ptr[i + 1]] for i in range(children)]
+    L, _, cl, st = ctx.level_dppr(G, sets, ALPHA, 1e-6, out64=True)
+    assert st == 0
+    ref = np.array([[D[np.ix_(a, b)].sum() / (len(a) * len(b)) for b in sets] for a in sets])
+    miss = np.array([cert[a].mean() for a in sets])
+    assert (np.abs(L - ref) <= (cl + miss)[:, None] + 1e-12 * np.abs(ref)).all()
