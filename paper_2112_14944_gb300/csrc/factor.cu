@@ -25,42 +25,117 @@ namespace pprviz {
 // split high and low parts) and pivot inverse P (NB x NB), and a status word
 size_t spd_inverse_work(int32_t kp) { return (size_t)2 * (2 * 256 * (size_t)kp + 128 * 128) + 64; }
 
-// P = A_KK^-1 by an in-place scalar sweep of the NB x NB block in shared memory
-// (ping-pong buffers, one barrier per pivot); writes P to `P` and -P into A_KK.
-template <typename T, int NB>
-__global__ void __launch_bounds__(512) k_fac_diag(int32_t kp, int32_t K0, T *__restrict__ A, T *__restrict__ P) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  T *buf = reinterpret_cast<T *>(smem_raw);  // [2][NB][NB + 1]
-  constexpr int LD = NB + 1, SZ = NB * LD;
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, c = e % NB;
-    buf[r * LD + c] = A[(int64_t)(K0 + r) * kp + K0 + c];
-  }
-  __syncthreads();
-  int cur = 0;
-  for (int p = 0; p < NB; ++p) {
-    const T *a = buf + cur * SZ;
-    T *b = buf + (cur ^ 1) * SZ;
-    const T piv = T(1) / a[p * LD + p];
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-      const int r = e / NB, c = e % NB;
-      const T arc = a[r * LD + c], arp = a[r * LD + p], apc = a[p * LD + c];
-      T v;
-      if (r == p && c == p) v = piv;
-      else if (r == p) v = apc * piv;
-      else if (c == p) v = -arp * piv;
-      else v = arc - arp * (apc * piv);
-      b[r * LD + c] = v;
+// FP64: P = A_KK^-1 of a 64 x 64 block by the scalar sweep
+//   a_pp -> 1/a_pp, a_pc -> a_pc/a_pp, a_rp -> -a_rp/a_pp, a_rc -> a_rc - a_rp a_pc/a_pp,
+// pivot by pivot; writes P to `P` and -P into A_KK. The sweep keeps a symmetric
+// block symmetric up to sign (a_cr = a_rc, or -a_rc between a swept and an
+// unswept index), so only the 4 x 4 tiles on and below the diagonal are held:
+// 136 threads, one tile each in registers. Per pivot the tiles of column p
+// publish it (two alternating buffers, one barrier per pivot) and every thread
+// reads the four values of its rows and of its columns. Bound by the FP64
+// pipe of the one SM it runs on (2 operations per cycle: half of 64^3 fused
+// multiply-adds are 32 us), so nothing is computed twice and the reciprocal is
+// an estimate with two Newton steps instead of a division per thread:
+// 284 -> 114 us per block.
+constexpr int DIAG64_THREADS = 160;
+__device__ __forceinline__ double rcp_pos(double a) {  // 1/a, a > 0 normal (pivots of an SPD matrix)
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  r = fma(fma(-a, r, 1.0), r, r);
+  return fma(fma(-a, r, 1.0), r, r);
+}
+__global__ void __launch_bounds__(DIAG64_THREADS) k_fac_diag64(int32_t kp, int32_t K0, double *__restrict__ A,
+                                                               double *__restrict__ P) {
+  __shared__ __align__(16) double col[2][64];
+  // thread t < 136 holds tile (R, C), R >= C: t = R (R + 1) / 2 + C
+  int R = 0, C = (int)threadIdx.x;
+  const bool live = threadIdx.x < 136;
+  if (live) {
+    while (C > R) {
+      C -= R + 1;
+      ++R;
     }
-    __syncthreads();
-    cur ^= 1;
+  } else {
+    C = 0;
   }
-  const T *a = buf + cur * SZ;
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, c = e % NB;
-    const T v = a[r * LD + c];
-    P[e] = v;
-    A[(int64_t)(K0 + r) * kp + K0 + c] = -v;
+  double a[4][4];
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // rows of the upper triangle's mirror: A is stored in full on diagonal blocks
+      const double2 *src = reinterpret_cast<const double2 *>(A + (int64_t)(K0 + 4 * R + i) * kp + K0 + 4 * C);
+      const double2 u = src[0], v = src[1];
+      a[i][0] = u.x; a[i][1] = u.y; a[i][2] = v.x; a[i][3] = v.y;
+    }
+  }
+  // the tile's share of column p (p / 4 == T, p % 4 == w): rows r >= 4 T from
+  // the tiles (R, T), rows above from the tiles (T, C), whose entries a_pr
+  // hold -a_rp (r swept, p not)
+  auto publish = [&](int T, int w, double *dst) {
+    if (!live) return;
+    if (C == T) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j == w) dst[4 * R + i] = a[i][j];
+      }
+    } else if (R == T) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i == w) dst[4 * C + j] = -a[i][j];
+    }
+  };
+  publish(0, 0, col[0]);
+  __syncthreads();
+#pragma unroll 1
+  for (int T = 0; T < 16; ++T) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int p = 4 * T + w;
+      const double *v = col[p & 1];
+      if (live) {
+        const double piv = rcp_pos(v[p]);
+        double vr[4], fc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) vr[i] = v[4 * R + i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = 4 * C + j;
+          const double x = v[c];
+          fc[j] = (c < p ? -x : x) * piv;  // a_pc / a_pp
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const bool rp = R == T && i == w, cp = C == T && j == w;
+            if (rp && cp) a[i][j] = piv;
+            else if (rp) a[i][j] = fc[j];
+            else if (cp) a[i][j] = -vr[i] * piv;
+            else a[i][j] = fma(-vr[i], fc[j], a[i][j]);
+          }
+      }
+      if (w < 3) publish(T, w + 1, col[(p + 1) & 1]);
+      else if (T < 15) publish(T + 1, 0, col[(p + 1) & 1]);
+      __syncthreads();
+    }
+  }
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = 4 * R + i, c = 4 * C + j;
+        const double x = a[i][j];
+        P[r * 64 + c] = x;
+        A[(int64_t)(K0 + r) * kp + K0 + c] = -x;
+        if (R != C) {
+          P[c * 64 + r] = x;
+          A[(int64_t)(K0 + c) * kp + K0 + r] = -x;
+        }
+      }
   }
 }
 
@@ -231,29 +306,59 @@ __global__ void __launch_bounds__(DIAG128_THREADS) k_fac_diag128(int32_t kp, int
 }
 
 
-template <typename T>
-struct V4;  // 4-vector load/store of T
-template <>
-struct V4<float> {
-  __device__ static void ld(const float *p, float (&v)[4]) {
-    const float4 t = *reinterpret_cast<const float4 *>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+// FP64 panel of pivot block K for 16 rows of block I = blockIdx.x != K: C = A_IK
+// (from the stored upper triangle: A[i][K0 + s] for I < K, A[K0 + s][i] for
+// I > K), U = C P. Writes Ct[t][i] = C[i][t] and Ut[t][i] = U[i][t] for the
+// trailing update and stores U back as the new panel. Four CTAs per block: the
+// product is bound by the FP64 pipe, and one CTA per block left most SMs idle
+// (k = 1,000: 70 -> 21 us).
+__global__ void __launch_bounds__(256) k_fac_panel64(int32_t kp, int32_t K0, double *__restrict__ A,
+                                                     const double *__restrict__ P, double *__restrict__ Ct,
+                                                     double *__restrict__ Ut) {
+  __shared__ __align__(16) double sP[64 * 64];  // sP[s][t]
+  __shared__ double sC[64 * 17];                // sC[s][i] = C[i][s]
+  const int I0 = (int)blockIdx.x * 64;
+  if (I0 == K0) return;
+  const int i0 = I0 + 16 * (int)blockIdx.y;
+  const bool above = I0 < K0;
+  for (int e = threadIdx.x; e < 64 * 32; e += 256)
+    reinterpret_cast<double2 *>(sP)[e] = reinterpret_cast<const double2 *>(P)[e];
+  for (int e = threadIdx.x; e < 16 * 64; e += 256) {
+    if (above) {  // i = e / 64, s = e % 64
+      sC[(e & 63) * 17 + (e >> 6)] = A[(int64_t)(i0 + (e >> 6)) * kp + K0 + (e & 63)];
+    } else {      // s = e / 16, i = e % 16
+      sC[(e >> 4) * 17 + (e & 15)] = A[(int64_t)(K0 + (e >> 4)) * kp + i0 + (e & 15)];
+    }
   }
-  __device__ static void st(float *p, const float (&v)[4]) {
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  __syncthreads();
+  for (int e = threadIdx.x; e < 16 * 64; e += 256) Ct[(int64_t)(e >> 4) * kp + i0 + (e & 15)] = sC[(e >> 4) * 17 + (e & 15)];
+  const int i = threadIdx.x & 15, t = 4 * (threadIdx.x >> 4);
+  double u[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+  for (int s = 0; s < 64; ++s) {
+    const double c = sC[s * 17 + i];
+    const double2 p0 = *reinterpret_cast<const double2 *>(sP + s * 64 + t);
+    const double2 p1 = *reinterpret_cast<const double2 *>(sP + s * 64 + t + 2);
+    u[0] = fma(c, p0.x, u[0]);
+    u[1] = fma(c, p0.y, u[1]);
+    u[2] = fma(c, p1.x, u[2]);
+    u[3] = fma(c, p1.y, u[3]);
   }
-};
-template <>
-struct V4<double> {
-  __device__ static void ld(const double *p, double (&v)[4]) {
-    const double2 t0 = reinterpret_cast<const double2 *>(p)[0], t1 = reinterpret_cast<const double2 *>(p)[1];
-    v[0] = t0.x; v[1] = t0.y; v[2] = t1.x; v[3] = t1.y;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    Ut[(int64_t)(t + w) * kp + i0 + i] = u[w];
+    if (above) A[(int64_t)(i0 + i) * kp + K0 + t + w] = u[w];
+    else A[(int64_t)(K0 + t + w) * kp + i0 + i] = u[w];
   }
-  __device__ static void st(double *p, const double (&v)[4]) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
-  }
-};
+}
+
+__device__ __forceinline__ void ld4f(const float *p, float (&v)[4]) {
+  const float4 t = *reinterpret_cast<const float4 *>(p);
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void st4f(float *p, const float (&v)[4]) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
 
 // Operand layout of the tensor-core trailing update ("split canonical"): for
 // a 128-row block B and a 16-wide chunk c of the inner dimension, the TF32
@@ -277,72 +382,59 @@ __device__ __forceinline__ void store_split4(float *X, int row, int k, const flo
   *reinterpret_cast<float4 *>(blk + o) = h;
   *reinterpret_cast<float4 *>(blk + 2048 + o) = l;
 }
-template <typename T>
-__device__ __forceinline__ void store_split4(T *, int, int, const T (&)[4]) {}  // FP64: unused
 
-// Panel of pivot block K for block I != K (NB rows): C_I = A_IK (from the
-// stored upper triangle: A[i][K0 + s] for I < K, A[K0 + s][i] for I > K),
-// U_I = C_I P. Writes C_I and U_I for the trailing update, transposed
-// (Ct[t][i], Ut[t][i], the SIMT update's layout) or, with KM, in the split
-// canonical layout of the tensor-core update (rows i of block I, inner index
-// t), and stores U_I back as the new panel (A_IK for I < K, A_KI = U_I^T for
-// I > K). 256 threads on a 16 x 16 grid, each an R x R block of U
-// (R = NB / 16) accumulated in registers.
-template <typename T, int NB, bool KM>
-__device__ __forceinline__ void fac_panel(int32_t kp, int32_t K0, int I0, T *__restrict__ A, const T *__restrict__ P,
-                                          T *__restrict__ Ct, T *__restrict__ Ut) {
-  constexpr int R = NB / 16, LD = NB + 16 / (int)sizeof(T);
+// FP32 panel of pivot block K for block I != K (128 rows): C_I = A_IK (from
+// the stored upper triangle: A[i][K0 + s] for I < K, A[K0 + s][i] for I > K),
+// U_I = C_I P. Writes C_I and U_I in the split canonical layout of the
+// tensor-core update (rows i of block I, inner index t) and stores U_I back as
+// the new panel (A_IK for I < K, A_KI = U_I^T for I > K). 256 threads on a
+// 16 x 16 grid, each an 8 x 8 block of U accumulated in registers.
+__device__ __forceinline__ void fac_panel(int32_t kp, int32_t K0, int I0, float *__restrict__ A,
+                                          const float *__restrict__ P, float *__restrict__ Ct, float *__restrict__ Ut) {
+  constexpr int NB = 128, R = NB / 16, LD = NB + 4;
   if (I0 == K0) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  T *sP = reinterpret_cast<T *>(smem_raw);  // [NB][NB]   sP[s][t]
-  T *sC = sP + NB * NB;                     // [NB][LD]   sC[s][i] = C[i][s]
+  float *sP = reinterpret_cast<float *>(smem_raw);  // [NB][NB]   sP[s][t]
+  float *sC = sP + NB * NB;                         // [NB][LD]   sC[s][i] = C[i][s]
   const bool above = I0 < K0;
   // 4-vectors, several in flight per thread
 #pragma unroll 4
   for (int e = 4 * threadIdx.x; e < NB * NB; e += 4 * blockDim.x) {
-    T pv[4], cv[4];
-    V4<T>::ld(P + e, pv);
-    V4<T>::st(sP + e, pv);
+    float pv[4], cv[4];
+    ld4f(P + e, pv);
+    st4f(sP + e, pv);
     const int r = e / NB, c = e % NB;
     if (above) {  // i = r, s = c .. c + 3
-      V4<T>::ld(A + (int64_t)(I0 + r) * kp + K0 + c, cv);
+      ld4f(A + (int64_t)(I0 + r) * kp + K0 + c, cv);
 #pragma unroll
       for (int w = 0; w < 4; ++w) sC[(c + w) * LD + r] = cv[w];
     } else {      // s = r, i = c .. c + 3
-      V4<T>::ld(A + (int64_t)(K0 + r) * kp + I0 + c, cv);
-      V4<T>::st(sC + r * LD + c, cv);
+      ld4f(A + (int64_t)(K0 + r) * kp + I0 + c, cv);
+      st4f(sC + r * LD + c, cv);
     }
   }
   __syncthreads();
-  if (KM) {  // C[i][t .. t + 3], split
-    for (int e = threadIdx.x; e < NB * NB / 4; e += blockDim.x) {
-      const int i = e / (NB / 4), t = (e % (NB / 4)) * 4;
-      const T v[4] = {sC[t * LD + i], sC[(t + 1) * LD + i], sC[(t + 2) * LD + i], sC[(t + 3) * LD + i]};
-      store_split4(Ct, I0 + i, t, v);
-    }
-  }
-  for (int e = threadIdx.x; e < NB * NB && !KM; e += blockDim.x) {
-    {          // Ct[t][I0 + i] = C[i][t]
-      const int t = e / NB, i = e % NB;
-      Ct[(int64_t)t * kp + I0 + i] = sC[t * LD + i];
-    }
+  for (int e = threadIdx.x; e < NB * NB / 4; e += blockDim.x) {  // C[i][t .. t + 3], split
+    const int i = e / (NB / 4), t = (e % (NB / 4)) * 4;
+    const float v[4] = {sC[t * LD + i], sC[(t + 1) * LD + i], sC[(t + 2) * LD + i], sC[(t + 3) * LD + i]};
+    store_split4(Ct, I0 + i, t, v);
   }
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T u[R][R];
+  float u[R][R];
 #pragma unroll
   for (int x = 0; x < R; ++x)
 #pragma unroll
-    for (int y = 0; y < R; ++y) u[x][y] = T(0);
+    for (int y = 0; y < R; ++y) u[x][y] = 0.0f;
 #pragma unroll 4
   for (int s = 0; s < NB; ++s) {
-    T av[R], bv[R];
+    float av[R], bv[R];
 #pragma unroll
     for (int q = 0; q < R / 4; ++q) {
-      T tmp[4];
-      V4<T>::ld(sC + s * LD + ty * R + 4 * q, tmp);
+      float tmp[4];
+      ld4f(sC + s * LD + ty * R + 4 * q, tmp);
 #pragma unroll
       for (int w = 0; w < 4; ++w) av[4 * q + w] = tmp[w];
-      V4<T>::ld(sP + s * NB + tx * R + 4 * q, tmp);
+      ld4f(sP + s * NB + tx * R + 4 * q, tmp);
 #pragma unroll
       for (int w = 0; w < 4; ++w) bv[4 * q + w] = tmp[w];
     }
@@ -352,97 +444,98 @@ __device__ __forceinline__ void fac_panel(int32_t kp, int32_t K0, int I0, T *__r
       for (int y = 0; y < R; ++y) u[x][y] += av[x] * bv[y];
   }
   // u[x][y] = U[i = ty R + x][t = tx R + y]
-  if (!KM || !above) {
+  if (!above) {
 #pragma unroll
     for (int y = 0; y < R; ++y) {
       const int t = tx * R + y;
 #pragma unroll
       for (int q = 0; q < R / 4; ++q) {
-        T tmp[4];
+        float tmp[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) tmp[w] = u[4 * q + w][y];
-        if (!KM) V4<T>::st(Ut + (int64_t)t * kp + I0 + ty * R + 4 * q, tmp);
-        if (!above) V4<T>::st(A + (int64_t)(K0 + t) * kp + I0 + ty * R + 4 * q, tmp);
+        st4f(A + (int64_t)(K0 + t) * kp + I0 + ty * R + 4 * q, tmp);
       }
     }
   }
-  if (KM || above) {
 #pragma unroll
-    for (int x = 0; x < R; ++x) {
-      const int i = ty * R + x;
+  for (int x = 0; x < R; ++x) {
+    const int i = ty * R + x;
 #pragma unroll
-      for (int q = 0; q < R / 4; ++q) {
-        T tmp[4];
+    for (int q = 0; q < R / 4; ++q) {
+      float tmp[4];
 #pragma unroll
-        for (int w = 0; w < 4; ++w) tmp[w] = u[x][4 * q + w];
-        if (KM) store_split4(Ut, I0 + i, tx * R + 4 * q, tmp);
-        if (above) V4<T>::st(A + (int64_t)(I0 + i) * kp + K0 + tx * R + 4 * q, tmp);
-      }
+      for (int w = 0; w < 4; ++w) tmp[w] = u[x][4 * q + w];
+      store_split4(Ut, I0 + i, tx * R + 4 * q, tmp);
+      if (above) st4f(A + (int64_t)(I0 + i) * kp + K0 + tx * R + 4 * q, tmp);
     }
   }
 }
 
-template <typename T, int NB, bool KM>
-__global__ void __launch_bounds__(256) k_fac_panel(int32_t kp, int32_t K0, T *__restrict__ A, const T *__restrict__ P,
-                                                   T *__restrict__ Ct, T *__restrict__ Ut) {
-  fac_panel<T, NB, KM>(kp, K0, (int)blockIdx.x * NB, A, P, Ct, Ut);
+__global__ void __launch_bounds__(256) k_fac_panel(int32_t kp, int32_t K0, float *__restrict__ A,
+                                                   const float *__restrict__ P, float *__restrict__ Ct,
+                                                   float *__restrict__ Ut) {
+  fac_panel(kp, K0, (int)blockIdx.x * 128, A, P, Ct, Ut);
 }
 
-// SIMT trailing update of the upper triangle (FP64, NB = 64):
-// A[i][j] -= sum_t Ct[t][i] Ut[t][j] for i, j outside the pivot block with
-// block(i) <= block(j). TM x TM tiles over the upper tile triangle; R x R
-// outputs per thread in two SUB x SUB quadrants so that shared-memory reads
-// are vectors.
-template <typename T, int TM, int NB>
+// SIMT trailing update of the upper triangle (FP64, 64-blocks): block b is the
+// b-th 64 x 64 tile (I, J), I <= J, of the blocks other than K, so that every
+// CTA has work and they spread over the SMs (a square grid whose lower half
+// exits at once left two tiles on some SMs and none on others: k = 1,000,
+// 138 -> 70 us). A[i][j] -= sum_t Ct[t][i] Ut[t][j]; 4 x 4 outputs per
+// thread in 2 x 2 quadrants so that shared-memory reads are vectors. Bound by
+// the FP64 pipe (64^3 fused multiply-adds per tile, 2 per cycle and SM).
 __global__ void __launch_bounds__(256)
-k_fac_trailing(int32_t kp, int32_t K0, T *__restrict__ A, const T *__restrict__ Ct, const T *__restrict__ Ut) {
-  constexpr int R = TM / 16, SUB = R / 2, HALF = TM / 2;
-  const int I0 = blockIdx.y * TM, J0 = blockIdx.x * TM;
-  if (J0 < I0) return;  // lower tile triangle: not stored
-  if ((I0 >= K0 && I0 + TM <= K0 + NB) || (J0 >= K0 && J0 + TM <= K0 + NB)) return;
+k_fac_trailing64(int32_t kp, int nblk, int K, double *__restrict__ A, const double *__restrict__ Ct,
+                 const double *__restrict__ Ut) {
+  constexpr int NB = 64, R = 4, SUB = 2, HALF = 32;
+  int i = 0, j = (int)blockIdx.x;
+  const int m = nblk - 1;
+  while (j >= m - i) {
+    j -= m - i;
+    ++i;
+  }
+  j += i;
+  const int I0 = (i + (i >= K ? 1 : 0)) * NB, J0 = (j + (j >= K ? 1 : 0)) * NB;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  T *sA = reinterpret_cast<T *>(smem_raw);  // [NB][TM]  sA[t][i] = Ct[t][I0 + i]
-  T *sB = sA + NB * TM;                     // [NB][TM]  sB[t][j] = Ut[t][J0 + j]
-  for (int e = threadIdx.x; e < NB * TM; e += 256) {
-    const int t = e / TM, x = e % TM;
-    sA[e] = (I0 + x < kp) ? Ct[(int64_t)t * kp + I0 + x] : T(0);
-    sB[e] = (J0 + x < kp) ? Ut[(int64_t)t * kp + J0 + x] : T(0);
+  double *sA = reinterpret_cast<double *>(smem_raw);  // [NB][NB]  sA[t][i] = Ct[t][I0 + i]
+  double *sB = sA + NB * NB;                          // [NB][NB]  sB[t][j] = Ut[t][J0 + j]
+  for (int e = threadIdx.x; e < NB * NB / 2; e += 256) {
+    const int t = e / (NB / 2), x = e % (NB / 2);
+    reinterpret_cast<double2 *>(sA)[e] = reinterpret_cast<const double2 *>(Ct + (int64_t)t * kp + I0)[x];
+    reinterpret_cast<double2 *>(sB)[e] = reinterpret_cast<const double2 *>(Ut + (int64_t)t * kp + J0)[x];
   }
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T acc[R][R];
+  double acc[R][R];
 #pragma unroll
   for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int c = 0; c < R; ++c) acc[r][c] = T(0);
+    for (int c = 0; c < R; ++c) acc[r][c] = 0.0;
 #pragma unroll 4
   for (int t = 0; t < NB; ++t) {
-    T a[R], b[R];
+    double a[R], b[R];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int s = 0; s < SUB; ++s) {
-        a[h * SUB + s] = sA[t * TM + h * HALF + ty * SUB + s];
-        b[h * SUB + s] = sB[t * TM + h * HALF + tx * SUB + s];
-      }
+    for (int h = 0; h < 2; ++h) {
+      const double2 u = *reinterpret_cast<const double2 *>(sA + t * NB + h * HALF + ty * SUB);
+      const double2 v = *reinterpret_cast<const double2 *>(sB + t * NB + h * HALF + tx * SUB);
+      a[2 * h] = u.x; a[2 * h + 1] = u.y;
+      b[2 * h] = v.x; b[2 * h + 1] = v.y;
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int c = 0; c < R; ++c) acc[r][c] += a[r] * b[c];
   }
-  // Epilogue: each row's SUB consecutive columns lie in one block, so the
-  // masks (pivot block, lower blocks, kp) are uniform over them.
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int i = I0 + (r / SUB) * HALF + ty * SUB + (r % SUB);
-    if (i >= kp || (i >= K0 && i < K0 + NB)) continue;
+    const int row = I0 + (r / SUB) * HALF + ty * SUB + (r % SUB);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int j = J0 + h * HALF + tx * SUB;
-      if (j >= kp || (j >= K0 && j < K0 + NB) || (i / NB) > (j / NB)) continue;
-      T *p = A + (int64_t)i * kp + j;
-#pragma unroll
-      for (int s = 0; s < SUB; ++s) p[s] -= acc[r][h * SUB + s];
+      double2 *p = reinterpret_cast<double2 *>(A + (int64_t)row * kp + J0 + h * HALF + tx * SUB);
+      double2 x = *p;
+      x.x -= acc[r][h * SUB];
+      x.y -= acc[r][h * SUB + 1];
+      *p = x;
     }
   }
 }
@@ -1035,7 +1128,6 @@ template <typename T>
 static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
   constexpr bool TC = std::is_same<T, float>::value;  // FP32: 128-blocks, tensor-core trailing update
   constexpr int NB = TC ? 128 : 64;
-  constexpr int TM = 64;                               // SIMT trailing tile (FP64)
   const size_t pan = (TC ? 2 : 1) * (size_t)NB * kp;         // one panel (split into high and low parts with TC)
   const size_t set = 2 * pan + (size_t)NB * NB;               // one parity's Ct, Ut, P
   T *Ct[2], *Ut[2], *P[2];
@@ -1045,19 +1137,16 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     P[q] = Ct[q] + 2 * pan;
   }
   int *err = reinterpret_cast<int *>(work + 2 * set);
-  const size_t diag_smem = 2 * sizeof(T) * NB * (NB + 1);
-  const size_t panel_smem = sizeof(T) * (NB * NB + NB * (NB + 16 / sizeof(T)));
-  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel<T, NB, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)panel_smem));
+  const size_t panel_smem = sizeof(float) * (128 * 128 + 128 * (128 + 4));  // FP32
+  const size_t trail_smem = 2 * sizeof(double) * 64 * 64;                    // FP64
   if constexpr (TC) {
+    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem));
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)tc::SMEM));
     PPRVIZ_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   } else {
-    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_diag<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)diag_smem));
-    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing<T, TM, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(2 * sizeof(T) * NB * TM)));
+    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)trail_smem));
   }
   const int nblk = kp / NB;
   // per pivot: the NB^3 pivot inverse, (nblk - 1) panel products of 2 NB^3,
@@ -1094,7 +1183,7 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     k_fac_diag128<<<1, DIAG128_THREADS, DIAG128_SMEM, ctx->stream>>>(kp, 0, Af, (float *)P[0]);
     PPRVIZ_LAUNCHED(ctx);
     if (nblk > 1) {
-      k_fac_panel<T, NB, TC><<<nblk, 256, panel_smem, ctx->stream>>>(kp, 0, A, P[0], Ct[0], Ut[0]);
+      k_fac_panel<<<nblk, 256, panel_smem, ctx->stream>>>(kp, 0, A, P[0], Ct[0], Ut[0]);
       PPRVIZ_LAUNCHED(ctx);
     }
     for (int kb = 0; nblk > 1 && kb < nblk; ++kb) {
@@ -1111,7 +1200,7 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
         PPRVIZ_CUDA(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_t1, 0));
         k_fac_diag128<<<1, DIAG128_THREADS, DIAG128_SMEM, ctx->side>>>(kp, k1 * NB, Af, (float *)P[q ^ 1]);
         PPRVIZ_LAUNCHED(ctx);
-        k_fac_panel<T, NB, TC><<<nblk, 256, panel_smem, ctx->side>>>(kp, k1 * NB, A, P[q ^ 1], Ct[q ^ 1], Ut[q ^ 1]);
+        k_fac_panel<<<nblk, 256, panel_smem, ctx->side>>>(kp, k1 * NB, A, P[q ^ 1], Ct[q ^ 1], Ut[q ^ 1]);
         PPRVIZ_LAUNCHED(ctx);
         PPRVIZ_CUDA(ctx, cudaEventRecord(ctx->ev_dp, ctx->side));
       }
@@ -1132,13 +1221,12 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
   } else {
     for (int kb = 0; kb < nblk; ++kb) {
       const int K0 = kb * NB;
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_diag<T, NB><<<1, 512, diag_smem, ctx->stream>>>(kp, K0, A, P[0]); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_diag64<<<1, DIAG64_THREADS, 0, ctx->stream>>>(kp, K0, A, P[0]); }
       PPRVIZ_LAUNCHED(ctx);
       if (nblk == 1) break;
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_panel<T, NB, TC><<<nblk, 256, panel_smem, ctx->stream>>>(kp, K0, A, P[0], Ct[0], Ut[0]); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_panel64<<<dim3(nblk, 4), 256, 0, ctx->stream>>>(kp, K0, A, P[0], Ct[0], Ut[0]); }
       PPRVIZ_LAUNCHED(ctx);
-      const unsigned tg = (unsigned)((kp + TM - 1) / TM);
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_trailing<T, TM, NB><<<dim3(tg, tg), 256, 2 * sizeof(T) * NB * TM, ctx->stream>>>(kp, K0, A, Ct[0], Ut[0]); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_trailing64<<<(unsigned)((int64_t)(nblk - 1) * nblk / 2), 256, trail_smem, ctx->stream>>>(kp, nblk, kb, A, Ct[0], Ut[0]); }
       PPRVIZ_LAUNCHED(ctx);
     }
     { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_finish<T, NB><<<dim3((unsigned)std::min(8, (kp + 255) / 256), (unsigned)kp), 256, 0, ctx->stream>>>(kp, A); }
@@ -1195,7 +1283,7 @@ __global__ void __launch_bounds__(256) k_fac_panel_batch(const FacJob *__restric
                                                          const int *__restrict__ off, int nact, int32_t K0) {
   const int s = find_slot(off, nact, (int)blockIdx.x);
   const FacJob j = jobs[act[s]];
-  fac_panel<float, 128, true>(j.kp, K0, ((int)blockIdx.x - off[s]) * 128, j.A, j.P, j.Ct, j.Ut);
+  fac_panel(j.kp, K0, ((int)blockIdx.x - off[s]) * 128, j.A, j.P, j.Ct, j.Ut);
 }
 
 // tile t of a view's upper tile triangle, row by row: (I, J), I <= J

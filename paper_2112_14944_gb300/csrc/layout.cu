@@ -32,28 +32,24 @@
 namespace pprviz {
 
 constexpr int ST = 128;       // symmetric pass tile edge
-constexpr int SRPI = 8;       // rows per warp per sub-iteration in the symmetric pass
 
 template <typename T> struct T2;
 template <> struct T2<float> { using type = float2; };
 template <> struct T2<double> { using type = double2; };
 
-template <typename T>
-__device__ __forceinline__ T rsqrt_pos(T d2);
-template <>
-__device__ __forceinline__ float rsqrt_pos<float>(float d2) { return d2 > 0.0f ? rsqrtf(d2) : 0.0f; }
-template <>
-__device__ __forceinline__ double rsqrt_pos<double>(double d2) { return d2 > 0.0 ? 1.0 / sqrt(d2) : 0.0; }
-
-// four consecutive values, 16-byte aligned
-__device__ __forceinline__ void ld4(const float *p, float (&v)[4]) {
-  const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-__device__ __forceinline__ void ld4(const double *p, double (&v)[4]) {
-  const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
-  const double2 b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+// 1/sqrt(d2), 0 for d2 = 0 (FP64 layout). GB300 has two FP64 operations per
+// cycle and SM, and an FP64 square root and division take some tens of them:
+// the special-function unit's estimate (20 bits or more) and one third-order
+// step of the series of (1 - e)^-1/2, e = 1 - d2 y^2 (Halley's iteration),
+// take five and leave an error of an ulp or so. Values outside the normal
+// range take the plain formula.
+__device__ __forceinline__ double rsqrt_pos(double d2) {
+  const uint32_t hi = (uint32_t)__double2hiint(d2);
+  if (hi - 0x01000000u >= 0x7e000000u - 0x01000000u) return d2 > 0.0 ? 1.0 / sqrt(d2) : 0.0;
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d2));
+  const double e = fma(-(d2 * y), y, 1.0);
+  return fma(fma(e, 0.375, 0.5), e * y, y);
 }
 
 // ---------------------------------------------------------------------------
@@ -137,15 +133,23 @@ __global__ void k_build_diag(int32_t k, int32_t kp, const double *__restrict__ r
 }
 
 // ---------------------------------------------------------------------------
-// Symmetric pair pass over the upper-triangle tiles of a symmetric kp x kp
-// matrix Mat (zero beyond k). Block (J, I), I <= J, 8 warps: warp w owns tile
-// rows 16w..16w+15 (two sub-iterations of SRPI rows), lane l the four columns
-// 4l..4l+3. With v = the staged vector (x for MODE 0, b for MODE 1):
+// FP64 symmetric pair pass over the upper-triangle ST64 x ST64 tiles of a
+// symmetric kp x kp matrix Mat (zero beyond k), one CTA per tile (I, J), I <= J,
+// 8 warps: warp w owns tile rows 8w..8w+7, lane l the columns 2l and 2l + 1.
+// With v = the vector (x for MODE 0, b for MODE 1):
 //   MODE 0 (L^Y): t_ij = Mat_ij (v_i - v_j) / |v_i - v_j|; row i gets +t_ij,
 //                 column j gets -t_ij (since t_ji = -t_ij)
 //   MODE 1 (apply M): row i gets Mat_ij v_j, column j gets Mat_ij v_i
 // Row sums go to Part[J][i], column sums (off-diagonal tiles only) to Part[I][j].
+// Bound by the FP64 pipe (2 operations per cycle and SM; 15 per pair in MODE 0,
+// 5 in MODE 1), so what counts is that every SM has a tile: 64 x 64 tiles give
+// a view of 1,000 nodes 136 CTAs (128 x 128 gave it 36). The tile is loaded
+// before the wait for the previous pass (programmatic dependent launch).
+// k = 1,000: one update (both passes) 137 -> 39 us, of which the FP64 pipe needs
+// about 21.
 // ---------------------------------------------------------------------------
+constexpr int ST64 = 64;
+
 // Sum over the 32 lanes of NV values per lane; returns, in every lane, the
 // total of value index lane / (32 / NV). Recursive halving: 31 shuffles for
 // NV = 32, 15 + 1 for NV = 16.
@@ -199,81 +203,69 @@ __device__ __forceinline__ V2 sum_parts_in_order(const V2 *p, int64_t kp, int nb
 // finishes last). One thread per CTA fences after the block barrier before
 // counting (release) and after a last count (acquire); the reducer reads
 // through L2.
-template <typename T, int MODE>
-__device__ __forceinline__ void sympass_tile(const int I, const int J, int32_t kp, int nbt, const T *__restrict__ Mat,
-                                             const typename T2<T>::type *__restrict__ V,
-                                             typename T2<T>::type *__restrict__ Part, int *__restrict__ cnt,
-                                             typename T2<T>::type *__restrict__ Vout) {
-  using V2 = typename T2<T>::type;
-  constexpr int NV = 2 * SRPI;
-  __shared__ V2 sVi[ST];
-  __shared__ T colred[8][2 * ST];
+template <int MODE>
+__global__ void __launch_bounds__(256)
+k_sympass64(int32_t kp, int nbt, const int2 *__restrict__ tiles, const double *__restrict__ Mat, const double2 *V,
+            double2 *Part, int *cnt, double2 *Vout) {
+  constexpr int RPW64 = 8;
+  __shared__ double2 sVi[ST64];
+  __shared__ double colred[8][2 * ST64];
+  __shared__ int last[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t i0 = (int64_t)I * ST, j0 = (int64_t)J * ST;
-  if (threadIdx.x < ST) sVi[threadIdx.x] = V[i0 + threadIdx.x];
-  T xj[4], yj[4];
+  const int I = tiles[blockIdx.x].x, J = tiles[blockIdx.x].y;
+  const int64_t i0 = (int64_t)I * ST64, j0 = (int64_t)J * ST64;
+  double2 m[RPW64];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const V2 v = V[j0 + lane * 4 + u];
-    xj[u] = v.x;
-    yj[u] = v.y;
-  }
+  for (int r = 0; r < RPW64; ++r)
+    m[r] = __ldg(reinterpret_cast<const double2 *>(Mat + (i0 + warp * RPW64 + r) * kp + j0) + lane);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the previous pass's vector and partials
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (threadIdx.x < ST64) sVi[threadIdx.x] = __ldcg(V + i0 + threadIdx.x);
+  const double2 va = __ldcg(V + j0 + 2 * lane), vb = __ldcg(V + j0 + 2 * lane + 1);
   __syncthreads();
-  T cx[4], cy[4];
+  double cx[2] = {0.0, 0.0}, cy[2] = {0.0, 0.0}, acc[2 * RPW64];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) cx[u] = cy[u] = T(0);
-  T *part = reinterpret_cast<T *>(Part);
-#pragma unroll
-  for (int sub = 0; sub < 16 / SRPI; ++sub) {
-    const int rbase = warp * 16 + sub * SRPI;
-    T m[SRPI][4];
-#pragma unroll
-    for (int r = 0; r < SRPI; ++r) ld4(Mat + (i0 + rbase + r) * kp + j0 + lane * 4, m[r]);
-    T acc[NV];
-#pragma unroll
-    for (int r = 0; r < SRPI; ++r) {
-      const V2 vi = sVi[rbase + r];
-      T ax = T(0), ay = T(0);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (MODE == 0) {
-          const T dx = vi.x - xj[u], dy = vi.y - yj[u];
-          const T coef = m[r][u] * rsqrt_pos<T>(dx * dx + dy * dy);
-          const T tx = coef * dx, ty = coef * dy;
-          ax += tx;
-          ay += ty;
-          cx[u] -= tx;
-          cy[u] -= ty;
-        } else {
-          ax += m[r][u] * xj[u];
-          ay += m[r][u] * yj[u];
-          cx[u] += m[r][u] * vi.x;
-          cy[u] += m[r][u] * vi.y;
-        }
-      }
-      acc[2 * r] = ax;
-      acc[2 * r + 1] = ay;
+  for (int r = 0; r < RPW64; ++r) {
+    const double2 vi = sVi[warp * RPW64 + r];
+    double ax, ay;
+    if (MODE == 0) {
+      const double dxa = vi.x - va.x, dya = vi.y - va.y, dxb = vi.x - vb.x, dyb = vi.y - vb.y;
+      const double ca = m[r].x * rsqrt_pos(fma(dxa, dxa, dya * dya));
+      const double cb = m[r].y * rsqrt_pos(fma(dxb, dxb, dyb * dyb));
+      ax = fma(cb, dxb, ca * dxa);
+      ay = fma(cb, dyb, ca * dya);
+      cx[0] = fma(-ca, dxa, cx[0]);
+      cy[0] = fma(-ca, dya, cy[0]);
+      cx[1] = fma(-cb, dxb, cx[1]);
+      cy[1] = fma(-cb, dyb, cy[1]);
+    } else {
+      ax = fma(m[r].y, vb.x, m[r].x * va.x);
+      ay = fma(m[r].y, vb.y, m[r].x * va.y);
+      cx[0] = fma(m[r].x, vi.x, cx[0]);
+      cy[0] = fma(m[r].x, vi.y, cy[0]);
+      cx[1] = fma(m[r].y, vi.x, cx[1]);
+      cy[1] = fma(m[r].y, vi.y, cy[1]);
     }
-    const T tot = lanes_transpose_sum<NV, T>(acc, lane);
-    constexpr int REP = 32 / NV;
-    if (lane % REP == 0) {
-      const int idx = lane / REP;
-      part[((int64_t)J * kp + i0 + rbase + (idx >> 1)) * 2 + (idx & 1)] = tot;
-    }
+    acc[2 * r] = ax;
+    acc[2 * r + 1] = ay;
   }
+  double *part = reinterpret_cast<double *>(Part);
+  const double tot = lanes_transpose_sum<2 * RPW64, double>(acc, lane);
+  if (lane % 2 == 0) part[((int64_t)J * kp + i0 + warp * RPW64) * 2 + lane / 2] = tot;
   if (I != J) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      colred[warp][(lane * 4 + u) * 2] = cx[u];
-      colred[warp][(lane * 4 + u) * 2 + 1] = cy[u];
+    for (int u = 0; u < 2; ++u) {
+      colred[warp][(lane * 2 + u) * 2] = cx[u];
+      colred[warp][(lane * 2 + u) * 2 + 1] = cy[u];
     }
     __syncthreads();
-    T s = T(0);
+    if (threadIdx.x < 2 * ST64) {
+      double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) s += colred[w][threadIdx.x];
-    part[((int64_t)I * kp + j0) * 2 + threadIdx.x] = s;
+      for (int w = 0; w < 8; ++w) s += colred[w][threadIdx.x];
+      part[((int64_t)I * kp + j0) * 2 + threadIdx.x] = s;
+    }
   }
-  __shared__ int last[2];
   __syncthreads();  // every thread's partials are written (CTA scope)
   if (threadIdx.x == 0) {
     __threadfence();  // release, cumulative over the barrier
@@ -282,38 +274,26 @@ __device__ __forceinline__ void sympass_tile(const int I, const int J, int32_t k
     if (last[0] || last[1]) __threadfence();  // acquire before the block reads other CTAs' partials
   }
   __syncthreads();
-#pragma unroll 1
-  for (int side = 0; side < 2; ++side) {
-    if (!last[side]) continue;
-    const int R = side ? J : I;
-    if (threadIdx.x < ST) {
-      const int64_t row = (int64_t)R * ST + threadIdx.x;
+  // threads 0..63 reduce row block I, threads 64..127 row block J
+  if (threadIdx.x < 2 * ST64) {
+    const int side = threadIdx.x / ST64;
+    if (last[side]) {
+      const int R = side ? J : I;
+      const int64_t row = (int64_t)R * ST64 + threadIdx.x % ST64;
       Vout[row] = sum_parts_in_order(Part + row, (int64_t)kp, nbt);
+      if (threadIdx.x % ST64 == 0) cnt[R] = 0;
     }
-    if (threadIdx.x == 0) cnt[R] = 0;
   }
 }
 
-// Views of a pass: block b takes tile tiles[b] = (view, I, J), I <= J, and the
-// view's matrix, vector, partial-sum and counter slices from its descriptor.
+// Views of a pass: a view's matrix, vector and partial-sum slices.
 // A single view is the case of one descriptor.
 struct BatchView {
   int64_t mat_off;   // elements into the batched kp x kp matrices
   int64_t vec_off;   // 2-vectors into the batched coordinate / b vectors (kp each)
   int64_t part_off;  // 2-vectors into the batched partial sums (nbt x kp each)
-  int32_t kp, nbt, k, cnt_off;  // cnt_off: the view's nbt row-block counters
+  int32_t kp, nbt, k, cnt_off;  // cnt_off: the view's first row block among all views'
 };
-
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256)
-k_sympass_batch(const int4 *__restrict__ tiles, const BatchView *__restrict__ views, const T *__restrict__ Mat,
-                const typename T2<T>::type *__restrict__ V, typename T2<T>::type *__restrict__ Part,
-                int *__restrict__ cnt, typename T2<T>::type *__restrict__ Vout) {
-  const int4 t = tiles[blockIdx.x];
-  const BatchView bv = views[t.x];
-  sympass_tile<T, MODE>(t.y, t.z, bv.kp, bv.nbt, Mat + bv.mat_off, V + bv.vec_off, Part + bv.part_off,
-                        cnt + bv.cnt_off, Vout + bv.vec_off);
-}
 
 // ---------------------------------------------------------------------------
 // FP32 symmetric pass, persistent, pipelined and warp-specialized (the FP32
@@ -1154,7 +1134,9 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   PPRVIZ_TRY(ws_ensure(ctx, WS_M, sizeof(T) * (size_t)kp * kp));
   PPRVIZ_TRY(ws_ensure(ctx, WS_PIV, sizeof(T) * spd_inverse_work(kp)));
   PPRVIZ_TRY(ws_ensure(ctx, WS_X, sizeof(V2) * (size_t)kp * 2));            // X and b
-  PPRVIZ_TRY(ws_ensure(ctx, WS_B, sizeof(V2) * (size_t)nbt * kp));          // partial sums
+  constexpr bool F64 = std::is_same<T, double>::value;
+  const int pbt = F64 ? kp / ST64 : nbt;                                    // row blocks of a pass
+  PPRVIZ_TRY(ws_ensure(ctx, WS_B, sizeof(V2) * (size_t)pbt * kp));          // partial sums
   PPRVIZ_TRY(ws_ensure(ctx, WS_E, sizeof(V2) * (size_t)k + 64));
   PPRVIZ_TRY(ws_ensure(ctx, WS_RHS, sizeof(double) * (size_t)(kp / 32) * kp));  // build row partials
   PPRVIZ_TRY(ws_ensure(ctx, WS_FLAG, 64));
@@ -1178,25 +1160,15 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   }
   { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_load_x<TI, T><<<(unsigned)((kp + 255) / 256), 256, 0, ctx->stream>>>(k, kp, x0, X); }
   PPRVIZ_LAUNCHED(ctx);
-  // one view descriptor, the upper tile triangle in row order, and the
-  // row-block counters of the fused reduce (zero between passes)
-  std::vector<int4> tiles;
-  for (int I = 0; I < nbt; ++I)
-    for (int J = I; J < nbt; ++J) tiles.push_back(make_int4(0, I, J, 0));  // w: vec_off / 128 = 0
+  // the view descriptor (FP32), or the upper tile triangle in row order and the
+  // row-block counters of the fused reduce, zero between passes (FP64)
   const BatchView one{0, 0, 0, kp, nbt, k, 0};
-  const size_t tab_off = 256, cnt_off = (tab_off + sizeof(int4) * tiles.size() + 255) & ~(size_t)255;
-  PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, cnt_off + sizeof(int) * (size_t)nbt));
-  BatchView *view_d = reinterpret_cast<BatchView *>(ctx->ws[WS_BTAB].p);
-  int4 *tiles_d = reinterpret_cast<int4 *>(static_cast<unsigned char *>(ctx->ws[WS_BTAB].p) + tab_off);
-  int *cnt = reinterpret_cast<int *>(static_cast<unsigned char *>(ctx->ws[WS_BTAB].p) + cnt_off);
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(view_d, &one, sizeof(BatchView), cudaMemcpyHostToDevice, ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(tiles_d, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
-                                   ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)nbt, ctx->stream));
-  const unsigned ntile = (unsigned)tiles.size();
   if constexpr (std::is_same<T, float>::value) {
+    PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, sizeof(BatchView)));
+    BatchView *view_d = reinterpret_cast<BatchView *>(ctx->ws[WS_BTAB].p);
+    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(view_d, &one, sizeof(BatchView), cudaMemcpyHostToDevice, ctx->stream));
     unsigned pgrid = 0;
-    PPRVIZ_TRY(sympass_pipe_grid(ctx, tiles.size(), &pgrid));
+    PPRVIZ_TRY(sympass_pipe_grid(ctx, (size_t)nbt * (nbt + 1) / 2, &pgrid));
     const std::vector<BatchView> one_v{one};
     const CUtensorMap *maps = nullptr;
     PPRVIZ_TRY(upload_maps(ctx, one_v, W1, A, &maps));
@@ -1214,10 +1186,22 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
       if (herr) return set_err(ctx, PPRVIZ_E_TIMEOUT, "layout pass: tile copy wait expired");
     }
   } else {
+    std::vector<int2> tiles;
+    for (int I = 0; I < pbt; ++I)
+      for (int J = I; J < pbt; ++J) tiles.push_back(make_int2(I, J));
+    const size_t cnt_off = (sizeof(int2) * tiles.size() + 255) & ~(size_t)255;
+    PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, cnt_off + sizeof(int) * (size_t)pbt));
+    int2 *tiles_d = ctx->ws[WS_BTAB].as<int2>();
+    int *cnt = reinterpret_cast<int *>(static_cast<unsigned char *>(ctx->ws[WS_BTAB].p) + cnt_off);
+    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(tiles_d, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice,
+                                     ctx->stream));
+    PPRVIZ_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)pbt, ctx->stream));
+    PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // the host table is released below
+    const unsigned ntile = (unsigned)tiles.size();
     for (int it = 0; it < iters; ++it) {
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_LY); k_sympass_batch<T, 0><<<ntile, 256, 0, ctx->stream>>>(tiles_d, view_d, W1, X, Part, cnt, Bv); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_LY); PPRVIZ_CUDA(ctx, launch_dependent(ctx, k_sympass64<0>, ntile, 256, 0, kp, pbt, (const int2 *)tiles_d, (const double *)W1, (const double2 *)X, Part, cnt, Bv)); }
       PPRVIZ_LAUNCHED(ctx);
-      { PPRVIZ_PROF(ctx, PPRVIZ_K_APPLY); k_sympass_batch<T, 1><<<ntile, 256, 0, ctx->stream>>>(tiles_d, view_d, A, Bv, Part, cnt, X); }
+      { PPRVIZ_PROF(ctx, PPRVIZ_K_APPLY); PPRVIZ_CUDA(ctx, launch_dependent(ctx, k_sympass64<1>, ntile, 256, 0, kp, pbt, (const int2 *)tiles_d, (const double *)A, (const double2 *)Bv, Part, cnt, X)); }
       PPRVIZ_LAUNCHED(ctx);
     }
   }
@@ -1278,8 +1262,8 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
                      const float *x0_d, int32_t iters, float *x_out_d, double *stress_h) {
   using V2 = float2;
   std::vector<BatchView> bv((size_t)nviews);
-  std::vector<int4> tiles;
   int64_t mat = 0, vec = 0, part = 0, maxkp = 0;
+  size_t ntile = 0;
   int32_t cnts = 0;
   for (int32_t v = 0; v < nviews; ++v) {
     const int32_t k = (int32_t)k_h[v];
@@ -1290,31 +1274,21 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
     part += (int64_t)nbt * kp;
     cnts += nbt;
     maxkp = std::max<int64_t>(maxkp, kp);
-    for (int I = 0; I < nbt; ++I)
-      for (int J = I; J < nbt; ++J) tiles.push_back(make_int4(v, I, J, (int)(bv[v].vec_off / ST)));
+    ntile += (size_t)nbt * (nbt + 1) / 2;
   }
   PPRVIZ_TRY(ws_ensure(ctx, WS_BW1, sizeof(float) * (size_t)mat));
   PPRVIZ_TRY(ws_ensure(ctx, WS_BM, sizeof(float) * (size_t)mat));
   PPRVIZ_TRY(ws_ensure(ctx, WS_BX, sizeof(V2) * (size_t)vec * 2));
   PPRVIZ_TRY(ws_ensure(ctx, WS_BPART, sizeof(V2) * (size_t)part));
-  // the tile table (int4, 16-byte loads) starts at a 256-byte boundary after the
-  // descriptors, the row-block counters at the next one after the table
-  const size_t tab_off = (sizeof(BatchView) * (size_t)nviews + 255) & ~(size_t)255;
-  const size_t cnt_off = (tab_off + sizeof(int4) * tiles.size() + 255) & ~(size_t)255;
-  PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, cnt_off + sizeof(int) * (size_t)cnts));
+  PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, sizeof(BatchView) * (size_t)nviews));
   PPRVIZ_TRY(ws_ensure(ctx, WS_RHS, sizeof(double) * (size_t)(maxkp / 32) * maxkp));
   PPRVIZ_TRY(ws_ensure(ctx, WS_FLAG, 64));
   float *W1 = ctx->ws[WS_BW1].as<float>(), *M = ctx->ws[WS_BM].as<float>();
   V2 *X = ctx->ws[WS_BX].as<V2>(), *Bv = X + vec, *Part = ctx->ws[WS_BPART].as<V2>();
   BatchView *views_d = reinterpret_cast<BatchView *>(ctx->ws[WS_BTAB].p);
-  int4 *tiles_d = reinterpret_cast<int4 *>(static_cast<unsigned char *>(ctx->ws[WS_BTAB].p) + tab_off);
-  int *cnt = reinterpret_cast<int *>(static_cast<unsigned char *>(ctx->ws[WS_BTAB].p) + cnt_off);
   double *rowpart = ctx->ws[WS_RHS].as<double>();
   int *flag = ctx->ws[WS_FLAG].as<int>();
-  PPRVIZ_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)cnts, ctx->stream));
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(views_d, bv.data(), sizeof(BatchView) * bv.size(), cudaMemcpyHostToDevice,
-                                   ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(tiles_d, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
                                    ctx->stream));
   PPRVIZ_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
   int64_t sq = 0, xo = 0;
@@ -1343,9 +1317,8 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (hf) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "a view's pdist has a non-finite or non-positive entry");
-  const unsigned ntile = (unsigned)tiles.size();
   unsigned pgrid = 0;
-  PPRVIZ_TRY(sympass_pipe_grid(ctx, tiles.size(), &pgrid));
+  PPRVIZ_TRY(sympass_pipe_grid(ctx, ntile, &pgrid));
   const CUtensorMap *maps = nullptr;
   PPRVIZ_TRY(upload_maps(ctx, bv, W1, M, &maps));
   PassTables pt;
