@@ -139,164 +139,96 @@ __global__ void __launch_bounds__(DIAG64_THREADS) k_fac_diag64(int32_t kp, int32
   }
 }
 
-// D = A_JJ^-1 for the 32 x 32 block J of a 128 x 128 block whose column
-// block J is stored transposed in colT (colT[c][r] = A[r][32 J + c]), by one
-// warp: the element sweep above in registers, lane = row. Per pivot p lane p
-// publishes its row in a shared buffer (two, alternating, so one warp
-// barrier per pivot suffices) and every lane reads it back with 16-byte
-// broadcast loads. Writes D and its transpose.
-__device__ __noinline__ void warp_inv32(const float *colT, int J, float *D, float *DT, float *rowbuf) {
-  const int l = threadIdx.x & 31;
-  float d[32];
-#pragma unroll
-  for (int c = 0; c < 32; ++c) d[c] = colT[c * 128 + 32 * J + l];
-#pragma unroll
-  for (int p = 0; p < 32; ++p) {
-    float *rb = rowbuf + (p & 1) * 32;
-    if (l == p) {
-#pragma unroll
-      for (int c = 0; c < 32; c += 4)
-        *reinterpret_cast<float4 *>(rb + c) = make_float4(d[c], d[c + 1], d[c + 2], d[c + 3]);
-    }
-    __syncwarp();
-    const float piv = 1.0f / rb[p];
-    const float f = d[p] * piv;  // a_lp / a_pp
-#pragma unroll
-    for (int c = 0; c < 32; c += 4) {
-      const float4 v = *reinterpret_cast<const float4 *>(rb + c);
-      const float vs[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) d[c + e] = (l == p) ? vs[e] * piv : fmaf(-f, vs[e], d[c + e]);
-    }
-    d[p] = (l == p) ? piv : -f;
-  }
-#pragma unroll
-  for (int c = 0; c < 32; ++c) {
-    D[l * 32 + c] = d[c];
-    DT[c * 32 + l] = d[c];
-  }
-}
-
-// The same sweep for a 128 x 128 FP32 block, in four 32-wide block steps
-// (the block form of the sweep: sweeping the 32 pivots of block J at once is
-// D = A_JJ^-1, A_JL <- D A_JL, A_IJ <- -A_IJ D, A_IL <- A_IL - A_IJ D A_JL,
-// A_JJ <- D, the same result as 32 single-pivot sweeps). The block lives in
-// registers, a 4 x 8 tile per thread (512 threads): thread t owns rows
-// 4 (t / 16) + i and columns 8 (t % 16) + j. Per block step the old row block
-// J and the old column block J (transposed) go to shared memory, one warp
-// inverts A_JJ, and every thread updates its tile with 32-term products
-// (three 16-byte shared loads per 32 FMAs): four barriers per block step
-// instead of one per pivot. Dynamic shared memory: DIAG128_SMEM bytes.
-constexpr int DIAG128_THREADS = 512;
-constexpr int DIAG128_SMEM = (3 * 32 * 128 + 2 * 32 * 32 + 64) * 4;
+// The same sweep for a 128 x 128 FP32 block: 528 threads hold the 4 x 4 tiles on
+// and below the diagonal (16 registers each), one barrier per pivot. Bound by
+// the chain publish -> barrier -> read -> reciprocal -> update of its 128
+// pivots and by issuing ~45 instructions per thread and pivot on one SM; a
+// version in four 32-wide block steps, each waiting for a one-warp inverse of
+// its 32 x 32 pivot, took 59 us, this one 35 us.
+constexpr int DIAG128_THREADS = 544;
 __device__ __forceinline__ void fac_diag128(int32_t kp, int32_t K0, float *__restrict__ A, float *__restrict__ P) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  float *sRowJ = reinterpret_cast<float *>(smem_raw);  // [32][128] old rows of block J
-  float *sColT = sRowJ + 32 * 128;                     // [32][128] old column block J, transposed
-  float *sNewT = sColT + 32 * 128;                     // [32][128] new column block J, transposed
-  float *sD = sNewT + 32 * 128;                        // [32][32] A_JJ^-1
-  float *sDT = sD + 32 * 32;                           // [32][32] its transpose
-  float *sPiv = sDT + 32 * 32;                         // [2][32] pivot rows of the warp inverse
-  const int rb = threadIdx.x >> 4, cb = threadIdx.x & 15;
-  float a[4][8];  // a[i][j] = row 4 rb + i, column 8 cb + j
+  __shared__ __align__(16) float col[2][128];
+  // thread t < 528 holds tile (R, C), R >= C: t = R (R + 1) / 2 + C
+  const int t = (int)threadIdx.x;
+  const bool live = t < 528;
+  int R = live ? (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f) : 0;
+  if (live && (R + 1) * (R + 2) / 2 <= t) ++R;
+  if (live && R * (R + 1) / 2 > t) --R;
+  const int C = live ? t - R * (R + 1) / 2 : 0;
+  float a[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float *src = A + (int64_t)(K0 + 4 * rb + i) * kp + K0 + 8 * cb;
-    const float4 v0 = *reinterpret_cast<const float4 *>(src), v1 = *reinterpret_cast<const float4 *>(src + 4);
-    a[i][0] = v0.x; a[i][1] = v0.y; a[i][2] = v0.z; a[i][3] = v0.w;
-    a[i][4] = v1.x; a[i][5] = v1.y; a[i][6] = v1.z; a[i][7] = v1.w;
+    const float4 u = *reinterpret_cast<const float4 *>(A + (int64_t)(K0 + 4 * R + i) * kp + K0 + 4 * C);
+    a[i][0] = u.x; a[i][1] = u.y; a[i][2] = u.z; a[i][3] = u.w;
   }
+  // the tile's share of column 4 T + w: rows from 4 T on lie in the tiles
+  // (R, T); the rows above, all swept, in the tiles (T, C) as a_pr = -a_rp
+  auto publish = [&](int T, int w, float *dst) {
+    if (!live) return;
+    if (C == T) {
+      float4 v;
+      v.x = w == 0 ? a[0][0] : w == 1 ? a[0][1] : w == 2 ? a[0][2] : a[0][3];
+      v.y = w == 0 ? a[1][0] : w == 1 ? a[1][1] : w == 2 ? a[1][2] : a[1][3];
+      v.z = w == 0 ? a[2][0] : w == 1 ? a[2][1] : w == 2 ? a[2][2] : a[2][3];
+      v.w = w == 0 ? a[3][0] : w == 1 ? a[3][1] : w == 2 ? a[3][2] : a[3][3];
+      *reinterpret_cast<float4 *>(dst + 4 * R) = v;
+    } else if (R == T) {
+      const float *r = w == 0 ? a[0] : w == 1 ? a[1] : w == 2 ? a[2] : a[3];
+      *reinterpret_cast<float4 *>(dst + 4 * C) = make_float4(-r[0], -r[1], -r[2], -r[3]);
+    }
+  };
+  publish(0, 0, col[0]);
+  __syncthreads();
 #pragma unroll 1
-  for (int J = 0; J < 4; ++J) {
-    const bool rowJ = (rb >> 3) == J, colJ = (cb >> 2) == J;
-    const int ri = 4 * (rb & 7), ci = 8 * (cb & 3);  // offsets inside block J
-    if (rowJ) {
+  for (int T = 0; T < 32; ++T) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float *dst = sRowJ + (ri + i) * 128 + 8 * cb;
-        *reinterpret_cast<float4 *>(dst) = make_float4(a[i][0], a[i][1], a[i][2], a[i][3]);
-        *reinterpret_cast<float4 *>(dst + 4) = make_float4(a[i][4], a[i][5], a[i][6], a[i][7]);
-      }
-    }
-    if (colJ) {
+    for (int w = 0; w < 4; ++w) {
+      const float *v = col[w & 1];  // 4 T is even
+      {
+        // 1 / a_pp: the estimate and one Newton step
+        const float app = v[4 * T + w];
+        float piv;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(piv) : "f"(app));
+        piv = fmaf(fmaf(-app, piv, 1.0f), piv, piv);
+        const float4 r4 = *reinterpret_cast<const float4 *>(v + 4 * R);
+        const float4 c4 = *reinterpret_cast<const float4 *>(v + 4 * C);
+        const float vr[4] = {r4.x, r4.y, r4.z, r4.w};
+        const float vc[4] = {c4.x, c4.y, c4.z, c4.w};
+        float fc[4];  // a_pc / a_pp; a_pc = -a_cp where c is swept
+        const float ps = C < T ? -piv : piv;
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<float4 *>(sColT + (ci + j) * 128 + 4 * rb) = make_float4(a[0][j], a[1][j], a[2][j], a[3][j]);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) warp_inv32(sColT, J, sD, sDT, sPiv);
-    __syncthreads();
-    if (rowJ) {  // A_JL <- D A_JL (the pivot block itself becomes D)
-      if (colJ) {
+        for (int j = 0; j < 4; ++j) fc[j] = vc[j] * (j < w && C == T ? -piv : ps);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) a[i][j] = sD[(ri + i) * 32 + ci + j];
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) a[i][j] = 0.0f;
-#pragma unroll 4
-        for (int t = 0; t < 32; ++t) {
-          const float4 x = *reinterpret_cast<const float4 *>(sDT + t * 32 + ri);
-          const float4 y0 = *reinterpret_cast<const float4 *>(sRowJ + t * 128 + 8 * cb);
-          const float4 y1 = *reinterpret_cast<const float4 *>(sRowJ + t * 128 + 8 * cb + 4);
-          const float xs[4] = {x.x, x.y, x.z, x.w};
-          const float ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) a[i][j] = fmaf(xs[i], ys[j], a[i][j]);
-        }
+          for (int j = 0; j < 4; ++j) {
+            float n = fmaf(-vr[i], fc[j], a[i][j]);
+            if (i == w) n = R == T ? fc[j] : n;
+            if (j == w) n = C == T ? ((i == w && R == T) ? piv : -vr[i] * piv) : n;
+            a[i][j] = n;
+          }
       }
-    } else if (colJ) {  // A_IJ <- -A_IJ D, also published for the other tiles of the rows
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) a[i][j] = 0.0f;
-#pragma unroll 4
-      for (int t = 0; t < 32; ++t) {
-        const float4 x = *reinterpret_cast<const float4 *>(sColT + t * 128 + 4 * rb);
-        const float4 y0 = *reinterpret_cast<const float4 *>(sD + t * 32 + ci);
-        const float4 y1 = *reinterpret_cast<const float4 *>(sD + t * 32 + ci + 4);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
-        const float ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) a[i][j] = fmaf(-xs[i], ys[j], a[i][j]);
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<float4 *>(sNewT + (ci + j) * 128 + 4 * rb) = make_float4(a[0][j], a[1][j], a[2][j], a[3][j]);
+      if (w < 3) publish(T, w + 1, col[(w + 1) & 1]);
+      else if (T < 31) publish(T + 1, 0, col[0]);
+      __syncthreads();
     }
-    __syncthreads();
-    if (!rowJ && !colJ) {  // A_IL <- A_IL + (-A_IJ D) A_JL
-#pragma unroll 4
-      for (int t = 0; t < 32; ++t) {
-        const float4 x = *reinterpret_cast<const float4 *>(sNewT + t * 128 + 4 * rb);
-        const float4 y0 = *reinterpret_cast<const float4 *>(sRowJ + t * 128 + 8 * cb);
-        const float4 y1 = *reinterpret_cast<const float4 *>(sRowJ + t * 128 + 8 * cb + 4);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
-        const float ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) a[i][j] = fmaf(xs[i], ys[j], a[i][j]);
-      }
-    }
-    __syncthreads();  // before the next block step restages
   }
+  if (!live) return;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int r = 4 * rb + i;
-    float *p = P + r * 128 + 8 * cb;
-    float *q = A + (int64_t)(K0 + r) * kp + K0 + 8 * cb;
-    *reinterpret_cast<float4 *>(p) = make_float4(a[i][0], a[i][1], a[i][2], a[i][3]);
-    *reinterpret_cast<float4 *>(p + 4) = make_float4(a[i][4], a[i][5], a[i][6], a[i][7]);
-    *reinterpret_cast<float4 *>(q) = make_float4(-a[i][0], -a[i][1], -a[i][2], -a[i][3]);
-    *reinterpret_cast<float4 *>(q + 4) = make_float4(-a[i][4], -a[i][5], -a[i][6], -a[i][7]);
+    const int r = 4 * R + i;
+    *reinterpret_cast<float4 *>(P + r * 128 + 4 * C) = make_float4(a[i][0], a[i][1], a[i][2], a[i][3]);
+    *reinterpret_cast<float4 *>(A + (int64_t)(K0 + r) * kp + K0 + 4 * C) =
+        make_float4(-a[i][0], -a[i][1], -a[i][2], -a[i][3]);
+  }
+  if (R != C) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = 4 * C + j;
+      *reinterpret_cast<float4 *>(P + r * 128 + 4 * R) = make_float4(a[0][j], a[1][j], a[2][j], a[3][j]);
+      *reinterpret_cast<float4 *>(A + (int64_t)(K0 + r) * kp + K0 + 4 * R) =
+          make_float4(-a[0][j], -a[1][j], -a[2][j], -a[3][j]);
+    }
   }
 }
 
@@ -352,14 +284,6 @@ __global__ void __launch_bounds__(256) k_fac_panel64(int32_t kp, int32_t K0, dou
   }
 }
 
-__device__ __forceinline__ void ld4f(const float *p, float (&v)[4]) {
-  const float4 t = *reinterpret_cast<const float4 *>(p);
-  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-__device__ __forceinline__ void st4f(float *p, const float (&v)[4]) {
-  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-
 // Operand layout of the tensor-core trailing update ("split canonical"): for
 // a 128-row block B and a 16-wide chunk c of the inner dimension, the TF32
 // high parts (x with its low 13 mantissa bits cleared) and the remainders
@@ -383,98 +307,104 @@ __device__ __forceinline__ void store_split4(float *X, int row, int k, const flo
   *reinterpret_cast<float4 *>(blk + 2048 + o) = l;
 }
 
-// FP32 panel of pivot block K for block I != K (128 rows): C_I = A_IK (from
-// the stored upper triangle: A[i][K0 + s] for I < K, A[K0 + s][i] for I > K),
-// U_I = C_I P. Writes C_I and U_I in the split canonical layout of the
-// tensor-core update (rows i of block I, inner index t) and stores U_I back as
-// the new panel (A_IK for I < K, A_KI = U_I^T for I > K). 256 threads on a
-// 16 x 16 grid, each an 8 x 8 block of U accumulated in registers.
+// FP32 panel of pivot block K for 64 rows (from row I0) of a block I != K:
+// C = A_IK (from the stored upper triangle: A[i][K0 + s] for I < K,
+// A[K0 + s][i] for I > K), U = C P. Writes C and U in the split canonical
+// layout of the tensor-core update (rows i of block I, inner index t) and
+// stores U back as the new panel (A_IK for I < K, A_KI = U^T for I > K). 256
+// threads on a 16 x 16 grid, each 4 rows x 8 columns of U in registers. C and
+// then U pass through shared memory with the lanes along i, which keeps the
+// transposed accesses at one or two wavefronts and every global write in
+// whole 128-byte lines (lanes along t: 16 wavefronts and 16-byte pieces;
+// 35 us per 128-row block against 12 us for its two halves).
+constexpr int PANEL_ROWS = 64;
+constexpr int PANEL_SMEM = (128 * 128 + 128 * (PANEL_ROWS + 4)) * 4;
 __device__ __forceinline__ void fac_panel(int32_t kp, int32_t K0, int I0, float *__restrict__ A,
                                           const float *__restrict__ P, float *__restrict__ Ct, float *__restrict__ Ut) {
-  constexpr int NB = 128, R = NB / 16, LD = NB + 4;
-  if (I0 == K0) return;
+  constexpr int NB = 128, LD = PANEL_ROWS + 4, LDU = NB + 4;
+  if (I0 >= K0 && I0 < K0 + NB) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   float *sP = reinterpret_cast<float *>(smem_raw);  // [NB][NB]   sP[s][t]
   float *sC = sP + NB * NB;                         // [NB][LD]   sC[s][i] = C[i][s]
+  float *sU = sC;                                   // [PANEL_ROWS][LDU], over sC once it is consumed
   const bool above = I0 < K0;
-  // 4-vectors, several in flight per thread
-#pragma unroll 4
-  for (int e = 4 * threadIdx.x; e < NB * NB; e += 4 * blockDim.x) {
-    float pv[4], cv[4];
-    ld4f(P + e, pv);
-    st4f(sP + e, pv);
-    const int r = e / NB, c = e % NB;
-    if (above) {  // i = r, s = c .. c + 3
-      ld4f(A + (int64_t)(I0 + r) * kp + K0 + c, cv);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 8
+  for (int q = 0; q < 16; ++q) {
+    const int e = 4 * (q * 256 + threadIdx.x);
+    *reinterpret_cast<float4 *>(sP + e) = *reinterpret_cast<const float4 *>(P + e);
+  }
 #pragma unroll
-      for (int w = 0; w < 4; ++w) sC[(c + w) * LD + r] = cv[w];
-    } else {      // s = r, i = c .. c + 3
-      ld4f(A + (int64_t)(K0 + r) * kp + I0 + c, cv);
-      st4f(sC + r * LD + c, cv);
+  for (int q = 0; q < 8; ++q) {
+    if (above) {  // row r, inner 4 c4 .. 4 c4 + 3
+      const int r = (lane & 7) + 8 * warp, c4 = (lane >> 3) + 4 * q;
+      const float4 v = *reinterpret_cast<const float4 *>(A + (int64_t)(I0 + r) * kp + K0 + 4 * c4);
+      sC[(4 * c4 + 0) * LD + r] = v.x;
+      sC[(4 * c4 + 1) * LD + r] = v.y;
+      sC[(4 * c4 + 2) * LD + r] = v.z;
+      sC[(4 * c4 + 3) * LD + r] = v.w;
+    } else {      // inner s, rows 4 i4 .. 4 i4 + 3
+      const int e = q * 256 + threadIdx.x, i4 = e & 15, sr = e >> 4;
+      *reinterpret_cast<float4 *>(sC + sr * LD + 4 * i4) =
+          *reinterpret_cast<const float4 *>(A + (int64_t)(K0 + sr) * kp + I0 + 4 * i4);
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < NB * NB / 4; e += blockDim.x) {  // C[i][t .. t + 3], split
-    const int i = e / (NB / 4), t = (e % (NB / 4)) * 4;
+#pragma unroll 4
+  for (int q = 0; q < 8; ++q) {  // C[i][t .. t + 3], split
+    const int e = q * 256 + threadIdx.x, i = e & 63, t = (e >> 6) * 4;
     const float v[4] = {sC[t * LD + i], sC[(t + 1) * LD + i], sC[(t + 2) * LD + i], sC[(t + 3) * LD + i]};
     store_split4(Ct, I0 + i, t, v);
   }
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float u[R][R];
+  float u[4][8];  // rows 4 ty + x; columns 4 tx + y (y < 4) and 64 + 4 tx + y - 4
 #pragma unroll
-  for (int x = 0; x < R; ++x)
+  for (int x = 0; x < 4; ++x)
 #pragma unroll
-    for (int y = 0; y < R; ++y) u[x][y] = 0.0f;
+    for (int y = 0; y < 8; ++y) u[x][y] = 0.0f;
+#pragma unroll 8
+  for (int sr = 0; sr < NB; ++sr) {
+    const float4 c = *reinterpret_cast<const float4 *>(sC + sr * LD + 4 * ty);
+    const float4 p0 = *reinterpret_cast<const float4 *>(sP + sr * NB + 4 * tx);
+    const float4 p1 = *reinterpret_cast<const float4 *>(sP + sr * NB + 64 + 4 * tx);
+    const float av[4] = {c.x, c.y, c.z, c.w};
+    const float bv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) u[x][y] = fmaf(av[x], bv[y], u[x][y]);
+  }
+  __syncthreads();  // sC is consumed
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    float *o = sU + (4 * ty + x) * LDU + 4 * tx;
+    *reinterpret_cast<float4 *>(o) = make_float4(u[x][0], u[x][1], u[x][2], u[x][3]);
+    *reinterpret_cast<float4 *>(o + 64) = make_float4(u[x][4], u[x][5], u[x][6], u[x][7]);
+    if (above) {
+      float *g = A + (int64_t)(I0 + 4 * ty + x) * kp + K0 + 4 * tx;
+      *reinterpret_cast<float4 *>(g) = make_float4(u[x][0], u[x][1], u[x][2], u[x][3]);
+      *reinterpret_cast<float4 *>(g + 64) = make_float4(u[x][4], u[x][5], u[x][6], u[x][7]);
+    }
+  }
+  __syncthreads();
 #pragma unroll 4
-  for (int s = 0; s < NB; ++s) {
-    float av[R], bv[R];
+  for (int q = 0; q < 8; ++q) {  // U[i][t .. t + 3], split; transposed into A below the pivot row
+    const int e = q * 256 + threadIdx.x, i = e & 63, t = (e >> 6) * 4;
+    const float4 w = *reinterpret_cast<const float4 *>(sU + i * LDU + t);
+    const float v[4] = {w.x, w.y, w.z, w.w};
+    store_split4(Ut, I0 + i, t, v);
+    if (!above) {
 #pragma unroll
-    for (int q = 0; q < R / 4; ++q) {
-      float tmp[4];
-      ld4f(sC + s * LD + ty * R + 4 * q, tmp);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) av[4 * q + w] = tmp[w];
-      ld4f(sP + s * NB + tx * R + 4 * q, tmp);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) bv[4 * q + w] = tmp[w];
-    }
-#pragma unroll
-    for (int x = 0; x < R; ++x)
-#pragma unroll
-      for (int y = 0; y < R; ++y) u[x][y] += av[x] * bv[y];
-  }
-  // u[x][y] = U[i = ty R + x][t = tx R + y]
-  if (!above) {
-#pragma unroll
-    for (int y = 0; y < R; ++y) {
-      const int t = tx * R + y;
-#pragma unroll
-      for (int q = 0; q < R / 4; ++q) {
-        float tmp[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) tmp[w] = u[4 * q + w][y];
-        st4f(A + (int64_t)(K0 + t) * kp + I0 + ty * R + 4 * q, tmp);
-      }
-    }
-  }
-#pragma unroll
-  for (int x = 0; x < R; ++x) {
-    const int i = ty * R + x;
-#pragma unroll
-    for (int q = 0; q < R / 4; ++q) {
-      float tmp[4];
-#pragma unroll
-      for (int w = 0; w < 4; ++w) tmp[w] = u[x][4 * q + w];
-      store_split4(Ut, I0 + i, tx * R + 4 * q, tmp);
-      if (above) st4f(A + (int64_t)(I0 + i) * kp + K0 + tx * R + 4 * q, tmp);
+      for (int y = 0; y < 4; ++y) A[(int64_t)(K0 + t + y) * kp + I0 + i] = v[y];
     }
   }
 }
 
+// grid (blocks, halves)
 __global__ void __launch_bounds__(256) k_fac_panel(int32_t kp, int32_t K0, float *__restrict__ A,
                                                    const float *__restrict__ P, float *__restrict__ Ct,
                                                    float *__restrict__ Ut) {
-  fac_panel(kp, K0, (int)blockIdx.x * 128, A, P, Ct, Ut);
+  fac_panel(kp, K0, (int)blockIdx.x * 128 + (int)blockIdx.y * PANEL_ROWS, A, P, Ct, Ut);
 }
 
 // SIMT trailing update of the upper triangle (FP64, 64-blocks): block b is the
@@ -1137,10 +1067,9 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     P[q] = Ct[q] + 2 * pan;
   }
   int *err = reinterpret_cast<int *>(work + 2 * set);
-  const size_t panel_smem = sizeof(float) * (128 * 128 + 128 * (128 + 4));  // FP32
   const size_t trail_smem = 2 * sizeof(double) * 64 * 64;                    // FP64
   if constexpr (TC) {
-    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem));
+    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM));
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)tc::SMEM));
     PPRVIZ_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
@@ -1170,7 +1099,6 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     }
     if (!ctx->ev_t1) PPRVIZ_CUDA(ctx, cudaEventCreateWithFlags(&ctx->ev_t1, cudaEventDisableTiming));
     if (!ctx->ev_dp) PPRVIZ_CUDA(ctx, cudaEventCreateWithFlags(&ctx->ev_dp, cudaEventDisableTiming));
-    PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_diag128, cudaFuncAttributeMaxDynamicSharedMemorySize, DIAG128_SMEM));
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing_pp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           tcp::SMEM));
     int nsm = 0;
@@ -1180,10 +1108,10 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     ctx->test_expire_wait = false;
     PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR);
     float *Af = (float *)A;
-    k_fac_diag128<<<1, DIAG128_THREADS, DIAG128_SMEM, ctx->stream>>>(kp, 0, Af, (float *)P[0]);
+    k_fac_diag128<<<1, DIAG128_THREADS, 0, ctx->stream>>>(kp, 0, Af, (float *)P[0]);
     PPRVIZ_LAUNCHED(ctx);
     if (nblk > 1) {
-      k_fac_panel<<<nblk, 256, panel_smem, ctx->stream>>>(kp, 0, A, P[0], Ct[0], Ut[0]);
+      k_fac_panel<<<dim3(nblk, 2), 256, PANEL_SMEM, ctx->stream>>>(kp, 0, A, P[0], Ct[0], Ut[0]);
       PPRVIZ_LAUNCHED(ctx);
     }
     for (int kb = 0; nblk > 1 && kb < nblk; ++kb) {
@@ -1198,9 +1126,9 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
         PPRVIZ_LAUNCHED(ctx);
         PPRVIZ_CUDA(ctx, cudaEventRecord(ctx->ev_t1, ctx->stream));
         PPRVIZ_CUDA(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_t1, 0));
-        k_fac_diag128<<<1, DIAG128_THREADS, DIAG128_SMEM, ctx->side>>>(kp, k1 * NB, Af, (float *)P[q ^ 1]);
+        k_fac_diag128<<<1, DIAG128_THREADS, 0, ctx->side>>>(kp, k1 * NB, Af, (float *)P[q ^ 1]);
         PPRVIZ_LAUNCHED(ctx);
-        k_fac_panel<<<nblk, 256, panel_smem, ctx->side>>>(kp, k1 * NB, A, P[q ^ 1], Ct[q ^ 1], Ut[q ^ 1]);
+        k_fac_panel<<<dim3(nblk, 2), 256, PANEL_SMEM, ctx->side>>>(kp, k1 * NB, A, P[q ^ 1], Ct[q ^ 1], Ut[q ^ 1]);
         PPRVIZ_LAUNCHED(ctx);
         PPRVIZ_CUDA(ctx, cudaEventRecord(ctx->ev_dp, ctx->side));
       }
@@ -1283,7 +1211,7 @@ __global__ void __launch_bounds__(256) k_fac_panel_batch(const FacJob *__restric
                                                          const int *__restrict__ off, int nact, int32_t K0) {
   const int s = find_slot(off, nact, (int)blockIdx.x);
   const FacJob j = jobs[act[s]];
-  fac_panel(j.kp, K0, ((int)blockIdx.x - off[s]) * 128, j.A, j.P, j.Ct, j.Ut);
+  fac_panel(j.kp, K0, ((int)blockIdx.x - off[s]) * 128 + (int)blockIdx.y * PANEL_ROWS, j.A, j.P, j.Ct, j.Ut);
 }
 
 // tile t of a view's upper tile triangle, row by row: (I, J), I <= J
@@ -1366,10 +1294,7 @@ int spd_inverse_batch_f32(pprviz_ctx *ctx, int32_t nviews, const int32_t *kp, fl
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(jobs_d, jobs.data(), sizeof(FacJob) * jobs.size(), cudaMemcpyHostToDevice,
                                    ctx->stream));
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(tab_d, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, ctx->stream));
-  const size_t panel_smem = sizeof(float) * (128 * 128 + 128 * (128 + 4));
-  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem));
-  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_diag128_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        DIAG128_SMEM));
+  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM));
   PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)SMEM));
   PPRVIZ_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
@@ -1378,10 +1303,10 @@ int spd_inverse_batch_f32(pprviz_ctx *ctx, int32_t nviews, const int32_t *kp, fl
     for (int kb = 0; kb < maxnb; ++kb) {
       const StepTab &st = steps[kb];
       const int32_t K0 = kb * 128;
-      k_fac_diag128_batch<<<(unsigned)st.nall, DIAG128_THREADS, DIAG128_SMEM, ctx->stream>>>(jobs_d, tab_d + st.act_all, K0);
+      k_fac_diag128_batch<<<(unsigned)st.nall, DIAG128_THREADS, 0, ctx->stream>>>(jobs_d, tab_d + st.act_all, K0);
       PPRVIZ_LAUNCHED(ctx);
       if (st.nmulti == 0) continue;
-      k_fac_panel_batch<<<(unsigned)st.npan, 256, panel_smem, ctx->stream>>>(jobs_d, tab_d + st.act_multi,
+      k_fac_panel_batch<<<dim3((unsigned)st.npan, 2), 256, PANEL_SMEM, ctx->stream>>>(jobs_d, tab_d + st.act_multi,
                                                                               tab_d + st.pan, st.nmulti, K0);
       PPRVIZ_LAUNCHED(ctx);
       k_fac_trailing_tc_batch<<<(unsigned)st.ntrl, 256, SMEM, ctx->stream>>>(jobs_d, tab_d + st.act_multi,

@@ -62,12 +62,35 @@ __device__ __forceinline__ double rsqrt_pos(double d2) {
 // Every consumer reads the upper triangle of 128-row blocks (diagonal 128
 // blocks in full), so tiles below the diagonal 128 blocks are not written: the
 // mirrored tile above supplies their row sums as its column sums (W1 and A are
-// symmetric entry by entry), and checks the mirrored inputs.
+// symmetric entry by entry), and checks the mirrored inputs. One thread per row
+// and column adds the tile's squares (one FP64 shuffle sum per element bounded
+// the pass on the FP64 pipe): k = 10,000 (0.8 GB), 891 -> 228 us.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T recip(T d) { return T(1) / d; }
 template <>
 __device__ __forceinline__ float recip<float>(float d) { return __frcp_rn(d); }
+
+// Sum of 32 values p[0], p[stride], ...: FP64 additions, or, for floats, a float
+// sum with its exact rounding errors (TwoSum, Knuth), which is as exact and
+// stays off GB300's narrow FP64 pipe.
+__device__ __forceinline__ double sum32(const double *p, int stride) {
+  double s = 0.0;
+  for (int e = 0; e < 32; ++e) s += p[e * stride];
+  return s;
+}
+__device__ __forceinline__ double sum32(const float *p, int stride) {
+  float s = 0.0f, c = 0.0f;
+#pragma unroll
+  for (int e = 0; e < 32; ++e) {
+    const float q = p[e * stride];
+    const float t = __fadd_rn(s, q);
+    const float bb = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(q, bb)));
+    s = t;
+  }
+  return (double)s + (double)c;
+}
 
 template <typename TI, typename T>
 __global__ void k_build_sym(int32_t k, int32_t kp, const TI *__restrict__ D, T *__restrict__ W1,
@@ -76,50 +99,45 @@ __global__ void k_build_sym(int32_t k, int32_t kp, const TI *__restrict__ D, T *
   if ((by >> 2) > (bx >> 2)) return;  // below the diagonal 128 blocks
   const bool mirror = (by >> 2) < (bx >> 2);
   __shared__ TI tr[32][33];
-  __shared__ double csum[8][33];
+  __shared__ T sq[32][33];  // 1/Delta_s^2
   const int i0 = by * 32, j0 = bx * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int jj = ty; jj < 32; jj += 8) {
-    const int j = j0 + jj, i = i0 + tx;
+  TI own[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int jj = ty + 8 * e, j = j0 + jj, i = i0 + tx;
     tr[jj][tx] = (j < k && i < k) ? D[(int64_t)j * k + i] : TI(0);
+    const int io = i0 + jj, jo = j0 + tx;
+    own[e] = (io < k && jo < k) ? D[(int64_t)io * k + jo] : TI(0);
   }
   __syncthreads();
   const T invk = (T)(1.0 / (double)k);
   int bad = 0;
-  double colacc = 0.0;  // column j0 + tx over this thread's rows
-  for (int ii = ty; ii < 32; ii += 8) {
-    const int i = i0 + ii, j = j0 + tx;
-    double wsq_d = 0.0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int ii = ty + 8 * e, i = i0 + ii, j = j0 + tx;
+    T wsq = T(0);
     if (i < k && j < k && i != j) {
-      const TI a = D[(int64_t)i * k + j], b = tr[tx][ii];
+      const TI a = own[e], b = tr[tx][ii];
       // every input entry must itself be a valid distance (this element checks
       // a; b is checked by the element (j, i), or here when that tile is not built)
-      if (!(a > TI(0)) || !isfinite((double)a)) bad = 1;
-      if (mirror && (!(b > TI(0)) || !isfinite((double)b))) bad = 1;
+      if (!(a > TI(0)) || !isfinite(a)) bad = 1;
+      if (mirror && (!(b > TI(0)) || !isfinite(b))) bad = 1;
       const T d = (T)((a + b) * TI(0.5));
       const T w1 = recip(d);
-      const T wsq = w1 * w1;
+      wsq = w1 * w1;
       W1[(int64_t)i * kp + j] = w1;
       A[(int64_t)i * kp + j] = invk - wsq;
-      wsq_d = (double)wsq;
     } else {
       W1[(int64_t)i * kp + j] = T(0);
       if (i != j || i >= k) A[(int64_t)i * kp + j] = (i == j) ? T(1) : T(0);
     }
-    colacc += wsq_d;
-    for (int o = 16; o > 0; o >>= 1) wsq_d += __shfl_xor_sync(0xffffffffu, wsq_d, o);
-    if (tx == 0) rowpart[(int64_t)bx * kp + i] = wsq_d;
+    sq[ii][tx] = wsq;
   }
-  if (mirror) {  // the row sums of the tile (bx, by) below: this tile's column sums
-    csum[ty][tx] = colacc;
-    __syncthreads();
-    if (ty == 0) {
-      double c = 0.0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) c += csum[e][tx];
-      rowpart[(int64_t)by * kp + j0 + tx] = c;
-    }
-  }
+  __syncthreads();
+  if (ty == 0) rowpart[(int64_t)bx * kp + i0 + tx] = sum32(&sq[tx][0], 1);
+  // the row sums of the tile (bx, by) below: this tile's column sums
+  if (mirror && ty == 1) rowpart[(int64_t)by * kp + j0 + tx] = sum32(&sq[0][tx], 33);
   if (bad) atomicOr(flag, 1);
 }
 
