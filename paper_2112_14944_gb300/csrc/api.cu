@@ -97,6 +97,7 @@ static int stage_in(pprviz_ctx *ctx, const void *p, size_t bytes, bool device, i
 static int begin(pprviz_ctx *ctx) {
   ctx->err.clear();
   ctx->scnt_clear = false;
+  ctx->sw_invd = ctx->sw_vy = nullptr;
   ctx->launches = 0;
   memset(&ctx->stats, 0, sizeof(ctx->stats));
   PPRVIZ_CUDA(ctx, cudaSetDevice(ctx->device));
@@ -331,6 +332,9 @@ void pprviz_graph_free(pprviz_graph *g) {
   g->prp.release();
   g->pcol.release();
   g->pw.release();
+  g->pws.release();
+  g->per_vy.release();
+  g->per_u.release();
   delete g;
 }
 

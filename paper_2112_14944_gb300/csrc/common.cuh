@@ -59,6 +59,8 @@ enum Slot {
   WS_TPR, WS_TPQ, WS_TPFA, WS_TPFB, WS_TPVAL, WS_TPCNT, WS_TPMAP, WS_TPTAB,
   // Louvain+: per-node round state, scan scratch, the level pair lists, the pair table
   WS_LPNODE, WS_LPSCAN, WS_LPEDGE, WS_LPHASH,
+  // directed sweeps: per-node scale and Perron vector for the call's alpha
+  WS_DIRS,
   WS_COUNT
 };
 
@@ -85,6 +87,10 @@ struct pprviz_ctx {
   size_t ws_limit = 0;  // cap on the summed workspace capacity (0 = none); pprviz_set_workspace_limit
   bool test_expire_wait = false;  // pprviz_test_expire_wait: the next FP32 inverse withholds one copy
   bool scnt_clear = false;        // the split sweep's arrival counters are zero (set per call)
+  // directed FP32 solves (set per call by directed_prepare, propagate.cu): the
+  // sweeps' 1 / dw, and the y-scaled Perron vector of the deflated start or NULL
+  const float *sw_invd = nullptr, *sw_vy = nullptr;
+  float sw_clambda = 0.0f;  // c lambda of that vector
   pprviz_stats stats{};
   int launches = 0;  // kernels launched in the current call
   // source-group widths chosen by the sweep autotuner, by graph size class
@@ -121,6 +127,17 @@ struct pprviz_graph {
   // in-edges the entry (j, 0)), so that no gather row is empty
   bool directed = false;
   pprviz::DevBuf prp, pcol, pw;
+  // the pull weights of the FP32 sweeps: pw without the dangling nodes' own
+  // entries (the sweeps solve for those nodes directly, see directed_prepare)
+  pprviz::DevBuf pws;
+  // directed graphs, on first use (graph_perron): the dominant mode of the walk
+  // among the non-dangling nodes. vy = its left vector / dw (for a dangling
+  // node what flows into it from the left vector), u = its right vector, scaled
+  // to v u = 1, and the rate of the modes beside it (estimate + margin)
+  mutable pprviz::DevBuf per_vy, per_u;
+  mutable std::vector<float> h_u;
+  mutable double per_lambda = 0.0, per_b = 1.0;
+  mutable bool per_ok = false, per_ready = false;
 };
 
 namespace pprviz {
@@ -133,6 +150,8 @@ inline const int32_t *pull_col(const pprviz_graph *g) {
 inline const float *pull_w(const pprviz_graph *g) {
   return g->directed ? g->pw.as<float>() : (g->weighted ? g->w.as<float>() : nullptr);
 }
+// The weights of the FP32 sweeps.
+inline const float *sweep_w(const pprviz_graph *g) { return g->directed ? g->pws.as<float>() : pull_w(g); }
 inline bool pull_weighted(const pprviz_graph *g) { return g->directed || g->weighted; }
 }  // namespace pprviz
 
@@ -233,6 +252,9 @@ int louvain_plus_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, std::v
 // ---- graph analysis for the deflated sweeps (spectral.cu) ------------------
 // Fills g->comp / h_comp / h_mc / spec_b / spec_deflate once per graph.
 int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g);
+
+// Directed graphs: fills g->per_* once per graph.
+int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g);
 
 // ---- dense tensor-core sweeps (dense.cu) ----------------------------------
 // True when the graph holds enough of all pairs for a dense contraction to

@@ -180,6 +180,7 @@ int pull_csr_build(pprviz_ctx *ctx, pprviz_graph *g, const int64_t *rp, const in
   cudaError_t e = g->prp.ensure(sizeof(int64_t) * (size_t)(n + 1));
   if (e == cudaSuccess) e = g->pcol.ensure(sizeof(int32_t) * pcol.size());
   if (e == cudaSuccess) e = g->pw.ensure(sizeof(float) * pw.size());
+  if (e == cudaSuccess) e = g->pws.ensure(sizeof(float) * pw.size());
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, PPRVIZ_E_OOM, "pull CSR of the directed graph: allocation failed");
@@ -189,6 +190,15 @@ int pull_csr_build(pprviz_ctx *ctx, pprviz_graph *g, const int64_t *rp, const in
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(g->pcol.p, pcol.data(), sizeof(int32_t) * pcol.size(), cudaMemcpyHostToDevice,
                                    ctx->stream));
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(g->pw.p, pw.data(), sizeof(float) * pw.size(), cudaMemcpyHostToDevice,
+                                   ctx->stream));
+  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  // the sweeps' weights: a dangling node's own entry (the only entry of a row
+  // whose column is the row) carries none
+  for (int64_t j = 0; j < n; ++j)
+    if (extra[(size_t)j])
+      for (int64_t q = cnt[(size_t)j]; q < cnt[(size_t)j + 1]; ++q)
+        if (pcol[(size_t)q] == (int32_t)j) pw[(size_t)q] = 0.0f;
+  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(g->pws.p, pw.data(), sizeof(float) * pw.size(), cudaMemcpyHostToDevice,
                                    ctx->stream));
   PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   g->directed = true;

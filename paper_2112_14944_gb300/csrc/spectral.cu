@@ -148,7 +148,173 @@ __global__ void k_spec_normalise(int64_t n, const double *__restrict__ nrm2, dou
   const double s = nrm2[0];
   if (i < n && s > 0.0) v[i] *= 1.0 / sqrt(s);
 }
+
+// Directed graphs, the walk T among the nodes with out-edges (a dangling node
+// keeps its walk and feeds nobody; it counts as 0 here):
+// LEFT: out_j = sum_{i -> j} w_ij v_i / dw_i over the pull rows (the dangling
+// nodes' own entries weigh 0); at a dangling j 0, or with `keep` what flows in.
+// Right: out_i = (1 / dw_i) sum_{i -> j} w_ij v_j over the out rows. One warp per row.
+template <bool LEFT>
+__global__ void k_dir_spmv(int64_t n, const int64_t *__restrict__ orp, const int64_t *__restrict__ rp,
+                           const int32_t *__restrict__ col, const float *__restrict__ w,
+                           const double *__restrict__ invdw, const double *__restrict__ v, double *__restrict__ out,
+                           bool keep) {
+  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (j >= n) return;
+  const bool dangling = orp[j] == orp[j + 1];
+  double acc = 0.0;
+  for (int64_t p = rp[j] + lane; p < rp[j + 1]; p += 32) {
+    const int32_t i = col[p];
+    const double wi = w ? (double)w[p] : 1.0;
+    acc += LEFT ? wi * (v[i] * invdw[i]) : wi * v[i];
+  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) out[j] = (dangling && !keep) ? 0.0 : LEFT ? acc : acc * invdw[j];
+}
+
+// the starts: 1, or the hashed vector of the spectral bound, on nodes with out-edges
+__global__ void k_dir_start(int64_t n, const int64_t *__restrict__ orp, bool hashed, double *__restrict__ v) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) v[i] = orp[i] == orp[i + 1] ? 0.0 : hashed ? start_u(i) : 1.0;
+}
+
+// part[blk] = the block's strided share of sum_i a_i b_i
+__global__ void k_dir_dot(int64_t n, const double *__restrict__ a, const double *__restrict__ b,
+                          double *__restrict__ part) {
+  __shared__ double red[256];
+  double s = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    s += a[i] * b[i];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+}
+
+// z -= (zu / vu) v
+__global__ void k_dir_project(int64_t n, const double *__restrict__ zu, const double *__restrict__ vu,
+                              const double *__restrict__ v, double *__restrict__ z) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n && vu[0] > 0.0) z[i] -= zu[0] / vu[0] * v[i];
+}
+
+// vy = v / dw (non-dangling), the inflow (dangling); u scaled to v u = 1, rounded to float
+__global__ void k_dir_finish(int64_t n, const int64_t *__restrict__ orp, const double *__restrict__ invdw,
+                             const double *__restrict__ v, const double *__restrict__ flow,
+                             const double *__restrict__ u, double vu, float *__restrict__ vy, float *__restrict__ uf) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  vy[i] = (float)(orp[i] == orp[i + 1] ? flow[i] : v[i] * invdw[i]);
+  uf[i] = (float)(u[i] / vu);
+}
 }  // namespace
+
+// The dominant mode of the walk among the non-dangling nodes: left and right
+// power iterations in FP64 (normalised every 8 steps), lambda by the two-sided
+// Rayleigh quotient, then the decay of a hashed vector without that mode gives
+// the rate of the rest. An unconverged pair or a low estimate costs sweeps,
+// never exactness: the FP64 residual certificate decides, and a refinement
+// pass that gains too little falls back to the plain rate.
+int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
+  if (g->per_ready) return PPRVIZ_OK;
+  constexpr int STEPS = 40, DECAY = 8;
+  const int64_t n = g->n;
+  const unsigned nb = (unsigned)((n + 255) / 256), wb = (unsigned)((n * 32 + 255) / 256);
+  PPRVIZ_CUDA(ctx, g->per_vy.ensure(sizeof(float) * (size_t)n));
+  PPRVIZ_CUDA(ctx, g->per_u.ensure(sizeof(float) * (size_t)n));
+  PPRVIZ_TRY(ws_ensure(ctx, WS_SPEC, sizeof(double) * (size_t)(4 * n + kSpecBlocks + 8)));
+  double *v = ctx->ws[WS_SPEC].as<double>(), *u = v + n, *z = u + n, *t = z + n, *part = t + n,
+         *sc = part + kSpecBlocks;
+  const int64_t *orp = g->rp.as<int64_t>();
+  const double *invdw = g->invdw_d.as<double>();
+  auto left = [&](const double *in, double *out, bool keep) -> int {
+    PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH);
+    k_dir_spmv<true><<<wb, 256, 0, ctx->stream>>>(n, orp, g->prp.as<int64_t>(), g->pcol.as<int32_t>(),
+                                                  g->pws.as<float>(), invdw, in, out, keep);
+    PPRVIZ_LAUNCHED(ctx);
+    return PPRVIZ_OK;
+  };
+  auto right = [&](const double *in, double *out) -> int {
+    PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH);
+    k_dir_spmv<false><<<wb, 256, 0, ctx->stream>>>(n, orp, orp, g->col.as<int32_t>(),
+                                                   g->weighted ? g->w.as<float>() : nullptr, invdw, in, out, false);
+    PPRVIZ_LAUNCHED(ctx);
+    return PPRVIZ_OK;
+  };
+  auto dot = [&](const double *a, const double *b, double *out) -> int {
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_dot<<<kSpecBlocks, 256, 0, ctx->stream>>>(n, a, b, part); }
+    PPRVIZ_LAUNCHED(ctx);
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_spec_sum<<<1, 256, 0, ctx->stream>>>(kSpecBlocks, part, out); }
+    PPRVIZ_LAUNCHED(ctx);
+    return PPRVIZ_OK;
+  };
+  auto start = [&](double *out, bool hashed) -> int {
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_start<<<nb, 256, 0, ctx->stream>>>(n, orp, hashed, out); }
+    PPRVIZ_LAUNCHED(ctx);
+    return PPRVIZ_OK;
+  };
+  auto power = [&](double *x, bool is_left) -> int {
+    PPRVIZ_TRY(start(x, false));
+    for (int it = 0; it < STEPS; it += 2) {
+      PPRVIZ_TRY(is_left ? left(x, t, false) : right(x, t));
+      PPRVIZ_TRY(is_left ? left(t, x, false) : right(t, x));
+      if (it % 8 == 6) {
+        PPRVIZ_TRY(dot(x, x, sc));
+        { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_spec_normalise<<<nb, 256, 0, ctx->stream>>>(n, sc, x); }
+        PPRVIZ_LAUNCHED(ctx);
+      }
+    }
+    return PPRVIZ_OK;
+  };
+  PPRVIZ_TRY(power(v, true));
+  PPRVIZ_TRY(power(u, false));
+  PPRVIZ_TRY(dot(v, u, sc));        // v u
+  PPRVIZ_TRY(right(u, t));
+  PPRVIZ_TRY(dot(v, t, sc + 1));    // v T u
+  // the rest: DECAY steps to shed the fast modes, DECAY more are measured
+  PPRVIZ_TRY(start(z, true));
+  auto project = [&]() -> int {
+    PPRVIZ_TRY(dot(z, u, sc + 2));
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_project<<<nb, 256, 0, ctx->stream>>>(n, sc + 2, sc, v, z); }
+    PPRVIZ_LAUNCHED(ctx);
+    return PPRVIZ_OK;
+  };
+  for (int half = 0; half < 2; ++half) {
+    PPRVIZ_TRY(project());
+    for (int it = 0; it < DECAY; it += 2) {
+      PPRVIZ_TRY(left(z, t, false));
+      PPRVIZ_TRY(left(t, z, false));
+    }
+    PPRVIZ_TRY(project());
+    PPRVIZ_TRY(dot(z, z, sc + 3 + half));
+  }
+  PPRVIZ_TRY(left(v, t, true));  // what the left vector sends to the dangling nodes
+  double hs[5] = {0, 0, 0, 0, 0};
+  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(hs, sc, sizeof(hs), cudaMemcpyDeviceToHost, ctx->stream));
+  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  const double lambda = hs[0] > 0.0 ? hs[1] / hs[0] : 0.0;
+  g->per_ok = std::isfinite(lambda) && lambda > 1e-3 && lambda < 1.0 + 1e-9 && std::isfinite(hs[3]) &&
+              std::isfinite(hs[4]) && hs[3] > 0.0;
+  g->per_b = 1.0;
+  if (g->per_ok) {
+    g->per_lambda = std::min(lambda, 1.0);
+    const double b = pow(std::max(0.0, hs[4] / hs[3]), 0.5 / DECAY);
+    g->per_b = std::min(1.0, 1.05 * b + 0.02);
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_finish<<<nb, 256, 0, ctx->stream>>>(
+        n, orp, invdw, v, t, u, hs[0], g->per_vy.as<float>(), g->per_u.as<float>()); }
+    PPRVIZ_LAUNCHED(ctx);
+    g->h_u.resize((size_t)n);
+    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(g->h_u.data(), g->per_u.p, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost,
+                                     ctx->stream));
+    PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  }
+  g->per_ready = true;
+  return PPRVIZ_OK;
+}
 
 int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g) {
   if (g->spec_ready) return PPRVIZ_OK;
