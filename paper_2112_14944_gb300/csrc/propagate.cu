@@ -610,7 +610,7 @@ __device__ __forceinline__ void load4(const double *hi, const float *lo, double 
 // A group of 4 LPR < 128 columns (k_sweep_nw) has LPR lanes per row and 32 / LPR
 // rows per warp; the rows of a warp take their edges side by side.
 template <typename T, bool WEIGHTED, bool EXACT, bool BATCH, bool LEVEL, bool LO = true, int LPR = 32>
-__global__ void __launch_bounds__(kWarps * 32)
+__global__ void __launch_bounds__(kWarps * 32, 2)
 k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
            const float *__restrict__ w, const double *__restrict__ invdw, const float2 *__restrict__ dwff,
            const int32_t *__restrict__ src, const T *__restrict__ yhi, const float *__restrict__ ylo,
@@ -673,46 +673,76 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
       // every LPR edges. The residual is then formed in float-float arithmetic
       // (TwoProd by FMA, TwoSum), ~2^-48 relative to the row: GB300's FP64
       // rate is too low to spend FP64 operations per (node, source).
-      float shi[VEC], sc[VEC], slo[VEC], ah[VEC], al[VEC];
+      float shi[VEC], sc[VEC], ah[VEC], al[VEC];
 #pragma unroll
-      for (int u = 0; u < VEC; ++u) shi[u] = sc[u] = slo[u] = ah[u] = al[u] = 0.0f;
+      for (int u = 0; u < VEC; ++u) shi[u] = sc[u] = ah[u] = al[u] = 0.0f;
+      // the next chunk's indices are loaded a chunk ahead
+      int32_t nxc = lane < e - b ? col[b + lane] : 0;
+      float nxw = WEIGHTED && lane < e - b ? w[b + lane] : 0.0f;
       for (int64_t base = b; base < e; base += LPR) {
         const int cnt = (int)min((int64_t)LPR, e - base);
-        int32_t myc = lane < cnt ? col[base + lane] : 0;
-        float myw = 1.0f;
-        if (WEIGHTED) myw = lane < cnt ? w[base + lane] : 0.0f;
-        // GB neighbour rows in flight, then accumulated in edge order
-        constexpr int GB = WEIGHTED ? 4 : 8;
-        for (int t0 = 0; t0 < cnt; t0 += GB) {
+        const int32_t myc = nxc;
+        const float myw = nxw;
+        if (base + LPR + lane < e) {
+          nxc = col[base + LPR + lane];
+          if (WEIGHTED) nxw = w[base + LPR + lane];
+        }
+        // neighbour rows t0 .. t0 + GB - 1 of the chunk, all in flight, then
+        // accumulated in edge order, two columns per instruction (paired FP32);
+        // a missing edge (only in the last groups) reads zeros, which TwoSum
+        // passes through unchanged, so that no branch splits the arithmetic.
+        // n = 10,000, 512 columns: 112 -> 82 us without low parts (408 MB of
+        // neighbour rows), 123 with them (816 MB, near what L2 delivers)
+        auto edges = [&](auto gb, int t0, bool whole) {
+          constexpr int GB = decltype(gb)::value;
           float h[GB][VEC], l[GB][VEC], wv[GB];
 #pragma unroll
           for (int q = 0; q < GB; ++q) {
             const int32_t i = __shfl_sync(rmask, myc, (t0 + q) & (LPR - 1), LPR);
             wv[q] = WEIGHTED ? __shfl_sync(rmask, myw, (t0 + q) & (LPR - 1), LPR) : 1.0f;
-            if (t0 + q < cnt) {
+            if (whole || t0 + q < cnt) {
               const int64_t p = ((int64_t)i - rb) * ld + off;
               Vec<float>::load(reinterpret_cast<const float *>(yhi) + p, h[q]);
               if (LO && ylo) Vec<float>::load(ylo + p, l[q]);
+            } else if (LPR == 32) {
+#pragma unroll
+              for (int u = 0; u < VEC; ++u) h[q][u] = l[q][u] = 0.0f;
             }
           }
 #pragma unroll
           for (int q = 0; q < GB; ++q) {
-            if (t0 + q >= cnt) break;
-            const float wi = wv[q];
+            if (LPR < 32 && t0 + q >= cnt) break;
+            const float2 n1 = make_float2(-1.0f, -1.0f), w2 = make_float2(wv[q], wv[q]);
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) {
-              float a = h[q][u], pe = 0.0f;
+            for (int u = 0; u < VEC; u += 2) {
+              float2 a = make_float2(h[q][u], h[q][u + 1]), pe = make_float2(0.0f, 0.0f);
               if (WEIGHTED) {
-                a = wi * h[q][u];
-                pe = fmaf(wi, h[q][u], -a);
+                const float2 y2 = a;
+                a = __fmul2_rn(w2, y2);
+                pe = __ffma2_rn(w2, y2, __fmul2_rn(n1, a));
               }
-              const float s = shi[u] + a;
-              const float bb = s - shi[u];
-              sc[u] += ((shi[u] - (s - bb)) + (a - bb)) + pe;
-              shi[u] = s;
-              if (LO && ylo) slo[u] = fmaf(wi, l[q][u], slo[u]);
+              const float2 s0 = make_float2(shi[u], shi[u + 1]);
+              const float2 s = __fadd2_rn(s0, a);
+              const float2 bb = __ffma2_rn(n1, s0, s);                             // s - s0
+              const float2 e0 = __ffma2_rn(n1, __ffma2_rn(n1, bb, s), s0);         // s0 - (s - bb)
+              float2 er = __fadd2_rn(e0, __ffma2_rn(n1, bb, a));                   // + (a - bb)
+              if (WEIGHTED) er = __fadd2_rn(er, pe);
+              float2 c2 = __fadd2_rn(make_float2(sc[u], sc[u + 1]), er);
+              if (LO && ylo) c2 = __ffma2_rn(w2, make_float2(l[q][u], l[q][u + 1]), c2);
+              sc[u] = c2.x;
+              sc[u + 1] = c2.y;
+              shi[u] = s.x;
+              shi[u + 1] = s.y;
             }
           }
+        };
+        int t0 = 0;
+        if constexpr (LPR == 32) {
+          for (; t0 + 8 <= cnt; t0 += 8) edges(std::integral_constant<int, 8>(), t0, true);
+          for (; t0 < cnt; t0 += 2) edges(std::integral_constant<int, 2>(), t0, false);
+        } else {
+          // rows of different lengths share a warp: one loop for all of them
+          for (; t0 < cnt; t0 += 8) edges(std::integral_constant<int, 8>(), t0, false);
         }
 #pragma unroll
         for (int u = 0; u < VEC; ++u) {
@@ -732,10 +762,10 @@ k_residual(int64_t n, int64_t ld, const int64_t *__restrict__ rp, const int32_t 
 #pragma unroll
       for (int u = 0; u < VEC; ++u) {
         if (!(LO && ylo)) lrow[u] = 0.0f;
-        // S = shi + ah + al + slo (the neighbour sum), as float-float
+        // S = shi + ah + al (the neighbour sum), as float-float
         float Sh = shi[u] + ah[u];
         const float bb = Sh - shi[u];
-        float Sl = ((shi[u] - (Sh - bb)) + (ah[u] - bb)) + (al[u] + slo[u]);
+        float Sl = ((shi[u] - (Sh - bb)) + (ah[u] - bb)) + al[u];
         if (e == b) {  // no edges: the walk stays on j
           Sh = hrow[u];
           Sl = lrow[u];
