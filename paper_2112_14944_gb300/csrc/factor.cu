@@ -1055,7 +1055,7 @@ __global__ void k_fac_finish(int32_t kp, T *__restrict__ A) {
 }
 
 template <typename T>
-static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
+static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work, int *err) {
   constexpr bool TC = std::is_same<T, float>::value;  // FP32: 128-blocks, tensor-core trailing update
   constexpr int NB = TC ? 128 : 64;
   const size_t pan = (TC ? 2 : 1) * (size_t)NB * kp;         // one panel (split into high and low parts with TC)
@@ -1066,13 +1066,11 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     Ut[q] = Ct[q] + pan;
     P[q] = Ct[q] + 2 * pan;
   }
-  int *err = reinterpret_cast<int *>(work + 2 * set);
   const size_t trail_smem = 2 * sizeof(double) * 64 * 64;                    // FP64
   if constexpr (TC) {
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM));
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)tc::SMEM));
-    PPRVIZ_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   } else {
     PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_fac_trailing64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)trail_smem));
@@ -1160,18 +1158,14 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work) {
     { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_fac_finish<T, NB><<<dim3((unsigned)std::min(8, (kp + 255) / 256), (unsigned)kp), 256, 0, ctx->stream>>>(kp, A); }
     PPRVIZ_LAUNCHED(ctx);
   }
-  if constexpr (TC) {
-    int herr = 0;
-    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (herr) return set_err(ctx, PPRVIZ_E_TIMEOUT, "tensor-core trailing update: a bounded wait expired");
-  }
   return PPRVIZ_OK;
 }
 
-int spd_inverse_f32(pprviz_ctx *ctx, int32_t kp, float *A, float *work) { return spd_inverse<float>(ctx, kp, A, work); }
+int spd_inverse_f32(pprviz_ctx *ctx, int32_t kp, float *A, float *work, int *err) {
+  return spd_inverse<float>(ctx, kp, A, work, err);
+}
 int spd_inverse_f64(pprviz_ctx *ctx, int32_t kp, double *A, double *work) {
-  return spd_inverse<double>(ctx, kp, A, work);
+  return spd_inverse<double>(ctx, kp, A, work, nullptr);
 }
 
 

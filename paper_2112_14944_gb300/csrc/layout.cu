@@ -658,6 +658,185 @@ k_reduce_rows(const int2 *__restrict__ blocks, const BatchView *__restrict__ vie
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP32 updates of a view whose two matrices fit into the shared memories of
+// the GPU (2 k^2 floats: k up to about 2,000): one cooperative launch for all
+// updates. CTA c owns rows [c nr, (c + 1) nr) and keeps them, of 1/Delta_s and
+// of M, in shared memory; thread t owns the columns 4t..4t+3. Per update
+//   b_i = sum_j W_ij (x_i - x_j) / |x_i - x_j|   for the CTA's rows,
+//   grid barrier, x_i = sum_j M_ij b_j, grid barrier,
+// every row summed by its CTA alone (threads in column order, a fixed tree), so
+// there are no partial sums to reduce, and nothing but the 2 k coordinates
+// moves between CTAs. Reading both triangles doubles the arithmetic of the
+// streaming passes, which is small here; what bounds an update is the latency
+// of its two barriers and of the reads behind them. The streaming pipeline
+// spends four launches on it: k = 1,999, 21 -> 7.5 us an update;
+// k = 150, 19 -> 3.9 us. Above the limit the matrices stream from L2 or HBM
+// and the pipeline's half of the bytes counts.
+// Every barrier wait ends after a global-timer deadline: the CTA then records
+// the error and leaves, and so does every CTA that sees it.
+// ---------------------------------------------------------------------------
+namespace resident {
+constexpr int NRMAX = 16;                 // rows per CTA at most (2 NRMAX sums per thread)
+constexpr uint32_t GAVE_UP = 0x80000000u; // barrier word: a wait expired somewhere
+
+__device__ __forceinline__ uint64_t gtimer() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Grid barrier number `n` (1, 2, ...) of `ctas` CTAs on a counter that starts at
+// 0; false once a wait has expired. All threads of the CTA call it.
+__device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t n, uint32_t ctas, uint64_t limit_ns) {
+  __shared__ int ok_sh;
+  __syncthreads();  // the CTA's writes come before its arrival
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    const uint64_t t0 = gtimer();
+    for (uint32_t it = 0;; ++it) {
+      uint32_t v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v & GAVE_UP) {
+        ok = 0;
+        break;
+      }
+      if (v >= n * ctas) break;
+      if ((it & 255) == 255 && gtimer() - t0 > limit_ns) {
+        atomicOr(bar, GAVE_UP);
+        ok = 0;
+        break;
+      }
+    }
+    ok_sh = ok;
+  }
+  __syncthreads();
+  return ok_sh != 0;
+}
+
+// sums of the rows over all columns: acc[2 r], acc[2 r + 1] per thread -> out[r0 + r]
+template <int NR>
+__device__ __forceinline__ void row_sums(float (&acc)[2 * NR], float *red, int nr, float2 *out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  constexpr int REP = 32 / (2 * NR);
+  const float tot = lanes_transpose_sum<2 * NR, float>(acc, lane);
+  if (lane % REP == 0) red[warp * 2 * NR + lane / REP] = tot;
+  __syncthreads();
+  if ((int)threadIdx.x < 2 * nr) {
+    float s = red[threadIdx.x];
+    for (int w = 1; w < warps; ++w) s += red[w * 2 * NR + threadIdx.x];
+    __stcg(reinterpret_cast<float *>(out) + threadIdx.x, s);
+  }
+}
+}  // namespace resident
+
+// kq: columns rounded up to 4 (a row's stride in shared memory); blockDim.x >= kq / 4
+template <int NR>
+__global__ void __launch_bounds__(512, 1)
+k_layout_resident(int32_t k, int32_t kp, int32_t kq, int nrows, int iters, const float *__restrict__ W1,
+                  const float *__restrict__ M, float2 *X, float2 *B, uint32_t *bar, int *__restrict__ err,
+                  uint64_t limit_ns) {
+  using namespace resident;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  float *sW = reinterpret_cast<float *>(smem_raw);  // [nrows][kq]
+  float *sM = sW + (size_t)nrows * kq;              // [nrows][kq]
+  float *red = sM + (size_t)nrows * kq;             // [warps][2 NR]
+  __shared__ float2 sx[NR];
+  const int r0 = (int)blockIdx.x * nrows, nr = min(nrows, k - r0);
+  // the rows, from the stored upper triangle of 128-blocks: element (r, j) is
+  // at (j, r) where j's block comes before r's
+  for (int e = threadIdx.x; e < nr * kq; e += blockDim.x) {
+    const int r = e / kq, j = e - r * kq;
+    float w = 0.0f, m = 0.0f;
+    if (j < k && (j >> 7) >= ((r0 + r) >> 7)) {
+      w = W1[(int64_t)(r0 + r) * kp + j];
+      m = M[(int64_t)(r0 + r) * kp + j];
+    }
+    sW[e] = w;
+    sM[e] = m;
+  }
+  __syncthreads();
+  const int jlow = (((r0 + nr - 1) >> 7) << 7);  // columns of earlier blocks, for some row
+  for (int e = threadIdx.x; e < nr * jlow; e += blockDim.x) {
+    const int j = e / nr, r = e - j * nr;
+    if ((j >> 7) < ((r0 + r) >> 7)) {
+      sW[r * kq + j] = W1[(int64_t)j * kp + r0 + r];
+      sM[r * kq + j] = M[(int64_t)j * kp + r0 + r];
+    }
+  }
+  const int c0 = 4 * (int)threadIdx.x;
+  const bool has = c0 < kq;  // X and B are zero up to kp >= kq, and so are the matrices' padded columns
+  uint32_t nbar = 0;
+  for (int it = 0; it < iters; ++it) {
+    float acc[2 * NR];
+    // ---- b = L^Y(X) X
+    float4 v01 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), v23 = v01;
+    if (has) {
+      v01 = __ldcg(reinterpret_cast<const float4 *>(X + c0));
+      v23 = __ldcg(reinterpret_cast<const float4 *>(X + c0) + 1);
+    }
+    if ((int)threadIdx.x < nr) sx[threadIdx.x] = __ldcg(X + r0 + threadIdx.x);
+    __syncthreads();
+    {
+      const float2 xA = make_float2(-v01.x, -v01.z), yA = make_float2(-v01.y, -v01.w);
+      const float2 xB = make_float2(-v23.x, -v23.z), yB = make_float2(-v23.y, -v23.w);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        acc[2 * r] = acc[2 * r + 1] = 0.0f;
+        if (r < nr && has) {
+          const float4 m4 = *reinterpret_cast<const float4 *>(sW + r * kq + c0);
+          const float2 vi = sx[r];
+          const float2 vx = make_float2(vi.x, vi.x), vy = make_float2(vi.y, vi.y);
+          const float2 dxA = __fadd2_rn(vx, xA), dyA = __fadd2_rn(vy, yA);
+          const float2 dxB = __fadd2_rn(vx, xB), dyB = __fadd2_rn(vy, yB);
+          const float2 qA = __ffma2_rn(dyA, dyA, __fmul2_rn(dxA, dxA));
+          const float2 qB = __ffma2_rn(dyB, dyB, __fmul2_rn(dxB, dxB));
+          const float2 kA = __fmul2_rn(make_float2(m4.x, m4.y),
+                                       make_float2(spipe::rsqrt_clamped(qA.x), spipe::rsqrt_clamped(qA.y)));
+          const float2 kB = __fmul2_rn(make_float2(m4.z, m4.w),
+                                       make_float2(spipe::rsqrt_clamped(qB.x), spipe::rsqrt_clamped(qB.y)));
+          const float2 ra = __ffma2_rn(kB, dxB, __fmul2_rn(kA, dxA));
+          const float2 rb = __ffma2_rn(kB, dyB, __fmul2_rn(kA, dyA));
+          acc[2 * r] = ra.x + ra.y;
+          acc[2 * r + 1] = rb.x + rb.y;
+        }
+      }
+    }
+    row_sums<NR>(acc, red, nr, B + r0);
+    if (!grid_barrier(bar, ++nbar, gridDim.x, limit_ns)) break;
+    // ---- X = M b
+    if (has) {
+      v01 = __ldcg(reinterpret_cast<const float4 *>(B + c0));
+      v23 = __ldcg(reinterpret_cast<const float4 *>(B + c0) + 1);
+    }
+    {
+      const float2 xA = make_float2(v01.x, v01.z), yA = make_float2(v01.y, v01.w);
+      const float2 xB = make_float2(v23.x, v23.z), yB = make_float2(v23.y, v23.w);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        acc[2 * r] = acc[2 * r + 1] = 0.0f;
+        if (r < nr && has) {
+          const float4 m4 = *reinterpret_cast<const float4 *>(sM + r * kq + c0);
+          const float2 mA = make_float2(m4.x, m4.y), mB = make_float2(m4.z, m4.w);
+          const float2 ra = __ffma2_rn(mB, xB, __fmul2_rn(mA, xA));
+          const float2 rb = __ffma2_rn(mB, yB, __fmul2_rn(mA, yA));
+          acc[2 * r] = ra.x + ra.y;
+          acc[2 * r + 1] = rb.x + rb.y;
+        }
+      }
+    }
+    row_sums<NR>(acc, red, nr, X + r0);
+    if (!grid_barrier(bar, ++nbar, gridDim.x, limit_ns)) break;
+  }
+  // (an expired wait leaves its mark in the barrier word)
+  if (threadIdx.x == 0 && blockIdx.x == 0 && nbar > 0) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+    if (v & GAVE_UP) atomicOr(err, 1);
+  }
+}
+
 // X (kp x 2) = x0 for rows < k, zero on the padding.
 template <typename TI, typename T>
 __global__ void k_load_x(int32_t k, int32_t kp, const TI *__restrict__ x, typename T2<T>::type *__restrict__ X) {
@@ -1142,6 +1321,53 @@ int upload_maps(pprviz_ctx *ctx, const std::vector<BatchView> &bv, const float *
   return PPRVIZ_OK;
 }
 
+// All updates of one view in one cooperative launch (k_layout_resident).
+// *done = false (and nothing launched) where its rows do not fit.
+int resident_updates(pprviz_ctx *ctx, int32_t k, int32_t kp, int iters, const float *W1, const float *M, float2 *X,
+                     float2 *B, int *err, bool *done) {
+  *done = false;
+  int nsm = 0, smax = 0, coop = 0;
+  PPRVIZ_CUDA(ctx, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+  PPRVIZ_CUDA(ctx, cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+  PPRVIZ_CUDA(ctx, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device));
+  const int32_t kq = (k + 3) / 4 * 4;
+  const unsigned threads = (unsigned)((kq / 4 + 31) / 32 * 32);
+  // rows per CTA: as few as the SMs allow, but at least 4 (fewer CTAs wait on
+  // each other for less work)
+  const int nrows = std::max(4, (k + nsm - 1) / nsm);
+  const int NR = nrows <= 4 ? 4 : nrows <= 8 ? 8 : 16;
+  const size_t smem = sizeof(float) * (2 * (size_t)nrows * kq + (threads / 32) * 2 * NR);
+  const unsigned grid = (unsigned)((k + nrows - 1) / nrows);
+  if (!coop || threads > 512 || nrows > resident::NRMAX || smem + 1024 > (size_t)smax) return PPRVIZ_OK;
+  if (2 * (int64_t)iters * grid >= (int64_t)resident::GAVE_UP) return PPRVIZ_OK;  // the barrier word counts arrivals
+  PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, 64));
+  uint32_t *bar = ctx->ws[WS_BTAB].as<uint32_t>();
+  PPRVIZ_CUDA(ctx, cudaMemsetAsync(bar, 0, sizeof(uint32_t), ctx->stream));
+  const uint64_t limit_ns = 2000000000ull;  // bounded waits: 2 s
+  auto kernel = NR == 4 ? k_layout_resident<4> : NR == 8 ? k_layout_resident<8> : k_layout_resident<16>;
+  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PPRVIZ_PROF(ctx, PPRVIZ_K_LY);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, k, kp, kq, nrows, iters, W1, M, X, B, bar, err, limit_ns);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {  // not all CTAs fit at once: the pipeline takes it
+    cudaGetLastError();
+    return PPRVIZ_OK;
+  }
+  PPRVIZ_CUDA(ctx, e);
+  PPRVIZ_LAUNCHED(ctx);
+  *done = true;
+  return PPRVIZ_OK;
+}
+
 template <typename T, typename TI, typename TO>
 int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int32_t iters, TO *x_out,
                  double *stress_h) {
@@ -1161,19 +1387,18 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   T *W1 = ctx->ws[WS_W1].as<T>(), *A = ctx->ws[WS_M].as<T>();
   T *work = ctx->ws[WS_PIV].as<T>();
   V2 *X = ctx->ws[WS_X].as<V2>(), *Bv = X + kp, *Part = ctx->ws[WS_B].as<V2>();
+  PPRVIZ_CUDA(ctx, cudaMemsetAsync(Bv, 0, sizeof(V2) * (size_t)kp, ctx->stream));
   double *rowpart = ctx->ws[WS_RHS].as<double>();
   int *flag = ctx->ws[WS_FLAG].as<int>();
-  PPRVIZ_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
+  // status words, read once after the updates: [0] a bad distance, [1] an
+  // expired wait of the passes, [2] of the inverse
+  PPRVIZ_CUDA(ctx, cudaMemsetAsync(flag, 0, 3 * sizeof(int), ctx->stream));
   { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_build_sym<TI, T><<<dim3(kp / 32, kp / 32), dim3(32, 8), 0, ctx->stream>>>(k, kp, pdist, W1, A, rowpart, flag); }
   PPRVIZ_LAUNCHED(ctx);
   { PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR); k_build_diag<T><<<(unsigned)((k + 255) / 256), 256, 0, ctx->stream>>>(k, kp, rowpart, A); }
   PPRVIZ_LAUNCHED(ctx);
-  int hf = 0;
-  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  if (hf) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "pdist has a non-finite or non-positive off-diagonal entry");
   if (iters > 0) {
-    if constexpr (std::is_same<T, float>::value) PPRVIZ_TRY(spd_inverse_f32(ctx, kp, A, work));
+    if constexpr (std::is_same<T, float>::value) PPRVIZ_TRY(spd_inverse_f32(ctx, kp, A, work, flag + 2));
     else PPRVIZ_TRY(spd_inverse_f64(ctx, kp, A, work));
   }
   { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_load_x<TI, T><<<(unsigned)((kp + 255) / 256), 256, 0, ctx->stream>>>(k, kp, x0, X); }
@@ -1182,26 +1407,23 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   // row-block counters of the fused reduce, zero between passes (FP64)
   const BatchView one{0, 0, 0, kp, nbt, k, 0};
   if constexpr (std::is_same<T, float>::value) {
-    PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, sizeof(BatchView)));
-    BatchView *view_d = reinterpret_cast<BatchView *>(ctx->ws[WS_BTAB].p);
-    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(view_d, &one, sizeof(BatchView), cudaMemcpyHostToDevice, ctx->stream));
-    unsigned pgrid = 0;
-    PPRVIZ_TRY(sympass_pipe_grid(ctx, (size_t)nbt * (nbt + 1) / 2, &pgrid));
-    const std::vector<BatchView> one_v{one};
-    const CUtensorMap *maps = nullptr;
-    PPRVIZ_TRY(upload_maps(ctx, one_v, W1, A, &maps));
-    PassTables pt;
-    PPRVIZ_TRY(upload_pass_tables(ctx, one_v, pgrid, &pt));
-    PPRVIZ_TRY(ws_ensure(ctx, WS_RUNP, sizeof(V2) * ((size_t)pt.nruns * spipe::CWARPS * ST + 1)));
-    V2 *RunPart = ctx->ws[WS_RUNP].as<V2>();
     int *perr = flag + 1;
-    PPRVIZ_CUDA(ctx, cudaMemsetAsync(perr, 0, sizeof(int), ctx->stream));
-    for (int it = 0; it < iters; ++it) PPRVIZ_TRY(pass_pair(ctx, pgrid, pt, maps, view_d, X, Bv, Part, RunPart, perr));
-    if (iters > 0) {
-      int herr = 0;
-      PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&herr, perr, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-      PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-      if (herr) return set_err(ctx, PPRVIZ_E_TIMEOUT, "layout pass: tile copy wait expired");
+    bool done = false;
+    if (iters > 0) PPRVIZ_TRY(resident_updates(ctx, k, kp, iters, W1, A, X, Bv, perr, &done));
+    if (!done && iters > 0) {
+      PPRVIZ_TRY(ws_ensure(ctx, WS_BTAB, sizeof(BatchView)));
+      BatchView *view_d = reinterpret_cast<BatchView *>(ctx->ws[WS_BTAB].p);
+      PPRVIZ_CUDA(ctx, cudaMemcpyAsync(view_d, &one, sizeof(BatchView), cudaMemcpyHostToDevice, ctx->stream));
+      unsigned pgrid = 0;
+      PPRVIZ_TRY(sympass_pipe_grid(ctx, (size_t)nbt * (nbt + 1) / 2, &pgrid));
+      const std::vector<BatchView> one_v{one};
+      const CUtensorMap *maps = nullptr;
+      PPRVIZ_TRY(upload_maps(ctx, one_v, W1, A, &maps));
+      PassTables pt;
+      PPRVIZ_TRY(upload_pass_tables(ctx, one_v, pgrid, &pt));
+      PPRVIZ_TRY(ws_ensure(ctx, WS_RUNP, sizeof(V2) * ((size_t)pt.nruns * spipe::CWARPS * ST + 1)));
+      V2 *RunPart = ctx->ws[WS_RUNP].as<V2>();
+      for (int it = 0; it < iters; ++it) PPRVIZ_TRY(pass_pair(ctx, pgrid, pt, maps, view_d, X, Bv, Part, RunPart, perr));
     }
   } else {
     std::vector<int2> tiles;
@@ -1223,6 +1445,12 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
       PPRVIZ_LAUNCHED(ctx);
     }
   }
+  int hf[3] = {0, 0, 0};
+  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(hf, flag, sizeof(hf), cudaMemcpyDeviceToHost, ctx->stream));
+  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  if (hf[0]) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "pdist has a non-finite or non-positive off-diagonal entry");
+  if (hf[2]) return set_err(ctx, PPRVIZ_E_TIMEOUT, "tensor-core trailing update: a bounded wait expired");
+  if (hf[1]) return set_err(ctx, PPRVIZ_E_TIMEOUT, "layout pass: a bounded wait expired");
   V2 *Xc = ctx->ws[WS_E].as<V2>();
   { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_finish<T, TO><<<1, 1024, 0, ctx->stream>>>(k, X, x_out, Xc); }
   PPRVIZ_LAUNCHED(ctx);

@@ -1111,7 +1111,9 @@ int launch_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, bool cheb, 
   constexpr int VEC = Vec<T>::N;
   const float *invf = ctx->sw_invd && g->directed ? ctx->sw_invd : g->invdw_f.as<float>();
   if constexpr (std::is_same<T, float>::value) {
-    if (cheb && (wv ? wv->nsplit > 0 : true)) {
+    // (a graph whose longest row needs no split skips the plan)
+    const bool no_heavy = !wv && ld >= kChunk && !g->directed && g->max_row >= 0 && g->max_row <= kSegEdges;
+    if (cheb && !no_heavy && (wv ? wv->nsplit > 0 : true)) {
       // FP32 Chebyshev sweep: heavy rows split into segments
       if (!wv) PPRVIZ_TRY(sweep_plan(ctx, g));
       const int64_t nitems = wv ? wv->nitems : g->sp_nitems;

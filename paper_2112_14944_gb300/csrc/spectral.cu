@@ -26,6 +26,7 @@
 // All reductions run in a fixed order, so the estimate (and every result
 // downstream of it) is the same on every run.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 #include <cmath>
@@ -46,7 +47,8 @@ __global__ void k_cc_init(int64_t n, int32_t *__restrict__ parent) {
 }
 
 // bounded walk to the root (parent[x] <= x always, so at most x steps)
-__device__ __forceinline__ int32_t cc_root(const int32_t *parent, int32_t x) {
+template <typename P>
+__device__ __forceinline__ int32_t cc_root(P parent, int32_t x) {
   for (int it = 0; it < (1 << 20); ++it) {
     const int32_t p = parent[x];
     if (p == x) break;
@@ -147,6 +149,106 @@ __global__ void k_spec_normalise(int64_t n, const double *__restrict__ nrm2, dou
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const double s = nrm2[0];
   if (i < n && s > 0.0) v[i] *= 1.0 / sqrt(s);
+}
+
+// Sum over the CTA (1,024 threads), the same value in every thread.
+__device__ __forceinline__ double block_sum(double s, double *red) {
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  __syncthreads();  // red is free
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double t = red[threadIdx.x & 31];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// The whole analysis of a small graph (n <= kSpecSmall) by one CTA: components,
+// then the power steps, with the vectors in shared memory and 8 lanes per row.
+// The separate kernels below cost a launch per step and a host wait per
+// component round, ~345 us for a 150-node view; this one about 130 us with its read-back.
+// out: [0] <v, v>, [1] <P v, P v>, [2] 1 when the components are resolved, then
+// 1 / dw of the n nodes, then the component roots (int32).
+constexpr int64_t kSpecSmall = 1024;
+__global__ void __launch_bounds__(1024)
+k_spec_small(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ w,
+             const double *__restrict__ invdw, int32_t *__restrict__ comp, double *__restrict__ out) {
+  __shared__ int32_t parent[kSpecSmall];
+  __shared__ double va[kSpecSmall], vb[kSpecSmall], red[32];
+  const int g8 = threadIdx.x >> 3, l8 = threadIdx.x & 7;  // row group and lane in it
+  for (int i = threadIdx.x; i < n; i += 1024) parent[i] = i;
+  __syncthreads();
+  bool done = false;
+  for (int round = 0; round < kCcMaxRounds && !done; ++round) {
+    int ch = 0;
+    for (int u = g8; u < n; u += 128)
+      for (int64_t p = rp[u] + l8; p < rp[u + 1]; p += 8) {
+        const int32_t v = col[p];
+        if (v <= u) continue;
+        const int32_t ru = cc_root((volatile int32_t *)parent, u), rv = cc_root((volatile int32_t *)parent, v);
+        if (ru != rv) {
+          atomicMin(&parent[max(ru, rv)], min(ru, rv));
+          ch = 1;
+        }
+      }
+    done = __syncthreads_or(ch) == 0;
+    for (int i = threadIdx.x; i < n; i += 1024) {
+      const int32_t r = cc_root((volatile int32_t *)parent, i);
+      *(volatile int32_t *)&parent[i] = r;
+    }
+    __syncthreads();
+  }
+  int32_t *comp_out = reinterpret_cast<int32_t *>(out + 3 + n);
+  for (int i = threadIdx.x; i < n; i += 1024) {
+    comp[i] = parent[i];
+    comp_out[i] = parent[i];
+    out[3 + i] = invdw[i];
+  }
+  // dst = P src (FIRST: (P - I) u with the start vector)
+  auto step = [&](const double *src, double *dst) {
+    for (int j0 = 0; j0 < n; j0 += 128) {
+      const int j = j0 + g8;
+      double acc = 0.0;
+      int64_t b = 0, e = 0;
+      if (j < n) {
+        b = rp[j];
+        e = rp[j + 1];
+        for (int64_t p = b + l8; p < e; p += 8) {
+          const int32_t i = col[p];
+          acc += (w ? (double)w[p] : 1.0) * (src ? src[i] : start_u(i));
+        }
+      }
+      for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (j < n && l8 == 0) {
+        const double vj = src ? src[j] : start_u(j);
+        const double pv = (e == b) ? vj : acc * invdw[j];
+        dst[j] = src ? pv : pv - vj;
+      }
+    }
+    __syncthreads();
+  };
+  auto dot = [&](const double *a) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 1024) s += a[i] * a[i] / invdw[i];
+    return block_sum(s, red);
+  };
+  step(nullptr, va);
+  for (int it = 0; it < kSpecIters; ++it) {
+    step(va, vb);
+    step(vb, va);
+    if (it % 4 == 3) {
+      const double s = dot(va);
+      if (s > 0.0)
+        for (int i = threadIdx.x; i < n; i += 1024) va[i] *= 1.0 / sqrt(s);
+      __syncthreads();
+    }
+  }
+  step(va, vb);
+  const double vv = dot(va), pp = dot(vb);
+  if (threadIdx.x == 0) {
+    out[0] = vv;
+    out[1] = pp;
+    out[2] = done ? 1.0 : 0.0;
+  }
 }
 
 // Directed graphs, the walk T among the nodes with out-edges (a dangling node
@@ -330,6 +432,35 @@ int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g) {
   const float *w = g->weighted ? g->w.as<float>() : nullptr;
   const double *invdw = g->invdw_d.as<double>();
 
+  // |lambda| <= b off the stationary modes, from <v, v>_D and <P v, P v>_D
+  auto bound = [&](bool resolved, double vv, double pp) {
+    double b = 1.0;
+    if (!resolved) {
+      b = 1.0;  // components unresolved: keep the full interval and no deflation
+    } else if (vv > 0.0 && std::isfinite(vv) && std::isfinite(pp)) {
+      b = std::min(1.0, 1.05 * sqrt(std::max(0.0, pp / vv)) + 0.02);
+    } else {
+      b = 0.02;  // no non-stationary mode reached: every component is trivial
+    }
+    g->spec_b = b;
+    g->spec_deflate = resolved;
+    g->spec_ready = true;
+  };
+  if (n <= kSpecSmall) {
+    double *out = ctx->ws[WS_SPEC].as<double>();
+    { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_spec_small<<<1, 1024, 0, ctx->stream>>>((int)n, rp, col, w, invdw, parent, out); }
+    PPRVIZ_LAUNCHED(ctx);
+    std::vector<double> h((size_t)(3 + n + (n + 1) / 2));
+    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(h.data(), out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, ctx->stream));
+    PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    g->h_comp.resize((size_t)n);
+    memcpy(g->h_comp.data(), h.data() + 3 + n, sizeof(int32_t) * (size_t)n);
+    g->h_mc.assign((size_t)n, 0.0);
+    for (int64_t i = 0; i < n; ++i) g->h_mc[(size_t)g->h_comp[i]] += 1.0 / h[(size_t)(3 + i)];
+    bound(h[2] != 0.0, h[0], h[1]);
+    return PPRVIZ_OK;
+  }
+
   // ---- connected components
   { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_cc_init<<<nb, 256, 0, ctx->stream>>>(n, parent); }
   PPRVIZ_LAUNCHED(ctx);
@@ -387,17 +518,7 @@ int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g) {
   double hs[2] = {0.0, 0.0};
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(hs, scal, sizeof(hs), cudaMemcpyDeviceToHost, ctx->stream));
   PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  double b = 1.0;
-  if (!done) {
-    b = 1.0;  // components unresolved: keep the full interval and no deflation
-  } else if (hs[0] > 0.0 && std::isfinite(hs[0]) && std::isfinite(hs[1])) {
-    b = std::min(1.0, 1.05 * sqrt(std::max(0.0, hs[1] / hs[0])) + 0.02);
-  } else {
-    b = 0.02;  // no non-stationary mode reached: every component is trivial
-  }
-  g->spec_b = b;
-  g->spec_deflate = done;
-  g->spec_ready = true;
+  bound(done, hs[0], hs[1]);
   return PPRVIZ_OK;
 }
 
