@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <new>
+#include <unordered_set>
 #include <vector>
 
 #include "common.cuh"
@@ -464,11 +465,17 @@ static int leaf_sets_in(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, co
   } else {
     memcpy(li.data(), leaf_idx, sizeof(int32_t) * li.size());
   }
-  std::vector<char> seen((size_t)g->n, 0);
+  // a map over the nodes, or a hash set where the leaves are few (the map of a
+  // 2M-node graph costs more than a query's pushes)
+  const bool few = nleaf < g->n / 32;
+  std::vector<char> seen(few ? 0 : (size_t)g->n, 0);
+  std::unordered_set<int32_t> seen_few;
+  if (few) seen_few.reserve((size_t)nleaf);
   for (int32_t t : li) {
     if (t < 0 || (int64_t)t >= g->n) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "leaf id out of range");
-    if (seen[t]) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "leaf sets must be disjoint (a node is listed twice)");
-    seen[t] = 1;
+    if (few ? !seen_few.insert(t).second : seen[t] != 0)
+      return set_err(ctx, PPRVIZ_E_INVALID_ARG, "leaf sets must be disjoint (a node is listed twice)");
+    if (!few) seen[t] = 1;
   }
   *lp_d = leaf_ptr;
   *li_d = leaf_idx;
@@ -597,22 +604,10 @@ int pprviz_tau_push(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const 
   const int64_t *lp_d = nullptr;
   const int32_t *li_d = nullptr;
   PPRVIZ_TRY(leaf_sets_in(ctx, g, nsup, leaf_ptr, leaf_idx, dev, lp, li, &lp_d, &li_d));
-  // the DPR index: checked on the host (a negative or non-finite entry is an error)
-  std::vector<double> dh((size_t)g->n);
-  if (dev) {
-    PPRVIZ_CUDA(ctx, cudaMemcpyAsync(dh.data(), dpr, sizeof(double) * dh.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  } else {
-    memcpy(dh.data(), dpr, sizeof(double) * dh.size());
-  }
-  for (double x : dh)
-    if (!(x >= 0.0) || !isfinite(x)) return set_err(ctx, PPRVIZ_E_INVALID_ARG, "DPR entries must be finite and >= 0");
-  const double *dpr_d = dpr;
-  if (!dev) {
-    const void *p = nullptr;
-    PPRVIZ_TRY(stage_in(ctx, dh.data(), sizeof(double) * dh.size(), false, WS_OUT1, &p));
-    dpr_d = (const double *)p;
-  }
+  // the DPR index (its entries are checked on the device)
+  const void *dpr_p = nullptr;
+  PPRVIZ_TRY(stage_in(ctx, dpr, sizeof(double) * (size_t)g->n, dev, WS_OUT1, &dpr_p));
+  const double *dpr_d = (const double *)dpr_p;
   const size_t kk = (size_t)nsup * (size_t)nsup;
   const size_t ob = (out64 ? sizeof(double) : sizeof(float)) * kk;
   void *ld_d = nullptr;

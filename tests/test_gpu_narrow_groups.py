@@ -71,3 +71,32 @@ def test_narrow_level_groups(ctx, kind, children):
     ref = np.array([[D[np.ix_(a, b)].sum() / (len(a) * len(b)) for b in sets] for a in sets])
     miss = np.array([cert[a].mean() for a in sets])
     assert (np.abs(L - ref) <= (cl + miss)[:, None] + 1e-12 * np.abs(ref)).all()
+
+
+def test_tau_push_checks_its_inputs_on_the_device(ctx):
+    """Bad DPR entries at either end are refused for host and device arrays, -0.0 is
+    accepted, and repeated leaves are refused for few leaves and for many."""
+    import paper_2112_14944_gb300 as P
+    import torch
+    g = synth.chung_lu(901, 12, 2.2, seed=3)
+    G = ctx.upload_graph(g)
+    dpr, _ = ctx.dpr(G)
+    ptr, idx = synth.random_leaf_sets(g.n, [3, 2, 4], seed=1)
+    ok, _, _ = ctx.tau_push(G, ptr, idx, dpr)
+    zero = dpr.copy()
+    zero[-1] = -0.0 if zero[-1] == 0.0 else zero[-1]
+    assert np.allclose(ctx.tau_push(G, ptr, idx, zero)[0], ok, rtol=1e-12, atol=0)
+    for at, value in ((0, -1e-300), (g.n - 1, np.nan), (450, np.inf), (7, -np.inf)):
+        bad = dpr.copy()
+        bad[at] = value
+        with pytest.raises(P.PPRVizError):
+            ctx.tau_push(G, ptr, idx, bad)
+        out = torch.empty(3, 3, dtype=torch.float64, device="cuda")
+        dev = [torch.from_numpy(a).cuda() for a in (ptr, idx, bad)]
+        with pytest.raises(P.PPRVizError):
+            ctx.tau_push(G, *dev, ldppr_out=out, want_pdist=False)
+    for many in (False, True):
+        ptr, idx = synth.random_leaf_sets(g.n, [40, 40] if many else [2, 2], seed=2)
+        idx[-1] = idx[0]
+        with pytest.raises(P.PPRVizError):
+            ctx.tau_push(G, ptr, idx, dpr)
