@@ -27,15 +27,16 @@
 // the same FP64 residual over the CSR, restore the eps bound (each pass
 // gains what one BF16 solve resolves).
 //
-// Tiling: one CTA per 128 (target rows j) x NT (sources q) output tile, the
-// inner dimension i streamed in 32-wide chunks through two shared-memory
-// stages. Both operands are staged K-major in the canonical no-swizzle layout
-// (8-row x 16-byte core matrices): W rows are K-contiguous in memory; the state
-// Y[i][q] is source-contiguous and is transposed while staging (lanes run over
-// q, each thread packs 4 consecutive i). The global loads of chunk c + 1 are
-// issued before the MMAs of chunk c are waited on, and every mbarrier wait has
-// an iteration limit: on expiry the CTA sets the error word, skips its output
-// and still frees its tensor memory.
+// Both operands are staged K-major in the canonical no-swizzle layout (8-row x
+// 16-byte core matrices): W rows are K-contiguous in memory; the state Y[i][q]
+// is source-contiguous and is transposed while staging (lanes run over q, each
+// thread packs 4 consecutive i). The TF32 kernel (k_dsweep_ws) is
+// warp-specialized; the BF16 kernel (k_dsweep_tc) is one CTA per 128 (target
+// rows j) x NT (sources q) tile with the inner dimension i streamed in 32-wide
+// chunks through two shared-memory stages, the global loads of chunk c + 1
+// issued before the MMAs of chunk c are waited on. Every mbarrier wait is
+// bounded: on expiry the CTA sets the error word, skips its output and still
+// frees its tensor memory.
 #include <math.h>
 
 #include <algorithm>
@@ -198,20 +199,263 @@ __device__ __forceinline__ void store_chunk(const Chunk<NT> &ch, unsigned char *
 }
 }  // namespace dtc
 
-// One Chebyshev sweep of a source group on the tensor cores:
+namespace dws {
+constexpr int NT = 128;              // sources per tile
+constexpr int NST = 3;               // operand stages
+constexpr int A_B = dtc::TM * dtc::KC * 4, B_B = NT * dtc::KC * 4;  // one split part (16 KiB)
+constexpr int STAGE = 2 * A_B + 2 * B_B;
+constexpr int SMEM = NST * STAGE + 1024;
+constexpr int EPI = 8, PROD = 8;     // epilogue and staging warps
+constexpr int THREADS = (EPI + PROD + 1) * 32;
+constexpr int SEG = 16;              // chunks accumulated in tensor memory before they are drained
+constexpr uint32_t TCOLS = 512;      // two segment accumulators and the cross terms' (128 columns each)
+
+__device__ __forceinline__ uint64_t gtimer() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Bounded wait for the phase `parity` of `bar`: false once the deadline passes
+// or another role of the CTA has given up.
+__device__ __forceinline__ bool wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns, volatile int *abort_f) {
+  uint32_t done = 0;
+  uint64_t t0 = 0;
+  for (int it = 0;; ++it) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(done)
+        : "r"(dtc::smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 63) == 0) {
+      if (*abort_f) return false;
+      const uint64_t t = gtimer();
+      if (it == 0) t0 = t;
+      else if (t - t0 > limit_ns) return false;
+    }
+  }
+}
+__device__ __forceinline__ void arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(dtc::smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+      dtc::smem_u32(bar)));
+}
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(dtc::desc<false>(a)), "l"(dtc::desc<false>(b)), "r"(dtc::Cfg<NT, false>::IDESC), "r"(acc));
+}
+__device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+}  // namespace dws
+
+// One Chebyshev sweep of a source group on the tensor cores, split TF32:
 //   ACC[j][q] = sum_i W[j][i] ycur[i][q]
 //   yout[j][q] = om1 * yold[j][q] + om * (b_jq + c * ACC[j][q]) * invdw[j]
 // with b_jq = alpha [j == src[q]], or rhs[j][q] when RHS. yout may alias
 // yold (each element is read and written by the same thread).
 // W: mw x nw FP32 (mw = n rounded up to 128, nw = n rounded up to 32, zero
-// padded); the state has n rows of ld floats; grid (ld / NT, mw / 128).
-template <int NT, bool RHS, bool BF>
-__global__ void __launch_bounds__(dtc::THREADS, BF ? 2 : 1)
+// padded); the state has n rows of ld floats; grid (ld / 128, mw / 128).
+//
+// Roles: eight warps stage the 32-wide chunks (load, split, store; each warp on
+// its own, a chunk ahead in registers), one lane issues the MMAs of a chunk,
+// eight warps drain. The tensor cores add into tensor memory by truncation:
+// over n / 8 steps of positive terms that is a bias of ~n 2^-28 of the sum
+// (7e-5 at n = 6,000, and every refinement pass could gain no more than
+// 6,000x). So W_hi Y_hi is accumulated over SEG chunks only, in two alternating
+// accumulators that the drain warps add up in registers (rounded FP32 adds),
+// and the two cross terms, 2^-11 of the sum, go to an accumulator of their own.
+// Bound by shared memory (64 KiB written and 96 KiB read by the MMAs per chunk,
+// 1,250 cycles against the MMAs' 1,045): n = 6,000, 2,048 sources, 3xTF32,
+// 1.076 -> DWS_MS ms a sweep (the one-role kernel staged, synchronised and
+// multiplied in turn).
+template <bool RHS>
+__global__ void __launch_bounds__(dws::THREADS, 1)
+k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, const float *__restrict__ invdw,
+            const int32_t *__restrict__ src, const float *__restrict__ rhs, const float *__restrict__ ycur,
+            const float *yold, float *yout, float alpha, float c, float om, float om1, int *__restrict__ err,
+            uint64_t limit_ns) {
+  using namespace dws;
+  using dtc::KC;
+  using dtc::smem_u32;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full[NST], empty[NST], accf[2], acce[2], fin;
+  __shared__ uint32_t tmem_sh;
+  __shared__ int abort_sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char *sbuf = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t sb = smem_u32(sbuf);
+  volatile int *abort_f = &abort_sh;
+  const int64_t q0 = (int64_t)blockIdx.x * NT, j0 = (int64_t)blockIdx.y * dtc::TM;
+  const int nch = (int)(nw / KC), nseg = (nch + SEG - 1) / SEG;
+  if (warp == EPI + PROD) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
+                 "r"(TCOLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    auto init = [](uint64_t *b, uint32_t count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
+    };
+    for (int q = 0; q < NST; ++q) {
+      init(&full[q], PROD);
+      init(&empty[q], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      init(&accf[q], 1);
+      init(&acce[q], EPI);
+    }
+    init(&fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    abort_sh = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_sh;
+  bool ok = true;
+  if (warp >= EPI && warp < EPI + PROD) {
+    // ---- staging: each warp stores its share of every chunk
+    const int pt = tid - EPI * 32;
+    dtc::Chunk<NT> ch;
+    dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, 0, pt);
+    for (int g = 0; g < nch; ++g) {
+      const int st = g % NST;
+      if (g >= NST && !__all_sync(0xffffffffu, wait(&empty[st], (uint32_t)((g / NST - 1) & 1), limit_ns, abort_f))) {
+        ok = false;
+        break;
+      }
+      dtc::store_chunk<NT, false>(ch, sbuf + st * STAGE, pt);
+      if (g + 1 < nch) dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, (int64_t)(g + 1) * KC, pt);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) arrive(&full[st]);
+    }
+  } else if (warp == EPI + PROD) {
+    // ---- MMA issuer (one lane)
+    if (lane == 0) {
+      for (int g = 0; g < nch; ++g) {
+        const int st = g % NST, seg = g / SEG, buf = seg & 1;
+        const bool first = g % SEG == 0;
+        if (!wait(&full[st], (uint32_t)((g / NST) & 1), limit_ns, abort_f) ||
+            (first && seg >= 2 && !wait(&acce[buf], (uint32_t)(((seg >> 1) - 1) & 1), limit_ns, abort_f))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a_hi = sb + st * STAGE, a_lo = a_hi + A_B, b_hi = a_hi + 2 * A_B, b_lo = b_hi + B_B;
+        const uint32_t dseg = tmem + (uint32_t)(buf * NT), dx = tmem + 2 * NT;
+#pragma unroll
+        for (int ks = 0; ks < KC / 8; ++ks) {
+          const uint32_t o = ks * 2 * dtc::LBO;
+          mma(dseg, a_hi + o, b_hi + o, first && ks == 0 ? 0u : 1u);
+          mma(dx, a_hi + o, b_lo + o, g == 0 && ks == 0 ? 0u : 1u);
+          mma(dx, a_lo + o, b_hi + o, 1u);
+        }
+        commit(&empty[st]);
+        if (g % SEG == SEG - 1 || g == nch - 1) commit(&accf[buf]);
+      }
+      if (!ok) {
+        atomicOr(err, 1);
+        abort_sh = 1;
+      }
+      // every MMA this lane issued has completed before the tensor memory is freed
+      commit(&fin);
+      if (!wait(&fin, 0u, limit_ns, abort_f)) {
+        volatile int zero = 0;
+        (void)wait(&fin, 0u, limit_ns, &zero);
+      }
+    }
+  } else {
+    // ---- drain: warp w holds rows 32 (w % 4) + lane, columns 64 (w / 4) .. + 63
+    const int lg = warp & 3, col0 = (warp >> 2) * 64;
+    const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)col0;
+    float acc[64];
+#pragma unroll
+    for (int t = 0; t < 64; ++t) acc[t] = 0.0f;
+    for (int seg = 0; seg < nseg; ++seg) {
+      const int buf = seg & 1;
+      if (!__all_sync(0xffffffffu, wait(&accf[buf], (uint32_t)((seg >> 1) & 1), limit_ns, abort_f))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t v[16];
+        ld16(trow + (uint32_t)(buf * NT + 16 * h), v);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) acc[16 * h + t] += __uint_as_float(v[t]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) arrive(&acce[buf]);
+    }
+    if (ok) {
+      // the last segment's commit covered every MMA: the cross terms are complete
+      const int64_t j = j0 + 32 * lg + lane;
+      const bool valid = j < n;
+      const float invd = valid ? invdw[j] : 0.0f;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t v[16];
+        ld16(trow + (uint32_t)(2 * NT + 16 * h), v);
+        if (!valid) continue;
+        const int64_t q = q0 + col0 + 16 * h, off = j * ld + q;
+#pragma unroll
+        for (int t4 = 0; t4 < 4; ++t4) {
+          const float4 o = *reinterpret_cast<const float4 *>(yold + off + 4 * t4);
+          float4 bq;
+          if (RHS) {
+            bq = __ldg(reinterpret_cast<const float4 *>(rhs + off + 4 * t4));
+          } else {
+            const int4 s4 = __ldg(reinterpret_cast<const int4 *>(src + q + 4 * t4));
+            bq.x = (s4.x == (int32_t)j) ? alpha : 0.0f;
+            bq.y = (s4.y == (int32_t)j) ? alpha : 0.0f;
+            bq.z = (s4.z == (int32_t)j) ? alpha : 0.0f;
+            bq.w = (s4.w == (int32_t)j) ? alpha : 0.0f;
+          }
+          const float *a = acc + 16 * h + 4 * t4;
+          float4 r;
+          r.x = om1 * o.x + om * ((bq.x + c * (a[0] + __uint_as_float(v[4 * t4 + 0]))) * invd);
+          r.y = om1 * o.y + om * ((bq.y + c * (a[1] + __uint_as_float(v[4 * t4 + 1]))) * invd);
+          r.z = om1 * o.z + om * ((bq.z + c * (a[2] + __uint_as_float(v[4 * t4 + 2]))) * invd);
+          r.w = om1 * o.w + om * ((bq.w + c * (a[3] + __uint_as_float(v[4 * t4 + 3]))) * invd);
+          *reinterpret_cast<float4 *>(yout + off + 4 * t4) = r;
+        }
+      }
+    }
+  }
+  if (!ok && lane == 0) {
+    atomicOr(err, 1);
+    abort_sh = 1;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == EPI + PROD)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
+}
+
+// The same sweep with BF16 operands (k_dsweep_ws has the semantics of the
+// arguments); grid (ld / NT, mw / 128).
+template <int NT, bool RHS>
+__global__ void __launch_bounds__(dtc::THREADS, 2)
 k_dsweep_tc(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, const float *__restrict__ invdw,
             const int32_t *__restrict__ src, const float *__restrict__ rhs, const float *__restrict__ ycur,
             const float *yold, float *yout, float alpha, float c, float om, float om1, int *__restrict__ err) {
   using namespace dtc;
-  using C = Cfg<NT, BF>;
+  using C = Cfg<NT, true>;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_sh;
@@ -245,7 +489,7 @@ k_dsweep_tc(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
       ok = false;
       break;
     }
-    store_chunk<NT, BF>(ch, st, tid);
+    store_chunk<NT, true>(ch, st, tid);
     if (cidx + 1 < nchunks) load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, (cidx + 1) * KC, tid);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -253,35 +497,16 @@ k_dsweep_tc(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (tid == 0) {
       const uint32_t base = smem_u32(st);
-      if (BF) {
-        // one BF16 product per 16-wide inner step (32 bytes = two core matrices)
+      // one BF16 product per 16-wide inner step (32 bytes = two core matrices)
 #pragma unroll
-        for (int ks = 0; ks < KC / C::K_STEP; ++ks) {
-          const uint64_t da = desc<true>(base + ks * 2 * LBO);
-          const uint64_t db = desc<true>(base + C::A_BYTES + ks * 2 * LBO);
-          const uint32_t acc = (cidx == 0 && ks == 0) ? 0u : 1u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-              "l"(da), "l"(db), "r"(C::IDESC), "r"(acc));
-        }
-      } else {
-#pragma unroll 1
-      for (int pass = 0; pass < 3; ++pass) {
-        // hi*hi, hi*lo (W_hi Y_lo), lo*hi (W_lo Y_hi)
-        const uint32_t pa = base + (pass == 2 ? C::A_BYTES : 0);
-        const uint32_t pb = base + 2 * C::A_BYTES + (pass == 1 ? C::B_BYTES : 0);
-#pragma unroll
-        for (int ks = 0; ks < KC / C::K_STEP; ++ks) {
-          const uint64_t da = desc<false>(pa + ks * 2 * LBO);
-          const uint64_t db = desc<false>(pb + ks * 2 * LBO);
-          const uint32_t acc = (cidx == 0 && pass == 0 && ks == 0) ? 0u : 1u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-              "l"(da), "l"(db), "r"(C::IDESC), "r"(acc));
-        }
-      }
+      for (int ks = 0; ks < KC / C::K_STEP; ++ks) {
+        const uint64_t da = desc<true>(base + ks * 2 * LBO);
+        const uint64_t db = desc<true>(base + C::A_BYTES + ks * 2 * LBO);
+        const uint32_t acc = (cidx == 0 && ks == 0) ? 0u : 1u;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+            "l"(da), "l"(db), "r"(C::IDESC), "r"(acc));
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
           smem_u32(&mbar[buf])));
@@ -409,37 +634,48 @@ int dense_prepare(pprviz_ctx *ctx, const pprviz_graph *g) {
   return PPRVIZ_OK;
 }
 
-template <int NT, bool RHS, bool BF>
-static int dsweep_launch(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src,
-                         const float *rhs, const float *ycur, float *yold, double alpha, double om, int *err) {
-  using C = dtc::Cfg<NT, BF>;
-  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_dsweep_tc<NT, RHS, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        C::SMEM));
+// BF16 operands
+template <int NT, bool RHS>
+static int dsweep_bf16(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
+                       const float *ycur, float *yold, double alpha, double om, int *err) {
+  using C = dtc::Cfg<NT, true>;
+  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_dsweep_tc<NT, RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
   const int64_t mw = (g->n + 127) / 128 * 128;
   const dim3 grid((unsigned)(ld / NT), (unsigned)(mw / dtc::TM));
-  const double c = 1.0 - alpha;
   PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
-  k_dsweep_tc<NT, RHS, BF><<<grid, dtc::THREADS, C::SMEM, ctx->stream>>>(
+  k_dsweep_tc<NT, RHS><<<grid, dtc::THREADS, C::SMEM, ctx->stream>>>(
       g->n, g->dense_nw, ld, g->dense.as<float>(), g->invdw_f.as<float>(), src, rhs, ycur, yold, yold,
-      (float)alpha, (float)c, (float)om, (float)(1.0 - om), err);
+      (float)alpha, (float)(1.0 - alpha), (float)om, (float)(1.0 - om), err);
   PPRVIZ_LAUNCHED(ctx);
   return PPRVIZ_OK;
 }
 
-template <bool BF>
-static int dense_sweep_t(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
-                         const float *ycur, float *yold, double alpha, double om, int *err) {
-  if (ld % 256 == 0)
-    return rhs ? dsweep_launch<256, true, BF>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
-               : dsweep_launch<256, false, BF>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
-  return rhs ? dsweep_launch<128, true, BF>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
-             : dsweep_launch<128, false, BF>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
+// split TF32 operands
+template <bool RHS>
+static int dsweep_tf32(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
+                       const float *ycur, float *yold, double alpha, double om, int *err) {
+  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_dsweep_ws<RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, dws::SMEM));
+  const int64_t mw = (g->n + 127) / 128 * 128;
+  const dim3 grid((unsigned)(ld / dws::NT), (unsigned)(mw / dtc::TM));
+  const uint64_t limit_ns = 2000000000ull;  // bounded waits: 2 s
+  PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
+  k_dsweep_ws<RHS><<<grid, dws::THREADS, dws::SMEM, ctx->stream>>>(
+      g->n, g->dense_nw, ld, g->dense.as<float>(), g->invdw_f.as<float>(), src, rhs, ycur, yold, yold,
+      (float)alpha, (float)(1.0 - alpha), (float)om, (float)(1.0 - om), err, limit_ns);
+  PPRVIZ_LAUNCHED(ctx);
+  return PPRVIZ_OK;
 }
 
 int dense_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
                 const float *ycur, float *yold, double alpha, double om, int *err, bool bf16) {
-  return bf16 ? dense_sweep_t<true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
-              : dense_sweep_t<false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
+  if (!bf16)
+    return rhs ? dsweep_tf32<true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
+               : dsweep_tf32<false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
+  if (ld % 256 == 0)
+    return rhs ? dsweep_bf16<256, true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
+               : dsweep_bf16<256, false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
+  return rhs ? dsweep_bf16<128, true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
+             : dsweep_bf16<128, false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
 }
 
 }  // namespace pprviz
