@@ -200,15 +200,18 @@ __device__ __forceinline__ void store_chunk(const Chunk<NT> &ch, unsigned char *
 }  // namespace dtc
 
 namespace dws {
-constexpr int NT = 128;              // sources per tile
-constexpr int NST = 3;               // operand stages
-constexpr int A_B = dtc::TM * dtc::KC * 4, B_B = NT * dtc::KC * 4;  // one split part (16 KiB)
-constexpr int STAGE = 2 * A_B + 2 * B_B;
-constexpr int SMEM = NST * STAGE + 1024;
-constexpr int EPI = 8, PROD = 8;     // epilogue and staging warps
-constexpr int THREADS = (EPI + PROD + 1) * 32;
-constexpr int SEG = 16;              // chunks accumulated in tensor memory before they are drained
-constexpr uint32_t TCOLS = 512;      // two segment accumulators and the cross terms' (128 columns each)
+// NT: sources per tile (256, or 128 for a group whose width is no multiple of 256)
+template <int NT>
+struct Cfg {
+  static constexpr int NST = NT == 256 ? 2 : 3;  // operand stages
+  static constexpr int A_B = dtc::TM * dtc::KC * 4, B_B = NT * dtc::KC * 4;  // one split part
+  static constexpr int STAGE = 2 * A_B + 2 * B_B;
+  static constexpr int SMEM = NST * STAGE + 1024;
+  static constexpr uint32_t TCOLS = 2 * NT;      // the segment's accumulator and the cross terms'
+};
+constexpr int WORK = 8;                // warps that stage and drain
+constexpr int THREADS = (WORK + 1) * 32;
+constexpr int SEG = 16;                // chunks accumulated in tensor memory before they are drained
 
 __device__ __forceinline__ uint64_t gtimer() {
   uint64_t t;
@@ -243,6 +246,7 @@ __device__ __forceinline__ void commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
       dtc::smem_u32(bar)));
 }
+template <int NT>
 __device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -265,31 +269,34 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&v)[16]) {
 // with b_jq = alpha [j == src[q]], or rhs[j][q] when RHS. yout may alias
 // yold (each element is read and written by the same thread).
 // W: mw x nw FP32 (mw = n rounded up to 128, nw = n rounded up to 32, zero
-// padded); the state has n rows of ld floats; grid (ld / 128, mw / 128).
+// padded); the state has n rows of ld floats; grid (ld / NT, mw / 128).
 //
 // Roles: eight warps stage the 32-wide chunks (load, split, store; each warp on
-// its own, a chunk ahead in registers), one lane issues the MMAs of a chunk,
-// eight warps drain. The tensor cores add into tensor memory by truncation:
-// over n / 8 steps of positive terms that is a bias of ~n 2^-28 of the sum
-// (7e-5 at n = 6,000, and every refinement pass could gain no more than
-// 6,000x). So W_hi Y_hi is accumulated over SEG chunks only, in two alternating
-// accumulators that the drain warps add up in registers (rounded FP32 adds),
-// and the two cross terms, 2^-11 of the sum, go to an accumulator of their own.
-// Bound by shared memory (64 KiB written and 96 KiB read by the MMAs per chunk,
-// 1,250 cycles against the MMAs' 1,045): n = 6,000, 2,048 sources, 3xTF32,
-// 1.076 -> DWS_MS ms a sweep (the one-role kernel staged, synchronised and
-// multiplied in turn).
-template <bool RHS>
+// its own, a chunk ahead in registers), one lane of a ninth issues the MMAs.
+// The tensor cores add into tensor memory by truncation: over n / 8 steps of
+// positive terms that is a bias of ~n 2^-28 of the sum (7e-5 at n = 6,000, and
+// every refinement pass could gain no more than 6,000x). So W_hi Y_hi is
+// accumulated over SEG chunks only; the staging warps then drain it and add it
+// up in registers (rounded FP32 adds) while the next segment's first chunk is
+// already staged. The two cross terms, 2^-11 of the sum, go to an accumulator
+// of their own. Bound by the shared-memory pipe (per chunk of a 128 x 256 tile
+// 96 KiB written, 144 KiB read by the MMAs and 48 KiB of global loads; 128-wide
+// tiles ran it at 94 % for half the sources): n = 6,000, 2,048 sources, 3xTF32,
+// 1.076 ms a sweep with one role for all warps, 1.05 with 128-wide tiles and
+// separate drain warps, now 0.93 ms (with the MMAs issued by one of the eight: 1.06).
+template <int NT, bool RHS>
 __global__ void __launch_bounds__(dws::THREADS, 1)
 k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, const float *__restrict__ invdw,
             const int32_t *__restrict__ src, const float *__restrict__ rhs, const float *__restrict__ ycur,
             const float *yold, float *yout, float alpha, float c, float om, float om1, int *__restrict__ err,
             uint64_t limit_ns) {
   using namespace dws;
+  using C = dws::Cfg<NT>;
   using dtc::KC;
   using dtc::smem_u32;
+  constexpr int NST = C::NST, COLS = NT / 2;  // columns of a thread's row share
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t full[NST], empty[NST], accf[2], acce[2], fin;
+  __shared__ __align__(8) uint64_t full[NST], empty[NST], accf, acce, fin;
   __shared__ uint32_t tmem_sh;
   __shared__ int abort_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -298,9 +305,9 @@ k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
   volatile int *abort_f = &abort_sh;
   const int64_t q0 = (int64_t)blockIdx.x * NT, j0 = (int64_t)blockIdx.y * dtc::TM;
   const int nch = (int)(nw / KC), nseg = (nch + SEG - 1) / SEG;
-  if (warp == EPI + PROD) {
+  if (warp == WORK) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
-                 "r"(TCOLS));
+                 "r"(C::TCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
@@ -308,13 +315,11 @@ k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
     };
     for (int q = 0; q < NST; ++q) {
-      init(&full[q], PROD);
+      init(&full[q], WORK);
       init(&empty[q], 1);
     }
-    for (int q = 0; q < 2; ++q) {
-      init(&accf[q], 1);
-      init(&acce[q], EPI);
-    }
+    init(&accf, 1);
+    init(&acce, WORK);
     init(&fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     abort_sh = 0;
@@ -324,92 +329,57 @@ k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_sh;
   bool ok = true;
-  if (warp >= EPI && warp < EPI + PROD) {
-    // ---- staging: each warp stores its share of every chunk
-    const int pt = tid - EPI * 32;
+  if (warp < WORK) {
+    // tensor memory: warp w reads rows 32 (w % 4) + lane, columns COLS (w / 4) .. + COLS - 1
+    const int lg = warp & 3, col0 = (warp >> 2) * COLS;
+    const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)col0;
+    float acc[COLS];
+#pragma unroll
+    for (int t = 0; t < COLS; ++t) acc[t] = 0.0f;
+    // adds segment `seg` (its last MMA committed) to the sums and frees the accumulator
+    auto drain = [&](int seg) -> bool {
+      if (!__all_sync(0xffffffffu, wait(&accf, (uint32_t)(seg & 1), limit_ns, abort_f))) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int h = 0; h < COLS / 16; ++h) {
+        uint32_t v[16];
+        ld16(trow + (uint32_t)(16 * h), v);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) acc[16 * h + t] += __uint_as_float(v[t]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) arrive(&acce);
+      return true;
+    };
     dtc::Chunk<NT> ch;
-    dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, 0, pt);
+    dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, 0, tid);
     for (int g = 0; g < nch; ++g) {
       const int st = g % NST;
       if (g >= NST && !__all_sync(0xffffffffu, wait(&empty[st], (uint32_t)((g / NST - 1) & 1), limit_ns, abort_f))) {
         ok = false;
         break;
       }
-      dtc::store_chunk<NT, false>(ch, sbuf + st * STAGE, pt);
-      if (g + 1 < nch) dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, (int64_t)(g + 1) * KC, pt);
+      dtc::store_chunk<NT, false>(ch, sbuf + st * C::STAGE, tid);
+      if (g + 1 < nch) dtc::load_chunk<NT>(ch, W, nw, j0, ycur, ld, q0, n, (int64_t)(g + 1) * KC, tid);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) arrive(&full[st]);
-    }
-  } else if (warp == EPI + PROD) {
-    // ---- MMA issuer (one lane)
-    if (lane == 0) {
-      for (int g = 0; g < nch; ++g) {
-        const int st = g % NST, seg = g / SEG, buf = seg & 1;
-        const bool first = g % SEG == 0;
-        if (!wait(&full[st], (uint32_t)((g / NST) & 1), limit_ns, abort_f) ||
-            (first && seg >= 2 && !wait(&acce[buf], (uint32_t)(((seg >> 1) - 1) & 1), limit_ns, abort_f))) {
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a_hi = sb + st * STAGE, a_lo = a_hi + A_B, b_hi = a_hi + 2 * A_B, b_lo = b_hi + B_B;
-        const uint32_t dseg = tmem + (uint32_t)(buf * NT), dx = tmem + 2 * NT;
-#pragma unroll
-        for (int ks = 0; ks < KC / 8; ++ks) {
-          const uint32_t o = ks * 2 * dtc::LBO;
-          mma(dseg, a_hi + o, b_hi + o, first && ks == 0 ? 0u : 1u);
-          mma(dx, a_hi + o, b_lo + o, g == 0 && ks == 0 ? 0u : 1u);
-          mma(dx, a_lo + o, b_hi + o, 1u);
-        }
-        commit(&empty[st]);
-        if (g % SEG == SEG - 1 || g == nch - 1) commit(&accf[buf]);
-      }
-      if (!ok) {
-        atomicOr(err, 1);
-        abort_sh = 1;
-      }
-      // every MMA this lane issued has completed before the tensor memory is freed
-      commit(&fin);
-      if (!wait(&fin, 0u, limit_ns, abort_f)) {
-        volatile int zero = 0;
-        (void)wait(&fin, 0u, limit_ns, &zero);
-      }
-    }
-  } else {
-    // ---- drain: warp w holds rows 32 (w % 4) + lane, columns 64 (w / 4) .. + 63
-    const int lg = warp & 3, col0 = (warp >> 2) * 64;
-    const uint32_t trow = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)col0;
-    float acc[64];
-#pragma unroll
-    for (int t = 0; t < 64; ++t) acc[t] = 0.0f;
-    for (int seg = 0; seg < nseg; ++seg) {
-      const int buf = seg & 1;
-      if (!__all_sync(0xffffffffu, wait(&accf[buf], (uint32_t)((seg >> 1) & 1), limit_ns, abort_f))) {
+      if (g > 0 && g % SEG == 0 && !drain(g / SEG - 1)) {
         ok = false;
         break;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        uint32_t v[16];
-        ld16(trow + (uint32_t)(buf * NT + 16 * h), v);
-#pragma unroll
-        for (int t = 0; t < 16; ++t) acc[16 * h + t] += __uint_as_float(v[t]);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) arrive(&acce[buf]);
     }
+    if (ok) ok = drain(nseg - 1);
     if (ok) {
       // the last segment's commit covered every MMA: the cross terms are complete
       const int64_t j = j0 + 32 * lg + lane;
       const bool valid = j < n;
       const float invd = valid ? invdw[j] : 0.0f;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
+      for (int h = 0; h < COLS / 16; ++h) {
         uint32_t v[16];
-        ld16(trow + (uint32_t)(2 * NT + 16 * h), v);
+        ld16(trow + (uint32_t)(NT + 16 * h), v);
         if (!valid) continue;
         const int64_t q = q0 + col0 + 16 * h, off = j * ld + q;
 #pragma unroll
@@ -435,6 +405,39 @@ k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
         }
       }
     }
+  } else if (lane == 0) {
+    // ---- MMA issuer
+    for (int g = 0; g < nch; ++g) {
+      const int st = g % NST, seg = g / SEG;
+      const bool first = g % SEG == 0;
+      if (!wait(&full[st], (uint32_t)((g / NST) & 1), limit_ns, abort_f) ||
+          (first && seg >= 1 && !wait(&acce, (uint32_t)((seg - 1) & 1), limit_ns, abort_f))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t a_hi = sb + st * C::STAGE, a_lo = a_hi + C::A_B, b_hi = a_hi + 2 * C::A_B, b_lo = b_hi + C::B_B;
+      const uint32_t dx = tmem + NT;
+#pragma unroll
+      for (int ks = 0; ks < KC / 8; ++ks) {
+        const uint32_t o = ks * 2 * dtc::LBO;
+        mma<NT>(tmem, a_hi + o, b_hi + o, first && ks == 0 ? 0u : 1u);
+        mma<NT>(dx, a_hi + o, b_lo + o, g == 0 && ks == 0 ? 0u : 1u);
+        mma<NT>(dx, a_lo + o, b_hi + o, 1u);
+      }
+      commit(&empty[st]);
+      if (g % SEG == SEG - 1 || g == nch - 1) commit(&accf);
+    }
+    if (!ok) {
+      atomicOr(err, 1);
+      abort_sh = 1;
+    }
+    // every MMA this lane issued has completed before the tensor memory is freed
+    commit(&fin);
+    if (!wait(&fin, 0u, limit_ns, abort_f)) {
+      volatile int zero = 0;
+      (void)wait(&fin, 0u, limit_ns, &zero);
+    }
   }
   if (!ok && lane == 0) {
     atomicOr(err, 1);
@@ -443,8 +446,8 @@ k_dsweep_ws(int64_t n, int64_t nw, int64_t ld, const float *__restrict__ W, cons
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == EPI + PROD)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
+  if (warp == WORK)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TCOLS));
 }
 
 // The same sweep with BF16 operands (k_dsweep_ws has the semantics of the
@@ -651,15 +654,16 @@ static int dsweep_bf16(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const
 }
 
 // split TF32 operands
-template <bool RHS>
+template <int NT, bool RHS>
 static int dsweep_tf32(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
                        const float *ycur, float *yold, double alpha, double om, int *err) {
-  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_dsweep_ws<RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, dws::SMEM));
+  using C = dws::Cfg<NT>;
+  PPRVIZ_CUDA(ctx, cudaFuncSetAttribute(k_dsweep_ws<NT, RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
   const int64_t mw = (g->n + 127) / 128 * 128;
-  const dim3 grid((unsigned)(ld / dws::NT), (unsigned)(mw / dtc::TM));
+  const dim3 grid((unsigned)(ld / NT), (unsigned)(mw / dtc::TM));
   const uint64_t limit_ns = 2000000000ull;  // bounded waits: 2 s
   PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
-  k_dsweep_ws<RHS><<<grid, dws::THREADS, dws::SMEM, ctx->stream>>>(
+  k_dsweep_ws<NT, RHS><<<grid, dws::THREADS, C::SMEM, ctx->stream>>>(
       g->n, g->dense_nw, ld, g->dense.as<float>(), g->invdw_f.as<float>(), src, rhs, ycur, yold, yold,
       (float)alpha, (float)(1.0 - alpha), (float)om, (float)(1.0 - om), err, limit_ns);
   PPRVIZ_LAUNCHED(ctx);
@@ -668,9 +672,12 @@ static int dsweep_tf32(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const
 
 int dense_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const int32_t *src, const float *rhs,
                 const float *ycur, float *yold, double alpha, double om, int *err, bool bf16) {
+  if (!bf16 && ld % 256 == 0)
+    return rhs ? dsweep_tf32<256, true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
+               : dsweep_tf32<256, false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
   if (!bf16)
-    return rhs ? dsweep_tf32<true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
-               : dsweep_tf32<false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
+    return rhs ? dsweep_tf32<128, true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
+               : dsweep_tf32<128, false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
   if (ld % 256 == 0)
     return rhs ? dsweep_bf16<256, true>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err)
                : dsweep_bf16<256, false>(ctx, g, ld, src, rhs, ycur, yold, alpha, om, err);
