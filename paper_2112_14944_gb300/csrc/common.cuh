@@ -194,6 +194,31 @@ struct ProfScope {
 };
 #define PPRVIZ_PROF(ctx, cls) ::pprviz::ProfScope prof_scope__(ctx, cls)
 
+// Launch on the context stream as a programmatic dependent of the previous
+// launch (the kernel itself waits for it with griddepcontrol.wait), so that
+// its blocks are scheduled, and the pass requests its first tiles, while the
+// previous launch finishes. With dep false it is an ordinary launch.
+template <typename... P, typename... A>
+cudaError_t launch_dependent_if(pprviz_ctx *ctx, bool dep, void (*kernel)(P...), unsigned grid, unsigned block,
+                                size_t smem, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dep ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(pprviz_ctx *ctx, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                             A... args) {
+  return launch_dependent_if(ctx, true, kernel, grid, block, smem, args...);
+}
+
 // ---- graph (graph.cu) ---------------------------------------------------
 int graph_build(pprviz_ctx *ctx, pprviz_graph *g, uint32_t flags);
 // The pull CSR of a directed graph from host copies of its out-edge CSR;

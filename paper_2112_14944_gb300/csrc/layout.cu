@@ -1260,33 +1260,13 @@ int upload_pass_tables(pprviz_ctx *ctx, const std::vector<BatchView> &bv, unsign
   return PPRVIZ_OK;
 }
 
-// One layout update of all views in the tables: L^Y pass over W1 from X into
-// Bv, apply pass over M from Bv into X, each followed by its reduce.
-// Launch on the context stream as a programmatic dependent of the previous
-// launch (the kernel itself waits for it with griddepcontrol.wait), so that
-// its blocks are scheduled, and the pass requests its first tiles, while the
-// previous launch finishes.
-template <typename... P, typename... A>
-cudaError_t launch_dependent(pprviz_ctx *ctx, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
-                             A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = ctx->stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // L2 bytes of each pass matrix kept resident across updates (evict_last):
 // the two matrices together stay well inside the 126 MB L2 next to the
 // partial sums and coordinates; the rest of each matrix streams from HBM
 constexpr double kPinBytes = 32.0 * 1024 * 1024;
 
+// One layout update of all views in the tables: L^Y pass over W1 from X into
+// Bv, apply pass over M from Bv into X, each followed by its reduce.
 int pass_pair(pprviz_ctx *ctx, unsigned grid, const PassTables &pt, const CUtensorMap *maps, const BatchView *views_d,
               float2 *X, float2 *Bv, float2 *Part, float2 *RunPart, int *perr) {
   const unsigned nb = (unsigned)pt.nblocks;

@@ -100,3 +100,28 @@ def test_tau_push_checks_its_inputs_on_the_device(ctx):
         idx[-1] = idx[0]
         with pytest.raises(P.PPRVizError):
             ctx.tau_push(G, ptr, idx, dpr)
+
+
+def resident_graph(kind, n):
+    if kind == "hubs":  # rows split into segments
+        return synth.chung_lu(n, 10, 2.2, seed=1)
+    if kind == "weighted":
+        return synth.dense_clustered(n, blocks=4, density=12.0 / n, seed=2)
+    i = np.arange(n, dtype=np.int64)  # a cycle: no split
+    col = np.sort(np.stack([(i - 1) % n, (i + 1) % n], 1), axis=1).astype(np.int32)
+    return synth.Graph(n, 2 * np.arange(n + 1, dtype=np.int64), col.ravel())
+
+
+@pytest.mark.parametrize("n", [40, 129, 4863, 4864, 4865, 5003])
+@pytest.mark.parametrize("kind", ["hubs", "flat", "weighted"])
+def test_sweeps_around_one_resident_grid(ctx, kind, n):
+    """Sweeps whose blocks are all resident at once (152 x 1,024 threads: 4,864 rows of
+    one 128-wide group) are launched as dependents of the one before, larger ones plainly:
+    the FP32 and FP64 solves agree within their certificates on both sides."""
+    import paper_2112_14944_gb300 as P
+    G = ctx.upload_graph(resident_graph(kind, n))
+    view = synth.sample_view(n, min(n, 128), seed=n)
+    D, _, c32, s32 = ctx.dppr(G, view, ALPHA, 1e-8, P.FP32_CSR, out64=True)
+    R, _, c64, s64 = ctx.dppr(G, view, ALPHA, 1e-11, P.FP64, out64=True)
+    assert s32 == 0 and s64 == 0
+    assert (np.abs(D - R) <= (c32 + c64)[:, None] + 2.0 ** -40 * np.abs(R)).all()
