@@ -530,7 +530,7 @@ def run_dense(args, rank, world, local_rank):
     ach = flops / sw_all * sw_n / (sw_ms / 1e3) / 1e12  # flops of the timed launches / their time
     issued = 1 if main == "bf16" else 3
     roof = {"kernel": ("tensor-core sweep (k_dsweep_tc, BF16 x BF16 -> FP32 tcgen05.mma kind::f16)" if main == "bf16"
-                       else "tensor-core sweep (k_dsweep_tc, 3xTF32 tcgen05.mma kind::tf32)"),
+                       else "tensor-core sweep (k_dsweep_ws, 3xTF32 tcgen05.mma kind::tf32)"),
             "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
             "executed_tflops": issued * ach, "executed_frac": issued * ach / peak,
             "launches": sw_all, "timed_launches": sw_n, "avg_launch_us": 1e3 * sw_ms / max(1, sw_n),
@@ -891,7 +891,7 @@ def run_level(args, rank, world, local_rank):
     sw_ms, sw_all, sw_n = ktimes["sweep"]
     per = state["bytes_per_sweep"]
     ach = per / (sw_ms / max(1, sw_n) / 1e3) / 1e9 if sw_n else None
-    roof = {"kernel": "propagation sweep (k_sweep_sp): the [2M][128] state streams from HBM", "bound": "hbm",
+    roof = {"kernel": "propagation sweep (k_sweep_nw): the [2M][32] state streams from HBM", "bound": "hbm",
             "alg_bytes_per_launch": per,
             "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm if ach else None,
             "avg_launch_us": 1e3 * sw_ms / max(1, sw_n), "traffic": None,
@@ -1235,7 +1235,7 @@ def run_view2m(args, rank, world, local_rank):
     sw_ms, sw_all, sw_n = ktimes["sweep"]
     per = bytes_sweep / max(1, sw_all)
     ach = per / (sw_ms / max(1, sw_n) / 1e3) / 1e9 if sw_n else None
-    roof = {"kernel": "propagation sweep (k_sweep): the [2M][G] state streams from HBM", "bound": "hbm",
+    roof = {"kernel": "propagation sweep (k_sweep_nw): the [2M][G] state streams from HBM", "bound": "hbm",
             "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm if ach else None,
             "launches": sw_all, "timed_launches": sw_n, "avg_launch_us": 1e3 * sw_ms / max(1, sw_n),
             "alg_bytes_per_launch": per, "traffic": None,

@@ -181,9 +181,10 @@ int pprviz_kernel_times(pprviz_ctx *ctx, double *ms_out, int64_t *launches_out, 
  *          out-edges (dangling) keeps its walk; the library builds the
  *          in-neighbour CSR the pull-form sweeps need. Directed graphs take
  *          the CSR sweeps only (no tensor-core sweeps, no batched views);
- *          their FP32 propagation runs power sweeps with the same FP64
- *          certificate and refinement (a directed walk has a complex
- *          spectrum, outside the Chebyshev recurrence's interval). Every rule
+ *          their FP32 propagation runs power sweeps with the dominant mode
+ *          deflated and the same FP64 certificate and refinement (a directed
+ *          walk has a complex spectrum, outside the Chebyshev recurrence's
+ *          interval). Every rule
  *          above is always checked on the device before the graph is
  *          accepted.
  * Host pointers unless mem_flags has PPRVIZ_DEVICE_PTRS. The library copies
