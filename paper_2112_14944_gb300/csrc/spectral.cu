@@ -162,13 +162,13 @@ __device__ __forceinline__ double block_sum(double s, double *red) {
   return t;
 }
 
-// The whole analysis of a small graph (n <= kSpecSmall) by one CTA: components,
+// The whole analysis of a small graph (n <= kSpecSmall, few edges) by one CTA: components,
 // then the power steps, with the vectors in shared memory and 8 lanes per row.
 // The separate kernels below cost a launch per step and a host wait per
 // component round, ~345 us for a 150-node view; this one about 130 us with its read-back.
 // out: [0] <v, v>, [1] <P v, P v>, [2] 1 when the components are resolved, then
 // 1 / dw of the n nodes, then the component roots (int32).
-constexpr int64_t kSpecSmall = 1024;
+constexpr int64_t kSpecSmall = 512;
 __global__ void __launch_bounds__(1024)
 k_spec_small(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ w,
              const double *__restrict__ invdw, int32_t *__restrict__ comp, double *__restrict__ out) {
@@ -446,7 +446,11 @@ int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g) {
     g->spec_deflate = resolved;
     g->spec_ready = true;
   };
-  if (n <= kSpecSmall) {
+  // One SM's rate against launches: 150 nodes and 3,000 edges 212 us (311 by the
+  // separate kernels), 12,000 edges 282 (333); 400 nodes and 4,000 edges 296
+  // (316), 8,000 edges 367 (319); 1,000 nodes and 5,000 edges 490 (335). The
+  // line 16 n + edges = 12,000 keeps to the side where the one launch is faster.
+  if (n <= kSpecSmall && 16 * n + g->nnz <= 12000) {
     double *out = ctx->ws[WS_SPEC].as<double>();
     { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_spec_small<<<1, 1024, 0, ctx->stream>>>((int)n, rp, col, w, invdw, parent, out); }
     PPRVIZ_LAUNCHED(ctx);

@@ -125,3 +125,21 @@ def test_sweeps_around_one_resident_grid(ctx, kind, n):
     R, _, c64, s64 = ctx.dppr(G, view, ALPHA, 1e-11, P.FP64, out64=True)
     assert s32 == 0 and s64 == 0
     assert (np.abs(D - R) <= (c32 + c64)[:, None] + 2.0 ** -40 * np.abs(R)).all()
+
+
+@pytest.mark.parametrize("n", [8, 102, 103, 512, 513])
+def test_analysis_of_small_graphs_in_one_launch(ctx, n):
+    """Complete graphs on either side of 16 n + edges = 12,000 and cycles around 512
+    nodes: the deflated sweeps converge from either analysis."""
+    import paper_2112_14944_gb300 as P
+    if n < 512:
+        col = np.array([[j for j in range(n) if j != i] for i in range(n)], dtype=np.int32).ravel()
+        g = synth.Graph(n, (n - 1) * np.arange(n + 1, dtype=np.int64), col)
+    else:
+        g = resident_graph("flat", n)
+    G = ctx.upload_graph(g)
+    view = np.arange(n, dtype=np.int32)
+    D, _, c32, s32 = ctx.dppr(G, view, ALPHA, 1e-8, P.FP32_CSR, out64=True)
+    R, _, c64, s64 = ctx.dppr(G, view, ALPHA, 1e-11, P.FP64, out64=True)
+    assert s32 == 0 and s64 == 0
+    assert (np.abs(D - R) <= (c32 + c64)[:, None] + 2.0 ** -40 * np.abs(R)).all()
