@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -129,8 +130,10 @@ struct pprviz_graph {
   bool directed = false;
   pprviz::DevBuf prp, pcol, pw;
   // the pull weights of the FP32 sweeps: pw without the dangling nodes' own
-  // entries (the sweeps solve for those nodes directly, see directed_prepare)
-  pprviz::DevBuf pws;
+  // entries (the sweeps solve for those nodes directly, see directed_prepare);
+  // made on first use (directed_weights)
+  mutable pprviz::DevBuf pws;
+  mutable bool pws_ready = false;
   // directed graphs, on first use (graph_perron): the dominant mode of the walk
   // among the non-dangling nodes. vy = its left vector / dw (for a dangling
   // node what flows into it from the left vector), u = its right vector, scaled
@@ -139,6 +142,7 @@ struct pprviz_graph {
   mutable std::vector<float> h_u;
   mutable double per_lambda = 0.0, per_b = 1.0;
   mutable bool per_ok = false, per_ready = false;
+  mutable std::atomic<int64_t> per_cols{0};  // source columns solved or asked for until then
 };
 
 namespace pprviz {
@@ -221,6 +225,8 @@ cudaError_t launch_dependent(pprviz_ctx *ctx, void (*kernel)(P...), unsigned gri
 
 // ---- graph (graph.cu) ---------------------------------------------------
 int graph_build(pprviz_ctx *ctx, pprviz_graph *g, uint32_t flags);
+// Fills g->pws of a directed graph, once.
+int directed_weights(pprviz_ctx *ctx, const pprviz_graph *g);
 // The pull CSR of a directed graph from host copies of its out-edge CSR;
 // marks the graph directed.
 int pull_csr_build(pprviz_ctx *ctx, pprviz_graph *g, const int64_t *rp, const int32_t *col, const float *w);

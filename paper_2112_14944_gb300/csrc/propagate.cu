@@ -1516,13 +1516,22 @@ int chebyshev_solve(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
 // eigenvalue 1 that every such node adds: the sweeps drop the node's own entry
 // (g->pws) and scale its row by 1 / alpha. What is left of the walk has one
 // dominant mode of lambda just below 1 (the walk among the other nodes before
-// it is absorbed). With `perron` a solve starts from that mode's exact multiple,
+// it is absorbed). With the mode known a solve starts from that mode's exact multiple,
 // kappa = (b u) / (1 - c lambda) for the vectors scaled to v u = 1, and only the
 // rest (per_b) is iterated: 114 sweeps per group at rate c = 0.85 become 25 on
-// the benchmark's directed graphs.
-int directed_prepare(pprviz_ctx *ctx, const pprviz_graph *g, double alpha, bool perron) {
+// the benchmark's directed graphs. The mode is computed (once per graph) when
+// the solves of that graph have come to kPerronColumns source columns, `perron`
+// being this call's: it costs 0.75 ms for 300 nodes, 1.0 for 4,000, 2.1 for 30,000, and
+// saves per 1,000 columns 0.9 (1,000 nodes), 0.3 (4,000), 2.5 (30,000) to 3.7
+// ms (7,001 of twice the degree), so a first call for a few sources is left
+// without it (4,000 nodes, one source: 1.23 ms, 1.79 with the analysis).
+constexpr int64_t kPerronColumns = 2048;
+int directed_prepare(pprviz_ctx *ctx, const pprviz_graph *g, double alpha, int64_t perron_cols) {
   const int64_t n = g->n;
-  if (perron) PPRVIZ_TRY(graph_perron(ctx, g));
+  bool perron = perron_cols > 0;
+  PPRVIZ_TRY(directed_weights(ctx, g));
+  if (perron && !g->per_ready && g->per_cols.fetch_add(perron_cols) + perron_cols >= kPerronColumns)
+    PPRVIZ_TRY(graph_perron(ctx, g));
   perron = perron && g->per_ok;
   const size_t vec = (sizeof(float) * (size_t)n + 255) & ~(size_t)255;
   PPRVIZ_TRY(ws_ensure(ctx, WS_DIRS, 2 * vec));
@@ -1600,7 +1609,7 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
   const bool power = g->directed;
   double prate = c;  // rate of the power sweeps
   if (!fp64 && power) {
-    PPRVIZ_TRY(directed_prepare(ctx, g, alpha, true));
+    PPRVIZ_TRY(directed_prepare(ctx, g, alpha, k));
     if (ctx->sw_vy) prate = c * g->per_b;
   }
   const bool perron = ctx->sw_vy != nullptr;
@@ -1902,7 +1911,7 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
   st.source_group = (int32_t)ld;
   const double c = 1.0 - alpha;
   const bool power = g->directed;
-  if (power) PPRVIZ_TRY(directed_prepare(ctx, g, alpha, false));
+  if (power) PPRVIZ_TRY(directed_prepare(ctx, g, alpha, 0));
   auto rate = [power, c](double delta) { return power ? c : (delta > 1e-12 ? chebyshev_rate(delta) : 0.0); };
   auto sweeps_for = [](double factor, double r) { return r > 0.0 ? (int)ceil(log(0.5 * factor) / log(r)) : 1; };
   const bool exact_res = eps < 1e-9;

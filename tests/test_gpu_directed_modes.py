@@ -67,3 +67,18 @@ def test_directed_fp32_within_certificates_of_fp64(ctx, kind, alpha):
     # the same graph twice: the first call computed the modes, the second reuses them
     D2, _, c2, _ = ctx.dppr(G, view, alpha, eps, P.FP32, out64=True)
     assert np.array_equal(D, D2) and np.array_equal(cert, c2)
+
+
+@pytest.mark.parametrize("kind", ["dag", "two_classes", "star_in", "no_edges", "sparse"])
+def test_directed_solves_before_and_after_the_mode_analysis(ctx, kind):
+    """The walk's dominant mode is computed once a graph's solves have come to 2,048
+    source columns; the solves before and after agree with the FP64 path."""
+    import paper_2112_14944_gb300 as P
+    G = ctx.upload_graph(graph(kind))
+    view = np.arange(G.n, dtype=np.int32)
+    R, _, c64, s64 = ctx.dppr(G, view, 0.15, 1e-11, P.FP64, out64=True)
+    assert s64 == 0
+    for _ in range(2048 // G.n + 2):
+        D, _, cert, st = ctx.dppr(G, view, 0.15, 1e-8, P.FP32_CSR, out64=True)
+        assert st == 0
+        assert (np.abs(D - R) <= (cert + c64)[:, None] + 2.0 ** -40 * np.abs(R)).all()
