@@ -217,11 +217,12 @@ __global__ void k_renorm(int64_t count, float *__restrict__ hi, float *__restric
 // dependent of the launch before it: its blocks are in place, with their row's
 // part of the graph (which no sweep writes) read, when that launch ends, which
 // takes the drain and the launch gap off the chain of sweeps of a small view
-// (n = 150: a whole view 905 -> 819 us, a sweep now as long as its launch, 4 us). A larger grid is launched plainly (dep false): its later blocks
-// would find the wait over, but the wait still costs them the gathered rows
-// that earlier blocks left in L1 (n = 10,000, 512 columns: 44.5 us a sweep
-// against 32.4). y_cur is an ordinary pointer in the sweeps, not a restricted
-// one, so that the reads of it stay below the wait.
+// (n = 150: a whole view 905 -> 819 us, a sweep now as long as its launch, 4
+// us). A larger grid is launched plainly (dep false): its later blocks would
+// find the wait over, but the wait still costs them the gathered rows that
+// earlier blocks left in L1 (n = 10,000, 512 columns: 44.5 us a sweep against
+// 32.4). y_cur is an ordinary pointer in the sweeps, not a restricted one, so
+// that the reads of it stay below the wait.
 __device__ __forceinline__ void sweep_wait(int dep) {
   if (dep) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -229,6 +230,7 @@ __device__ __forceinline__ void sweep_wait(int dep) {
   }
 }
 // The resident blocks of the sweep kernels: at most 64 registers a thread.
+// 2,000 nodes, 200 columns (4,000 blocks): 0.43 ms a call plainly, 0.37 so.
 bool sweep_dependent(int64_t blocks, int threads) { return blocks * threads <= 152 * 1024; }
 
 // One sweep for the rows of a group.  For each node j and source column q:
@@ -1211,7 +1213,8 @@ int launch_sweep(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, bool cheb, 
   const int64_t row0 = wv ? wv->row0 : 0;
   const int32_t g0 = wv ? wv->g0 : 0;
   if (wv) src = wv->lidx;
-  const bool dep = sweep_dependent(blocks, kSweepWarps * 32);
+  // (not FP64: 300 nodes, 0.80 ms a solve plainly, 0.92 so)
+  const bool dep = std::is_same<T, float>::value && sweep_dependent(blocks, kSweepWarps * 32);
   PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
 #define PPRVIZ_SWEEP(W, C, R, B)                                                                                  \
   PPRVIZ_CUDA(ctx, launch_dependent_if(ctx, dep, k_sweep<T, W, C, R, B>, blocks, kSweepWarps * 32, 0, nrows, ld, \
