@@ -37,6 +37,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <cstring>
 
@@ -1431,6 +1432,19 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
   return TunedShape{best, best_res};
 }
 
+// The larger of two certificates; NaN once either is NaN.
+double cert_max(double a, double b) { return b <= a || a != a ? a : b; }
+
+// The largest certificate that is a number: what another refinement pass can
+// still bring down. Infinite and NaN ones (the residual left FP32's range) stay
+// as they are, and are reported as not converged at the end.
+double finite_max(const std::vector<double> &cert) {
+  double m = 0.0;
+  for (double v : cert)
+    if (std::isfinite(v)) m = std::max(m, v);
+  return m;
+}
+
 // certificates of the group's sources: d(s) * ||res_s||_1 / alpha
 // (and the signed residual sums sigma_q = sum_j res_jq, which fix the
 // stationary coefficient of the next correction)
@@ -1724,8 +1738,7 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
       PPRVIZ_TRY(read_certs(ctx, g, view_h, g0, gvalid, ld, l1, alpha, cert, sigma));
       double cprev = 0.0;
       for (int pass = 0; pass < (bf16 ? kMaxRefineBf16 : kMaxRefine); ++pass) {
-        double cmax = 0.0;
-        for (double v : cert) cmax = std::max(cmax, v);
+        const double cmax = finite_max(cert);
         if (cmax <= eps) break;
         // a pass that gained less than 10x (BF16: 2x) means modes outside the
         // estimated interval: iterate the full interval [1 - c, 1 + c] from here on
@@ -1782,8 +1795,8 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
       ylo = lo;
     }
     for (int32_t q = 0; q < gvalid; ++q) {
-      st.max_cert = std::max(st.max_cert, cert[q]);
-      if (cert[q] > eps) not_converged = true;
+      st.max_cert = cert_max(st.max_cert, cert[q]);
+      if (!(cert[q] <= eps)) not_converged = true;
       if (cert_h) cert_h[g0 + q] = cert[q];
     }
     if (dppr_d) {
@@ -1957,8 +1970,7 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
     };
     PPRVIZ_TRY(certs(hi, nullptr));
     for (int pass = 0; pass < kMaxRefine; ++pass) {
-      double cmax = 0.0;
-      for (double v : cert) cmax = std::max(cmax, v);
+      const double cmax = finite_max(cert);
       if (cmax <= eps) break;
       int K2 = sweeps_for(0.5 * eps / cmax, rate(delta_c)) + 2;
       K2 = std::min(std::max(K2, 4), power ? 4 * kMaxRefineSweeps : kMaxRefineSweeps);
@@ -1982,8 +1994,8 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
       PPRVIZ_TRY(certs(hi, lo));
     }
     for (int32_t q = 0; q < gvalid; ++q) {
-      st.max_cert = std::max(st.max_cert, cert[q]);
-      if (cert[q] > eps) not_converged = true;
+      st.max_cert = cert_max(st.max_cert, cert[q]);
+      if (!(cert[q] <= eps)) not_converged = true;
       if (cert_h) cert_h[g0 + q] = cert[q];
     }
     {
@@ -2483,7 +2495,7 @@ int dppr_views_solve(pprviz_ctx *ctx, int32_t nviews, const pprviz_graph *const 
           const int64_t gv = std::min<int64_t>(ld, views[v]->n - g0);
           for (int64_t q = 0; q < gv; ++q) {
             const double cq = views[v]->h_deg[(size_t)(g0 + q)] * l1h[(size_t)(w * 2) * ld + q] / alpha;
-            cmax = std::max(cmax, cq);
+            if (std::isfinite(cq)) cmax = std::max(cmax, cq);  // (as finite_max)
           }
         }
         return PPRVIZ_OK;
@@ -2540,8 +2552,8 @@ int dppr_views_solve(pprviz_ctx *ctx, int32_t nviews, const pprviz_graph *const 
         if (gv <= 0) continue;
         for (int64_t q = 0; q < gv; ++q) {
           const double cq = g->h_deg[(size_t)(g0 + q)] * l1h[(size_t)(w * 2) * ld + q] / alpha;
-          st.max_cert = std::max(st.max_cert, cq);
-          if (cq > eps) not_converged = true;
+          st.max_cert = cert_max(st.max_cert, cq);
+          if (!(cq <= eps)) not_converged = true;
           if (cert_h) cert_h[node_off[v] + g0 + q] = cq;
         }
         const int64_t rs = uoff[v] - wd.row0;  // first state row of the view
