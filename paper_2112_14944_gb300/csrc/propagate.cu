@@ -1435,6 +1435,12 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
 // The larger of two certificates; NaN once either is NaN.
 double cert_max(double a, double b) { return b <= a || a != a ? a : b; }
 
+double cert_worst(const std::vector<double> &cert) {
+  double m = 0.0;
+  for (double v : cert) m = cert_max(m, v);
+  return m;
+}
+
 // The largest certificate that is a number: what another refinement pass can
 // still bring down. Infinite and NaN ones (the residual left FP32's range) stay
 // as they are, and are reported as not converged at the end.
@@ -1625,10 +1631,7 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
   // instead of Chebyshev sweeps, from a start that carries the dominant mode
   const bool power = g->directed;
   double prate = c;  // rate of the power sweeps
-  if (!fp64 && power) {
-    PPRVIZ_TRY(directed_prepare(ctx, g, alpha, k));
-    if (ctx->sw_vy) prate = c * g->per_b;
-  }
+  if (!fp64 && power) PPRVIZ_TRY(directed_prepare(ctx, g, alpha, k));
   const bool perron = ctx->sw_vy != nullptr;
   const float *sigw = perron ? g->per_u.as<float>() : nullptr;
   if (!fp64 && !power) {
@@ -1710,86 +1713,107 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
         PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
                                          cudaMemcpyHostToDevice, ctx->stream));
       }
-      if (perron) {
-        for (int64_t q = 0; q < ld; ++q)
-          kappa_h[q] = q < gvalid ? alpha * g->h_u[(size_t)view_h[g0 + q]] / (1.0 - c * g->per_lambda) : 0.0;
-        PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
-                                         cudaMemcpyHostToDevice, ctx->stream));
-        prate = c * g->per_b;
-      }
-      double delta_c = power ? 0.0 : c * bsp;
-      // main solve to a Chebyshev error bound 2 rho^K <= 1e-5: every further
-      // sweep here would only save one refinement sweep, and the refinement
-      // (driven by the exact FP64 residual) finishes the job
-      // (BF16: to 2 rho^K <= 1e-3, about what BF16 products resolve)
-      const int K1 = std::max(2, sweeps_for(bf16 ? 1e-3 : 1e-5, rate(delta_c)));
-      float *hi = nullptr;
-      PPRVIZ_TRY(chebyshev_solve(ctx, g, ld, src, (int32_t)ld, nullptr, bufs[0], bufs[1], K1, alpha, tcerr,
-                                 defl ? csrc : nullptr, defl || perron ? kappa : nullptr, delta_c, &hi, nullptr, bf16));
-      st.sweeps_main += K1;
-      if (dense) st.flops_dense += 2.0 * (double)g->n * (double)g->n * gvalid * (K1 - 1);
-      else st.bytes_sweep += 12.0 * (double)g->n * gvalid * (K1 - 1);
-      // free buffers for the correction solves; the first correction becomes x_lo
-      float *fa = hi == bufs[0] ? bufs[1] : bufs[0], *fb = bufs[2], *fc = bufs[3];
-      float *lo = nullptr;
-      PPRVIZ_TRY((exact_res ? launch_residual<float, true>(ctx, g, ld, src, hi, nullptr, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)
-                            : launch_residual<float, false>(ctx, g, ld, src, hi, nullptr, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)));
-      st.residual_passes++;
-      PPRVIZ_TRY(read_certs(ctx, g, view_h, g0, gvalid, ld, l1, alpha, cert, sigma));
-      double cprev = 0.0;
-      for (int pass = 0; pass < (bf16 ? kMaxRefineBf16 : kMaxRefine); ++pass) {
-        const double cmax = finite_max(cert);
-        if (cmax <= eps) break;
-        // a pass that gained less than 10x (BF16: 2x) means modes outside the
-        // estimated interval: iterate the full interval [1 - c, 1 + c] from here on
-        // (directed: the plain power rate c)
-        if (pass > 0 && cmax > (bf16 ? 0.5 : 0.1) * cprev) {
-          if (power) prate = c;
-          else delta_c = c;
-        }
-        cprev = cmax;
-        if (perron) {
-          for (int64_t q = 0; q < gvalid; ++q) kappa_h[q] = sigma[q] / (1.0 - c * g->per_lambda);
+      float *hi = nullptr, *lo = nullptr;
+      // Directed graphs with a usable mode start from it (mode). The analysis
+      // accepts what behaves as a mode on its own tests, not on this call's
+      // sources, so each start is judged by its certificates: far above what
+      // the main solve aims for, or above eps when the passes are used up, and
+      // the group is solved once more from the plain start.
+      bool mode = perron;
+      for (;;) {
+        const bool from_mode = mode;
+        prate = mode ? c * g->per_b : c;
+        if (mode) {
+          for (int64_t q = 0; q < ld; ++q)
+            kappa_h[q] = q < gvalid ? alpha * g->h_u[(size_t)view_h[g0 + q]] / (1.0 - c * g->per_lambda) : 0.0;
           PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
                                            cudaMemcpyHostToDevice, ctx->stream));
         }
-        // correction's stationary coefficient: sum_j res_jq / alpha over m_C
-        if (defl) {
-          for (int64_t q = 0; q < gvalid; ++q) kappa_h[q] = sigma[q] / (alpha * g->h_mc[(size_t)csrc_h[q]]);
-          PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
-                                           cudaMemcpyHostToDevice, ctx->stream));
-        }
-        // sweeps for the correction: its Chebyshev error must fall by eps / (4 cmax),
-        // but an FP32 correction resolves only ~1e-7 of itself per pass, so
-        // sweeps past 2 rho^K ~ 3e-8 are left to the next pass
-        int K2 = sweeps_for(0.5 * eps / cmax, rate(delta_c)) + 2;
-        K2 = std::min(std::max(K2, 4), power ? 4 * kMaxRefineSweeps : kMaxRefineSweeps);
-        if (bf16) K2 = std::min(K2, sweeps_for(1e-3, rate(delta_c)) + 1);
-        float *delta = nullptr;
-        PPRVIZ_TRY(chebyshev_solve(ctx, g, ld, src, (int32_t)ld, rhs, fa, fb, K2, alpha, tcerr,
-                                   defl ? csrc : nullptr, defl || perron ? kappa : nullptr, delta_c, &delta, nullptr, bf16));
-        st.sweeps_refine += K2;
-        if (dense) st.flops_dense += 2.0 * (double)g->n * (double)g->n * gvalid * (K2 - 1);
-        else st.bytes_sweep += 16.0 * (double)g->n * gvalid * (K2 - 1);
-        st.refine_passes++;
-        if (!lo) {
-          lo = delta;
-          fa = (delta == fa) ? fb : fa;
-          fb = fc;
-        } else {
-          const int64_t cnt = g->n * ld;
-          { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_axpy<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(cnt, delta, lo); }
-          PPRVIZ_LAUNCHED(ctx);
-        }
-        {
-          const int64_t cnt = g->n * ld;
-          { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_renorm<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(cnt, hi, lo); }
-          PPRVIZ_LAUNCHED(ctx);
-        }
-        PPRVIZ_TRY((exact_res ? launch_residual<float, true>(ctx, g, ld, src, hi, lo, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)
-                              : launch_residual<float, false>(ctx, g, ld, src, hi, lo, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)));
+        double delta_c = power ? 0.0 : c * bsp;
+        // main solve to a Chebyshev error bound 2 rho^K <= 1e-5: every further
+        // sweep here would only save one refinement sweep, and the refinement
+        // (driven by the exact FP64 residual) finishes the job
+        // (BF16: to 2 rho^K <= 1e-3, about what BF16 products resolve)
+        const int K1 = std::max(2, sweeps_for(bf16 ? 1e-3 : 1e-5, rate(delta_c)));
+        PPRVIZ_TRY(chebyshev_solve(ctx, g, ld, src, (int32_t)ld, nullptr, bufs[0], bufs[1], K1, alpha, tcerr,
+                                   defl ? csrc : nullptr, defl || mode ? kappa : nullptr, delta_c, &hi, nullptr, bf16));
+        st.sweeps_main += K1;
+        if (dense) st.flops_dense += 2.0 * (double)g->n * (double)g->n * gvalid * (K1 - 1);
+        else st.bytes_sweep += 12.0 * (double)g->n * gvalid * (K1 - 1);
+        // free buffers for the correction solves; the first correction becomes x_lo
+        float *fa = hi == bufs[0] ? bufs[1] : bufs[0], *fb = bufs[2], *fc = bufs[3];
+        lo = nullptr;
+        PPRVIZ_TRY((exact_res ? launch_residual<float, true>(ctx, g, ld, src, hi, nullptr, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)
+                              : launch_residual<float, false>(ctx, g, ld, src, hi, nullptr, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)));
         st.residual_passes++;
         PPRVIZ_TRY(read_certs(ctx, g, view_h, g0, gvalid, ld, l1, alpha, cert, sigma));
+        // (the main solve's goal, an error of 1e-5 of the source's mass, bounds the
+        // certificate by 2e-5 d(s) / alpha)
+        if (from_mode && !(cert_worst(cert) <= std::max(eps, 1e-4 * dmax / alpha))) {
+          mode = false;
+          continue;
+        }
+        double cprev = 0.0;
+        for (int pass = 0; pass < (bf16 ? kMaxRefineBf16 : kMaxRefine); ++pass) {
+          const double cmax = finite_max(cert);
+          if (cmax <= eps) break;
+          // a pass that gained less than 10x (BF16: 2x) means modes outside the
+          // estimated interval: iterate the full interval [1 - c, 1 + c] from here on
+          // (directed: the plain start and its rate c)
+          if (pass > 0 && cmax > (bf16 ? 0.5 : 0.1) * cprev) {
+            if (power) {
+              prate = c;
+              mode = false;
+            } else {
+              delta_c = c;
+            }
+          }
+          cprev = cmax;
+          if (mode) {
+            for (int64_t q = 0; q < gvalid; ++q) kappa_h[q] = sigma[q] / (1.0 - c * g->per_lambda);
+            PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
+                                             cudaMemcpyHostToDevice, ctx->stream));
+          }
+          // correction's stationary coefficient: sum_j res_jq / alpha over m_C
+          if (defl) {
+            for (int64_t q = 0; q < gvalid; ++q) kappa_h[q] = sigma[q] / (alpha * g->h_mc[(size_t)csrc_h[q]]);
+            PPRVIZ_CUDA(ctx, cudaMemcpyAsync(kappa, kappa_h.data(), sizeof(double) * (size_t)ld,
+                                             cudaMemcpyHostToDevice, ctx->stream));
+          }
+          // sweeps for the correction: its Chebyshev error must fall by eps / (4 cmax),
+          // but an FP32 correction resolves only ~1e-7 of itself per pass, so
+          // sweeps past 2 rho^K ~ 3e-8 are left to the next pass
+          int K2 = sweeps_for(0.5 * eps / cmax, rate(delta_c)) + 2;
+          K2 = std::min(std::max(K2, 4), power ? 4 * kMaxRefineSweeps : kMaxRefineSweeps);
+          if (bf16) K2 = std::min(K2, sweeps_for(1e-3, rate(delta_c)) + 1);
+          float *delta = nullptr;
+          PPRVIZ_TRY(chebyshev_solve(ctx, g, ld, src, (int32_t)ld, rhs, fa, fb, K2, alpha, tcerr,
+                                     defl ? csrc : nullptr, defl || mode ? kappa : nullptr, delta_c, &delta, nullptr, bf16));
+          st.sweeps_refine += K2;
+          if (dense) st.flops_dense += 2.0 * (double)g->n * (double)g->n * gvalid * (K2 - 1);
+          else st.bytes_sweep += 16.0 * (double)g->n * gvalid * (K2 - 1);
+          st.refine_passes++;
+          if (!lo) {
+            lo = delta;
+            fa = (delta == fa) ? fb : fa;
+            fb = fc;
+          } else {
+            const int64_t cnt = g->n * ld;
+            { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_axpy<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(cnt, delta, lo); }
+            PPRVIZ_LAUNCHED(ctx);
+          }
+          {
+            const int64_t cnt = g->n * ld;
+            { PPRVIZ_PROF(ctx, PPRVIZ_K_OTHER); k_renorm<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(cnt, hi, lo); }
+            PPRVIZ_LAUNCHED(ctx);
+          }
+          PPRVIZ_TRY((exact_res ? launch_residual<float, true>(ctx, g, ld, src, hi, lo, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)
+                                : launch_residual<float, false>(ctx, g, ld, src, hi, lo, rhs, l1, alpha, nullptr, res_blocks, nullptr, 0, sigw)));
+          st.residual_passes++;
+          PPRVIZ_TRY(read_certs(ctx, g, view_h, g0, gvalid, ld, l1, alpha, cert, sigma));
+        }
+        if (!from_mode || cert_worst(cert) <= eps) break;
+        mode = false;
       }
       yhi = hi;
       ylo = lo;
