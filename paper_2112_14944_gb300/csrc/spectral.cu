@@ -304,6 +304,45 @@ __global__ void k_dir_project(int64_t n, const double *__restrict__ zu, const do
   if (i < n && vu[0] > 0.0) z[i] -= zu[0] / vu[0] * v[i];
 }
 
+// What graph_perron judges the pair by, per block: v v, v (v T), |v T|^2, u u,
+// u (T u), |T u|^2, sum v, max u (all vectors >= 0). One pass over the four
+// vectors instead of a dot and its sum each; the host adds the blocks in order.
+constexpr int kDirSums = 8;
+__global__ void __launch_bounds__(256)
+k_dir_quality(int64_t n, const double *__restrict__ v, const double *__restrict__ vt, const double *__restrict__ u,
+              const double *__restrict__ tu, double *__restrict__ part) {
+  __shared__ double red[8][kDirSums];
+  double s[kDirSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double a = v[i], b = vt[i], c = u[i], d = tu[i];
+    s[0] += a * a;
+    s[1] += a * b;
+    s[2] += b * b;
+    s[3] += c * c;
+    s[4] += c * d;
+    s[5] += d * d;
+    s[6] += a;
+    s[7] = c > s[7] ? c : s[7];
+  }
+#pragma unroll
+  for (int q = 0; q < kDirSums; ++q) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, s[q], o);
+      s[q] = q < 7 ? s[q] + x : (x > s[q] ? x : s[q]);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][q] = s[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < kDirSums) {
+    double t = red[0][threadIdx.x];
+    for (int w = 1; w < 8; ++w) {
+      const double x = red[w][threadIdx.x];
+      t = threadIdx.x < 7 ? t + x : (x > t ? x : t);
+    }
+    part[blockIdx.x * kDirSums + threadIdx.x] = t;
+  }
+}
+
 // vy = v / dw (non-dangling), the inflow (dangling); u scaled to v u = 1, rounded to float
 __global__ void k_dir_finish(int64_t n, const int64_t *__restrict__ orp, const double *__restrict__ invdw,
                              const double *__restrict__ v, const double *__restrict__ flow,
@@ -318,9 +357,18 @@ __global__ void k_dir_finish(int64_t n, const int64_t *__restrict__ orp, const d
 // The dominant mode of the walk among the non-dangling nodes: left and right
 // power iterations in FP64 (normalised every 8 steps), lambda by the two-sided
 // Rayleigh quotient, then the decay of a hashed vector without that mode gives
-// the rate of the rest. An unconverged pair or a low estimate costs sweeps,
-// never exactness: the FP64 residual certificate decides, and a refinement
-// pass that gains too little falls back to the plain rate.
+// the rate of the rest. The pair is used only if it is a mode:
+//  * |v T - lambda v| and |T u - lambda u| at most kModeResidual lambda |v|, |u|.
+//    Without cycles (every eigenvalue 0) the iterations leave no eigenvector:
+//    40 steps on acyclic power-law and random graphs give residuals above 1,
+//    a walk with one slow mode 1e-4 and less;
+//  * the condition |v|_1 max u / (v u) at most kModeCondition: the start is that
+//    many times the solution at most, so its FP32 rounding (2^-24 of it) stays
+//    within the main solve's 1e-5. 1 to 22 on walks with cycles, 1e24 and more
+//    without. It also bounds u / (v u), which goes to FP32, since |v|_1 >= |v|;
+//  * the rest decays: else the rate is the plain one and the start gains nothing.
+// Otherwise, as for a walk without any mode, the solves start plainly.
+constexpr double kModeResidual = 1e-3, kModeCondition = 100.0;
 int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
   if (g->per_ready) return PPRVIZ_OK;
   constexpr int STEPS = 40, DECAY = 8;
@@ -328,9 +376,9 @@ int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
   const unsigned nb = (unsigned)((n + 255) / 256), wb = (unsigned)((n * 32 + 255) / 256);
   PPRVIZ_CUDA(ctx, g->per_vy.ensure(sizeof(float) * (size_t)n));
   PPRVIZ_CUDA(ctx, g->per_u.ensure(sizeof(float) * (size_t)n));
-  PPRVIZ_TRY(ws_ensure(ctx, WS_SPEC, sizeof(double) * (size_t)(4 * n + kSpecBlocks + 8)));
+  PPRVIZ_TRY(ws_ensure(ctx, WS_SPEC, sizeof(double) * (size_t)(4 * n + (1 + kDirSums) * kSpecBlocks + 8)));
   double *v = ctx->ws[WS_SPEC].as<double>(), *u = v + n, *z = u + n, *t = z + n, *part = t + n,
-         *sc = part + kSpecBlocks;
+         *sc = part + kSpecBlocks, *qual = sc + 8;
   const int64_t *orp = g->rp.as<int64_t>();
   const double *invdw = g->invdw_d.as<double>();
   auto left = [&](const double *in, double *out, bool keep) -> int {
@@ -377,6 +425,9 @@ int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
   PPRVIZ_TRY(dot(v, u, sc));        // v u
   PPRVIZ_TRY(right(u, t));
   PPRVIZ_TRY(dot(v, t, sc + 1));    // v T u
+  PPRVIZ_TRY(left(v, z, false));
+  { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_quality<<<kSpecBlocks, 256, 0, ctx->stream>>>(n, v, z, u, t, qual); }
+  PPRVIZ_LAUNCHED(ctx);
   // the rest: DECAY steps to shed the fast modes, DECAY more are measured
   PPRVIZ_TRY(start(z, true));
   auto project = [&]() -> int {
@@ -396,16 +447,29 @@ int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
   }
   PPRVIZ_TRY(left(v, t, true));  // what the left vector sends to the dangling nodes
   double hs[5] = {0, 0, 0, 0, 0};
+  std::vector<double> hq((size_t)kSpecBlocks * kDirSums);
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(hs, sc, sizeof(hs), cudaMemcpyDeviceToHost, ctx->stream));
+  PPRVIZ_CUDA(ctx, cudaMemcpyAsync(hq.data(), qual, sizeof(double) * hq.size(), cudaMemcpyDeviceToHost, ctx->stream));
   PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  double q[kDirSums] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int b = 0; b < kSpecBlocks; ++b)
+    for (int e = 0; e < kDirSums; ++e) {
+      const double x = hq[(size_t)b * kDirSums + e];
+      q[e] = e < 7 ? q[e] + x : std::max(q[e], x);
+    }
   const double lambda = hs[0] > 0.0 ? hs[1] / hs[0] : 0.0;
-  g->per_ok = std::isfinite(lambda) && lambda > 1e-3 && lambda < 1.0 + 1e-9 && std::isfinite(hs[3]) &&
-              std::isfinite(hs[4]) && hs[3] > 0.0;
+  // (comparisons that a NaN fails)
+  auto settled = [lambda](double xx, double xy, double yy) {  // |y - lambda x| <= kModeResidual lambda |x|
+    return xx > 0.0 && yy - 2.0 * lambda * xy + lambda * lambda * xx <= kModeResidual * kModeResidual * lambda * lambda * xx;
+  };
+  const double decay = hs[3] > 0.0 && hs[4] >= 0.0 ? pow(hs[4] / hs[3], 0.5 / DECAY) : 1.0;
+  const double rest = 1.05 * decay + 0.02;  // estimate + margin
+  g->per_ok = lambda > 1e-3 && lambda < 1.0 + 1e-9 && settled(q[0], q[1], q[2]) && settled(q[3], q[4], q[5]) &&
+              q[6] * q[7] <= kModeCondition * hs[0] && rest < 1.0;
   g->per_b = 1.0;
   if (g->per_ok) {
     g->per_lambda = std::min(lambda, 1.0);
-    const double b = pow(std::max(0.0, hs[4] / hs[3]), 0.5 / DECAY);
-    g->per_b = std::min(1.0, 1.05 * b + 0.02);
+    g->per_b = rest;
     { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_dir_finish<<<nb, 256, 0, ctx->stream>>>(
         n, orp, invdw, v, t, u, hs[0], g->per_vy.as<float>(), g->per_u.as<float>()); }
     PPRVIZ_LAUNCHED(ctx);

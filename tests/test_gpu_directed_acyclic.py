@@ -2,7 +2,8 @@
 the solves may start from the walk's dominant mode: graphs without cycles (no
 mode: what 40 power steps leave is no eigenvector), chains of classes, periodic
 walks, weighted graphs. Every entry lies within the two certificates of the
-plain FP64 power iteration."""
+plain FP64 power iteration, and where there is no mode to use a call takes the
+sweeps of one without the analysis (fewer than 2,048 columns)."""
 import numpy as np
 import pytest
 
@@ -114,6 +115,19 @@ def test_acyclic_graphs_converge_at_small_eps(ctx, kind, eps):
     D, _, cert, st = ctx.dppr(G, view, 0.15, eps, P.FP32_CSR, out64=True)
     assert st == 0
     within_certificates(ctx, G, view, 0.15, eps, D, cert)
+
+
+@pytest.mark.parametrize("kind", list(ACYCLIC))
+def test_acyclic_graphs_take_the_sweeps_of_the_plain_path(ctx, kind):
+    """One refinement pass at most, and the main sweeps of a call without the analysis."""
+    import paper_2112_14944_gb300 as P
+    G = ctx.upload_graph(ACYCLIC[kind]())
+    view = synth.sample_view(G.n, K, seed=7).astype(np.int32)
+    ctx.dppr(G, view[:FEW], 0.15, 1e-6, P.FP32_CSR)
+    few = per_group(ctx)
+    ctx.dppr(G, view, 0.15, 1e-6, P.FP32_CSR)
+    many = per_group(ctx)
+    assert many[0] == few[0] and many[1] <= max(1.0, few[1])
 
 
 @pytest.mark.parametrize("kind", ["power_law", "weighted"])
