@@ -1049,6 +1049,21 @@ int64_t choose_group_f32(int64_t n, int32_t k) {
   return choose_group(n, k, sizeof(float));
 }
 
+// Level-l DPPR, more than 64 supernodes and a state beyond L2: narrow groups
+// (k_sweep_nw) where they are the faster ones, as 64 columns, or on large graphs
+// as 32 where that pads less. A whole call at 32 / 64 / 128 columns, 128
+// supernodes, 10 edges per node: 45,000 nodes 3.5 / 2.0 / 1.75 ms, 60,000
+// 3.8 / 2.3 / 2.3, 100,000 4.6 / 3.4 / 4.0 (30 edges per node 7.8 / 6.0 / 6.2),
+// 2M 85 / 88 / 100; 200 supernodes: 100,000 nodes of 30 edges 13.4 / 11.8 / 11.9,
+// 200,000 of 10 13.0 / 15.2 / 16.5, 2M 150 / 176 / 203. Weighted, 128 supernodes:
+// 100,000 nodes of 30 edges 9.1 / 7.2 / 6.5, 300,000 of 10 15.5 / 13.7 / 13.8,
+// 2M 105 / 99 / 101.
+int64_t level_group(const pprviz_graph *g, int32_t nsup) {
+  const int64_t ld = choose_group_f32(g->n, nsup);
+  if (ld != kChunk || g->n < (pull_weighted(g) ? 300000 : 100000)) return ld;
+  return g->n >= 200000 && (nsup + 31) / 32 % 2 ? 32 : 64;
+}
+
 // A wave of batched views (see k_sweep): the state covers the union-graph
 // rows [row0, row0 + nrows), column q is source g0 + q of every row's view;
 // lidx[i] is node i's index within its view. The residual's blocks each cover
@@ -1925,8 +1940,7 @@ int level_dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, int32_t nsup, const
                      const std::vector<int32_t> &leaf_idx_h, double alpha, double eps, void *out_d, bool out64,
                      double *cert_h) {
   const int64_t n = g->n;
-  int64_t ld = choose_group_f32(n, nsup);
-  if (ld == kChunk && !state_fits(n, ld)) ld = 32;  // a state beyond L2: narrow groups (see k_sweep_nw)
+  const int64_t ld = level_group(g, nsup);
   const size_t sbytes = sizeof(float) * (size_t)(n * ld);
   PPRVIZ_TRY(ws_ensure(ctx, WS_Y0, sbytes));
   PPRVIZ_TRY(ws_ensure(ctx, WS_Y1, sbytes));
