@@ -30,7 +30,10 @@
  *  - The library owns the context, graph objects and its device workspace.
  *  - Dense matrices are row-major with leading dimension k. Node and view ids
  *    are 0-based. A view lists distinct node ids of the graph.
- *  - A context is used by one host thread at a time.
+ *  - A context is used by one host thread at a time. A graph may be used by
+ *    several contexts of its device at once; what the library keeps with it is
+ *    made on first use, by whichever call comes first. The caller frees a
+ *    graph when no call uses it any more.
  */
 #ifndef PPRVIZ_H
 #define PPRVIZ_H

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -109,21 +110,26 @@ struct pprviz_graph {
   double m = 0.0;
   std::vector<double> h_deg;  // host copy of d(v), for per-group decisions
   int64_t max_row = -1;       // edges of the longest row of the uploaded CSR, -1 if not known
+  // What follows up to the pull CSR, and the directed graph's own, is made on
+  // first use, by whichever context comes first: under `lazy`, finished on the
+  // device before its ready flag is set, and not changed afterwards.
+  mutable std::mutex lazy;
   // dense weight matrix for the tensor-core sweeps, built on first use
   mutable pprviz::DevBuf dense;
   mutable int64_t dense_nw = 0;
+  mutable std::atomic<bool> dense_ready{false};
   // component roots and spectral bound for the deflated sweeps, on first use
   mutable pprviz::DevBuf comp;             // root (smallest id) of each node's component
   mutable std::vector<int32_t> h_comp;     // host copy
   mutable std::vector<double> h_mc;        // m_C = sum of walk degrees, indexed by root
   mutable double spec_b = 1.0;             // |lambda| <= spec_b off the stationary modes (estimate + margin)
   mutable bool spec_deflate = false;       // components resolved
-  mutable bool spec_ready = false;
+  mutable std::atomic<bool> spec_ready{false};
   // sweep work items with heavy rows split into segments of at most 64 edges,
   // built on first use (sweep_plan in propagate.cu)
   mutable pprviz::DevBuf sp_items, sp_srow;
   mutable int64_t sp_nitems = 0, sp_nsplit = 0, sp_nslots = 0;
-  mutable bool sp_ready = false;
+  mutable std::atomic<bool> sp_ready{false};
   // directed graphs: the pull CSR (row j lists the in-neighbours i of j with
   // the weights w_ij, or 1; a dangling j has the entry (j, 1), a j without
   // in-edges the entry (j, 0)), so that no gather row is empty
@@ -133,7 +139,7 @@ struct pprviz_graph {
   // entries (the sweeps solve for those nodes directly, see directed_prepare);
   // made on first use (directed_weights)
   mutable pprviz::DevBuf pws;
-  mutable bool pws_ready = false;
+  mutable std::atomic<bool> pws_ready{false};
   // directed graphs, on first use (graph_perron): the dominant mode of the walk
   // among the non-dangling nodes. vy = its left vector / dw (for a dangling
   // node what flows into it from the left vector), u = its right vector, scaled
@@ -141,8 +147,9 @@ struct pprviz_graph {
   mutable pprviz::DevBuf per_vy, per_u;
   mutable std::vector<float> h_u;
   mutable double per_lambda = 0.0, per_b = 1.0;
-  mutable bool per_ok = false, per_ready = false;
-  mutable std::atomic<int64_t> per_cols{0};  // source columns solved or asked for until then
+  mutable bool per_ok = false;
+  mutable std::atomic<bool> per_ready{false};
+  mutable std::atomic<int64_t> per_cols{0};  // source columns solved or asked for
 };
 
 namespace pprviz {

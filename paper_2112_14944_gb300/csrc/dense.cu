@@ -617,7 +617,9 @@ int64_t dense_group(int32_t k) {
 int dense_prepare(pprviz_ctx *ctx, const pprviz_graph *g) {
   const int64_t n = g->n;
   const int64_t nw = (n + 31) / 32 * 32, mw = (n + 127) / 128 * 128;
-  if (g->dense.p && g->dense_nw == nw) return PPRVIZ_OK;
+  if (g->dense_ready) return PPRVIZ_OK;
+  std::lock_guard<std::mutex> lock(g->lazy);
+  if (g->dense_ready) return PPRVIZ_OK;
   const size_t bytes = sizeof(float) * (size_t)mw * (size_t)nw;
   cudaError_t e = g->dense.ensure(bytes);
   if (e != cudaSuccess) {
@@ -633,7 +635,9 @@ int dense_prepare(pprviz_ctx *ctx, const pprviz_graph *g) {
         g->dense.as<float>());
   }
   PPRVIZ_LAUNCHED(ctx);
+  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   g->dense_nw = nw;
+  g->dense_ready = true;
   return PPRVIZ_OK;
 }
 

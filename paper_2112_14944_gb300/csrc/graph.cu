@@ -226,6 +226,8 @@ int pull_csr_build(pprviz_ctx *ctx, pprviz_graph *g, const int64_t *rp, const in
 
 int directed_weights(pprviz_ctx *ctx, const pprviz_graph *g) {
   if (g->pws_ready) return PPRVIZ_OK;
+  std::lock_guard<std::mutex> lock(g->lazy);
+  if (g->pws_ready) return PPRVIZ_OK;
   int64_t pnnz = 0;
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(&pnnz, g->prp.as<int64_t>() + g->n, sizeof(pnnz), cudaMemcpyDeviceToHost,
                                    ctx->stream));
@@ -239,7 +241,7 @@ int directed_weights(pprviz_ctx *ctx, const pprviz_graph *g) {
   { PPRVIZ_PROF(ctx, PPRVIZ_K_GRAPH); k_drop_own<<<(unsigned)((g->n + 255) / 256), 256, 0, ctx->stream>>>(
       g->n, g->prp.as<int64_t>(), g->pcol.as<int32_t>(), g->pws.as<float>()); }
   PPRVIZ_LAUNCHED(ctx);
-  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));  // other contexts may use it from here on
+  PPRVIZ_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   g->pws_ready = true;
   return PPRVIZ_OK;
 }

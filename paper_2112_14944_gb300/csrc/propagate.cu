@@ -1115,6 +1115,8 @@ int64_t split_items(const std::vector<int64_t> &rp, int64_t r0, int64_t r1, std:
 // The split plan of a whole graph, built once and kept with it.
 int sweep_plan(pprviz_ctx *ctx, const pprviz_graph *g) {
   if (g->sp_ready) return PPRVIZ_OK;
+  std::lock_guard<std::mutex> lock(g->lazy);
+  if (g->sp_ready) return PPRVIZ_OK;
   const int64_t n = g->n;
   std::vector<int64_t> rp((size_t)n + 1);
   PPRVIZ_CUDA(ctx, cudaMemcpyAsync(rp.data(), pull_rp(g), sizeof(int64_t) * rp.size(), cudaMemcpyDeviceToHost,
@@ -1566,11 +1568,12 @@ int chebyshev_solve(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
 constexpr int64_t kPerronColumns = 2048;
 int directed_prepare(pprviz_ctx *ctx, const pprviz_graph *g, double alpha, int64_t perron_cols) {
   const int64_t n = g->n;
-  bool perron = perron_cols > 0;
   PPRVIZ_TRY(directed_weights(ctx, g));
-  if (perron && !g->per_ready && g->per_cols.fetch_add(perron_cols) + perron_cols >= kPerronColumns)
+  bool perron = perron_cols > 0 && g->per_cols.fetch_add(perron_cols) + perron_cols >= kPerronColumns;
+  if (perron) {
     PPRVIZ_TRY(graph_perron(ctx, g));
-  perron = perron && g->per_ok;
+    perron = g->per_ok;
+  }
   const size_t vec = (sizeof(float) * (size_t)n + 255) & ~(size_t)255;
   PPRVIZ_TRY(ws_ensure(ctx, WS_DIRS, 2 * vec));
   float *invd = ctx->ws[WS_DIRS].as<float>();

@@ -371,6 +371,8 @@ __global__ void k_dir_finish(int64_t n, const int64_t *__restrict__ orp, const d
 constexpr double kModeResidual = 1e-3, kModeCondition = 100.0;
 int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
   if (g->per_ready) return PPRVIZ_OK;
+  std::lock_guard<std::mutex> lock(g->lazy);
+  if (g->per_ready) return PPRVIZ_OK;
   constexpr int STEPS = 40, DECAY = 8;
   const int64_t n = g->n;
   const unsigned nb = (unsigned)((n + 255) / 256), wb = (unsigned)((n * 32 + 255) / 256);
@@ -483,6 +485,8 @@ int graph_perron(pprviz_ctx *ctx, const pprviz_graph *g) {
 }
 
 int graph_spectral(pprviz_ctx *ctx, const pprviz_graph *g) {
+  if (g->spec_ready) return PPRVIZ_OK;
+  std::lock_guard<std::mutex> lock(g->lazy);
   if (g->spec_ready) return PPRVIZ_OK;
   const int64_t n = g->n;
   const unsigned nb = (unsigned)((n + 255) / 256), wb = (unsigned)((n * 32 + 255) / 256);
