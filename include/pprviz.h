@@ -28,6 +28,13 @@
  *    pointers and are written before the call returns (the call waits for the
  *    values they need).
  *  - The library owns the context, graph objects and its device workspace.
+ *  - FP32 DPPR, PDist and what follows from them are reproducible to their
+ *    certificates, not to the last digit. The same call on the same context
+ *    returns the same digits again, except that a context chooses its launch
+ *    shapes by timing on the first call of a size class (another context may
+ *    choose others, which add up in another order), and that a directed
+ *    graph's solves start from the walk's dominant mode once the graph has
+ *    been asked for 2,048 source columns in all, by any context.
  *  - Dense matrices are row-major with leading dimension k. Node and view ids
  *    are 0-based. A view lists distinct node ids of the graph.
  *  - A context is used by one host thread at a time. A graph may be used by
