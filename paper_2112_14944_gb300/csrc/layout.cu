@@ -168,11 +168,10 @@ __global__ void k_build_diag(int32_t k, int32_t kp, const double *__restrict__ r
 // ---------------------------------------------------------------------------
 constexpr int ST64 = 64;
 
-// Sum over the 32 lanes of NV values per lane; returns, in every lane, the
-// total of value index lane / (32 / NV). Recursive halving: 31 shuffles for
-// NV = 32, 15 + 1 for NV = 16.
+// The halving steps of lanes_transpose_sum: value index lane / (32 / NV) summed
+// over the lanes of equal lane % (32 / NV).
 template <int NV, typename T>
-__device__ __forceinline__ T lanes_transpose_sum(T (&v)[NV], int lane) {
+__device__ __forceinline__ T lanes_fold(T (&v)[NV], int lane) {
   constexpr int LOG = NV == 32 ? 5 : NV == 16 ? 4 : NV == 8 ? 3 : NV == 4 ? 2 : NV == 2 ? 1 : 0;
 #pragma unroll
   for (int s = 0; s < LOG; ++s) {
@@ -186,7 +185,16 @@ __device__ __forceinline__ T lanes_transpose_sum(T (&v)[NV], int lane) {
       v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
     }
   }
-  T r = v[0];
+  return v[0];
+}
+
+// Sum over the 32 lanes of NV values per lane; returns, in every lane, the
+// total of value index lane / (32 / NV). Recursive halving: 31 shuffles for
+// NV = 32, 15 + 1 for NV = 16.
+template <int NV, typename T>
+__device__ __forceinline__ T lanes_transpose_sum(T (&v)[NV], int lane) {
+  constexpr int LOG = NV == 32 ? 5 : NV == 16 ? 4 : NV == 8 ? 3 : NV == 4 ? 2 : NV == 2 ? 1 : 0;
+  T r = lanes_fold<NV, T>(v, lane);
 #pragma unroll
   for (int off = 16 >> LOG; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
   return r;
@@ -897,16 +905,18 @@ __global__ void k_finish(int32_t k, const typename T2<T>::type *__restrict__ X, 
 // cycle and SM): one FP64 add and one conversion per pair alone cost five
 // times the read. In FP32 the squares e^2 are therefore summed as a float and
 // its exact rounding errors (TwoSum, Knuth), two rows at a time with the
-// paired FP32 instructions, and converted once per thread; the sum is as
-// exact as the FP64 sum it replaces (~2^-46). 1/Delta and 1/d come from the
-// special-function unit, each followed by one Newton step (Newton's iteration
-// for a^-1 and a^-1/2), which leaves them within about an ulp. Pairs outside
+// paired FP32 instructions, and go to an FP64 sum every QCH columns: over so
+// few terms the roundings of the error word come to ~2^-49 of them (FP64
+// additions: 2^-53 each; the squares themselves are rounded to 2^-24).
+// 1/Delta, d and (-2 e u) / d start from the special-function unit, each
+// followed by one correction from its residual (Newton's iteration), so that
+// each is rounded about once, as in the plain formulas. Pairs outside
 // the range in which those steps are safe (coincident or extremely close
 // points, huge or tiny values, infinities, NaN, the diagonal) and a last
 // group of fewer than ERPB rows take the plain formulas.
 // Measured at k = 8,192 on one GB300 (read 268 MB, write 268 MB with
-// grad_pdist), before -> now: energy alone 572 -> 95 us, both gradients
-// 692 -> 142 us. It now issues ~30 instructions per pair, most of them on
+// grad_pdist), before -> now, with the reduce: energy alone 581 -> 104 us, both
+// gradients 701 -> 161 us. It now issues ~30 instructions per pair, most of them on
 // the FMA pipe, and waits on loads for the rest.
 // ---------------------------------------------------------------------------
 constexpr int ERPB = 4;                 // rows of a row group
@@ -932,8 +942,25 @@ struct EAcc {
     c = __fadd2_rn(c, __fadd2_rn(e0, e1));
     s = t;
   }
-  __device__ __forceinline__ double total() const {
-    return d + (((double)s.x + (double)s.y) + ((double)c.x + (double)c.y));
+  // to the FP64 sum, before the roundings of c add up to one of its
+  __device__ __forceinline__ void flush() {
+    d += ((double)s.x + (double)s.y) + ((double)c.x + (double)c.y);
+    s = c = make_float2(0.0f, 0.0f);
+  }
+};
+
+// The shares of a row's gradient are added up with their rounding errors from
+// groups of eight threads on: a row has 256 shares, at k = 1,000 one for every
+// four terms, and plain sums of them lost more than 32 shares a row did. Root
+// mean square error of a gradient at k = 1,000, 32 plain shares, 256 plain, now:
+// FP32 4.4e-8, 5.2e-8, 2.9e-8; FP64 (k = 700) 7.7e-17, 9.6e-17, 5.2e-17. Both
+// gradients at k = 8,192: 153 -> 161 us.
+template <typename T>
+struct Sum2 {  // a sum and its rounding errors (TwoSum, Knuth)
+  T s, c;
+  __device__ __forceinline__ Sum2 operator+(Sum2 b) const {
+    const T t = s + b.s, bb = t - s;
+    return {t, ((s - (t - bb)) + (b.s - bb)) + (c + b.c)};
   }
 };
 
@@ -983,7 +1010,7 @@ k_energy(int32_t k, const T *__restrict__ Delta, const typename T2<T>::type *__r
   constexpr int WARPS = ETHREADS / 32;
   constexpr int QCH = 32;  // columns per thread between two runs of the plain formulas (bits of `plain`)
   __shared__ double se[WARPS];
-  __shared__ T sg[WARPS][2 * ERPB];
+  __shared__ Sum2<T> sg[WARPS][2 * ERPB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   EAcc<T> acc;
   int bad = 0;
@@ -1050,9 +1077,10 @@ k_energy(int32_t k, const T *__restrict__ Delta, const typename T2<T>::type *__r
               const float2 e = __ffma2_rn(__fmul2_rn(n, d), u, one);
               acc.add2(__fmul2_rn(e, e));
               if (GX) {
-                // 1 / d = y0 + y0 (1 - d y0)
-                const float2 y = __ffma2_rn(__ffma2_rn(__fmul2_rn(n, d), y0, one), y0, y0);
-                const float2 cf = __fmul2_rn(__fmul2_rn(make_float2(-2.0f, -2.0f), e), __fmul2_rn(u, y));
+                // (-2 e u) / d = q0 + y0 (t - d q0)
+                const float2 t = __fmul2_rn(__fmul2_rn(make_float2(-2.0f, -2.0f), e), u);
+                const float2 q0 = __fmul2_rn(t, y0);
+                const float2 cf = __ffma2_rn(__ffma2_rn(__fmul2_rn(n, d), q0, t), y0, q0);
                 const float2 gX = __ffma2_rn(cf, dx[p], make_float2(gxx[2 * p], gxx[2 * p + 1]));
                 const float2 gY = __ffma2_rn(cf, dy[p], make_float2(gxy[2 * p], gxy[2 * p + 1]));
                 gxx[2 * p] = gX.x;
@@ -1068,6 +1096,7 @@ k_energy(int32_t k, const T *__restrict__ Delta, const typename T2<T>::type *__r
               }
             }
           }
+          acc.flush();
         }
       }
       while (plain) {
@@ -1089,20 +1118,23 @@ k_energy(int32_t k, const T *__restrict__ Delta, const typename T2<T>::type *__r
         v[2 * r] = gxx[r];
         v[2 * r + 1] = gxy[r];
       }
-      const T tot = lanes_transpose_sum<2 * ERPB, T>(v, lane);
       constexpr int REP = 32 / (2 * ERPB);
+      Sum2<T> tot{lanes_fold<2 * ERPB, T>(v, lane), T(0)};
+#pragma unroll
+      for (int off = REP / 2; off > 0; off >>= 1)
+        tot = tot + Sum2<T>{__shfl_xor_sync(0xffffffffu, tot.s, off), __shfl_xor_sync(0xffffffffu, tot.c, off)};
       if (lane % REP == 0) sg[warp][lane / REP] = tot;
       __syncthreads();
       if (threadIdx.x < 2 * ERPB && r0 + (threadIdx.x >> 1) < k) {
-        T s = T(0);
+        Sum2<T> s = sg[0][threadIdx.x];
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) s += sg[w][threadIdx.x];
-        gx[2 * r0 + threadIdx.x] = scale * s;
+        for (int w = 1; w < WARPS; ++w) s = s + sg[w][threadIdx.x];
+        gx[2 * r0 + threadIdx.x] = scale * (s.s + s.c);
       }
       __syncthreads();  // before the next group's sums
     }
   }
-  double e = acc.total();
+  double e = acc.d;
   for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
   if (lane == 0) se[warp] = e;
   __syncthreads();
