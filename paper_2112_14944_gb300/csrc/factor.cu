@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "recip.cuh"
 
 namespace pprviz {
 
@@ -38,12 +39,6 @@ size_t spd_inverse_work(int32_t kp) { return (size_t)2 * (2 * 256 * (size_t)kp +
 // an estimate with two Newton steps instead of a division per thread:
 // 284 -> 114 us per block.
 constexpr int DIAG64_THREADS = 160;
-__device__ __forceinline__ double rcp_pos(double a) {  // 1/a, a > 0 normal (pivots of an SPD matrix)
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  r = fma(fma(-a, r, 1.0), r, r);
-  return fma(fma(-a, r, 1.0), r, r);
-}
 __global__ void __launch_bounds__(DIAG64_THREADS) k_fac_diag64(int32_t kp, int32_t K0, double *__restrict__ A,
                                                                double *__restrict__ P) {
   __shared__ __align__(16) double col[2][64];
@@ -185,11 +180,7 @@ __device__ __forceinline__ void fac_diag128(int32_t kp, int32_t K0, float *__res
     for (int w = 0; w < 4; ++w) {
       const float *v = col[w & 1];  // 4 T is even
       {
-        // 1 / a_pp: the estimate and one Newton step
-        const float app = v[4 * T + w];
-        float piv;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(piv) : "f"(app));
-        piv = fmaf(fmaf(-app, piv, 1.0f), piv, piv);
+        const float piv = rcp_pos(v[4 * T + w]);
         const float4 r4 = *reinterpret_cast<const float4 *>(v + 4 * R);
         const float4 c4 = *reinterpret_cast<const float4 *>(v + 4 * C);
         const float vr[4] = {r4.x, r4.y, r4.z, r4.w};

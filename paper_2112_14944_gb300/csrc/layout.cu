@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "recip.cuh"
 
 namespace pprviz {
 
@@ -36,21 +37,6 @@ constexpr int ST = 128;       // symmetric pass tile edge
 template <typename T> struct T2;
 template <> struct T2<float> { using type = float2; };
 template <> struct T2<double> { using type = double2; };
-
-// 1/sqrt(d2), 0 for d2 = 0 (FP64 layout). GB300 has two FP64 operations per
-// cycle and SM, and an FP64 square root and division take some tens of them:
-// the special-function unit's estimate (20 bits or more) and one third-order
-// step of the series of (1 - e)^-1/2, e = 1 - d2 y^2 (Halley's iteration),
-// take five and leave an error of an ulp or so. Values outside the normal
-// range take the plain formula.
-__device__ __forceinline__ double rsqrt_pos(double d2) {
-  const uint32_t hi = (uint32_t)__double2hiint(d2);
-  if (hi - 0x01000000u >= 0x7e000000u - 0x01000000u) return d2 > 0.0 ? 1.0 / sqrt(d2) : 0.0;
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d2));
-  const double e = fma(-(d2 * y), y, 1.0);
-  return fma(fma(e, 0.375, 0.5), e * y, y);
-}
 
 // ---------------------------------------------------------------------------
 // Build from Delta_s = (Delta + Delta^T) / 2, in 32 x 32 tiles with the mirrored
@@ -72,8 +58,8 @@ template <>
 __device__ __forceinline__ float recip<float>(float d) { return __frcp_rn(d); }
 
 // Sum of 32 values p[0], p[stride], ...: FP64 additions, or, for floats, a float
-// sum with its exact rounding errors (TwoSum, Knuth), which is as exact and
-// stays off GB300's narrow FP64 pipe.
+// sum with its exact rounding errors (TwoSum, Knuth), good to ~2^-50 of the sum
+// (it becomes part of an FP32 diagonal entry) and off GB300's narrow FP64 pipe.
 __device__ __forceinline__ double sum32(const double *p, int stride) {
   double s = 0.0;
   for (int e = 0; e < 32; ++e) s += p[e * stride];
