@@ -153,7 +153,7 @@ int pprviz_create(pprviz_ctx **out, int device, void *cuda_stream) {
 
 int pprviz_test_expire_wait(pprviz_ctx *ctx) {
   if (!ctx) return PPRVIZ_E_INVALID_ARG;
-  ctx->test_expire_wait = true;
+  ctx->test_expire_wait++;
   return PPRVIZ_OK;
 }
 

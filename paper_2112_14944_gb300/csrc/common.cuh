@@ -87,7 +87,10 @@ struct pprviz_ctx {
   std::string err;
   pprviz::DevBuf ws[pprviz::WS_COUNT];
   size_t ws_limit = 0;  // cap on the summed workspace capacity (0 = none); pprviz_set_workspace_limit
-  bool test_expire_wait = false;  // pprviz_test_expire_wait: the next FP32 inverse withholds one copy
+  // pprviz_test_expire_wait: the n-th launch from now of those that can withhold
+  // a signal does so (0: none); asked by each of them in turn
+  int test_expire_wait = 0;
+  bool expire_here() { return test_expire_wait > 0 && --test_expire_wait == 0; }
   bool scnt_clear = false;        // the split sweep's arrival counters are zero (set per call)
   // directed FP32 solves (set per call by directed_prepare, propagate.cu): the
   // sweeps' 1 / dw, and the y-scaled Perron vector of the deflated start or NULL

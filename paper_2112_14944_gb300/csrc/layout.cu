@@ -730,8 +730,9 @@ template <int NR>
 __global__ void __launch_bounds__(512, 1)
 k_layout_resident(int32_t k, int32_t kp, int32_t kq, int nrows, int iters, const float *__restrict__ W1,
                   const float *__restrict__ M, float2 *X, float2 *B, uint32_t *bar, int *__restrict__ err,
-                  uint64_t limit_ns) {
+                  uint64_t limit_ns, int withhold) {
   using namespace resident;
+  if (withhold && blockIdx.x + 1 == gridDim.x) return;  // (a test of the barrier's expiry: this CTA never arrives)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   float *sW = reinterpret_cast<float *>(smem_raw);  // [nrows][kq]
   float *sM = sW + (size_t)nrows * kq;              // [nrows][kq]
@@ -1354,8 +1355,10 @@ int resident_updates(pprviz_ctx *ctx, int32_t k, int32_t kp, int iters, const fl
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const int withhold = ctx->expire_here() ? 1 : 0;
   PPRVIZ_PROF(ctx, PPRVIZ_K_LY);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, k, kp, kq, nrows, iters, W1, M, X, B, bar, err, limit_ns);
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, kernel, k, kp, kq, nrows, iters, W1, M, X, B, bar, err, limit_ns, withhold);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // not all CTAs fit at once: the pipeline takes it
     cudaGetLastError();
     return PPRVIZ_OK;
