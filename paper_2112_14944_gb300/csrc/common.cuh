@@ -328,8 +328,9 @@ int pdist_launch(pprviz_ctx *ctx, const void *dppr_d, int32_t k, int64_t n_clamp
 // holds A^-1 on its upper 64-block triangle and on the 128 x 128 diagonal tiles.
 // `work` holds spd_inverse_work(kp) elements: two sets (the lookahead's
 // parities) of panels (2 x 2 NB x kp: Ct and Ut split into high and low
-// parts, NB = 128) and pivot inverse (NB x NB). The FP32 version runs its trailing updates on the tensor cores; *err
-// (device, zeroed by the caller) is set if one of their bounded waits expires.
+// parts, NB = 128) and pivot inverse (NB x NB). The FP32 version runs its trailing
+// updates on the tensor cores; *err (device, zeroed by the caller) is set if one
+// of their bounded waits expires.
 size_t spd_inverse_work(int32_t kp);  // elements of `work` for either type
 int spd_inverse_f32(pprviz_ctx *ctx, int32_t kp, float *A, float *work, int *err);
 // FP32 inverses of many SPD matrices at once (A[v]: kp[v] x kp[v] device,

@@ -23,8 +23,8 @@
 namespace pprviz {
 
 // two sets (the lookahead's parities) of panels Ct, Ut (2 NB x kp each: the
-// split high and low parts) and pivot inverse P (NB x NB), and a status word
-size_t spd_inverse_work(int32_t kp) { return (size_t)2 * (2 * 256 * (size_t)kp + 128 * 128) + 64; }
+// split high and low parts) and pivot inverse P (NB x NB)
+size_t spd_inverse_work(int32_t kp) { return (size_t)2 * (2 * 256 * (size_t)kp + 128 * 128); }
 
 // FP64: P = A_KK^-1 of a 64 x 64 block by the scalar sweep
 //   a_pp -> 1/a_pp, a_pc -> a_pc/a_pp, a_rp -> -a_rp/a_pp, a_rc -> a_rc - a_rp a_pc/a_pp,

@@ -304,7 +304,7 @@ struct BatchView {
   int64_t mat_off;   // elements into the batched kp x kp matrices
   int64_t vec_off;   // 2-vectors into the batched coordinate / b vectors (kp each)
   int64_t part_off;  // 2-vectors into the batched partial sums (nbt x kp each)
-  int32_t kp, nbt, k, cnt_off;  // cnt_off: the view's first row block among all views'
+  int32_t kp, nbt, k;
 };
 
 // ---------------------------------------------------------------------------
@@ -1406,7 +1406,7 @@ int layout_typed(pprviz_ctx *ctx, const TI *pdist, int32_t k, const TI *x0, int3
   PPRVIZ_LAUNCHED(ctx);
   // the view descriptor (FP32), or the upper tile triangle in row order and the
   // row-block counters of the fused reduce, zero between passes (FP64)
-  const BatchView one{0, 0, 0, kp, nbt, k, 0};
+  const BatchView one{0, 0, 0, kp, nbt, k};
   if constexpr (std::is_same<T, float>::value) {
     int *perr = flag + 1;
     bool done = false;
@@ -1511,15 +1511,13 @@ int layout_batch_run(pprviz_ctx *ctx, int32_t nviews, const int64_t *k_h, const 
   std::vector<BatchView> bv((size_t)nviews);
   int64_t mat = 0, vec = 0, part = 0, maxkp = 0;
   size_t ntile = 0;
-  int32_t cnts = 0;
   for (int32_t v = 0; v < nviews; ++v) {
     const int32_t k = (int32_t)k_h[v];
     const int32_t kp = (k + ST - 1) / ST * ST, nbt = kp / ST;
-    bv[v] = BatchView{mat, vec, part, kp, nbt, k, cnts};
+    bv[v] = BatchView{mat, vec, part, kp, nbt, k};
     mat += (int64_t)kp * kp;
     vec += kp;
     part += (int64_t)nbt * kp;
-    cnts += nbt;
     maxkp = std::max<int64_t>(maxkp, kp);
     ntile += (size_t)nbt * (nbt + 1) / 2;
   }

@@ -1033,10 +1033,6 @@ __global__ void k_extract(int32_t k, int32_t g0, int32_t gvalid, int64_t ld,
 // --------------------------------------------------------------------------
 namespace {
 
-struct GroupPlan {
-  int64_t ld;    // group width (multiple of kChunk)
-};
-
 int64_t choose_group(int64_t n, int32_t k, size_t elem) {
   // keep ~3 live [n][G] buffers within ~64 MB of L2
   const double budget = 64.0 * 1024 * 1024;
