@@ -37,7 +37,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <cmath>
 #include <type_traits>
 #include <cstring>
 
@@ -1470,7 +1469,7 @@ double cert_worst(const std::vector<double> &cert) {
 double finite_max(const std::vector<double> &cert) {
   double m = 0.0;
   for (double v : cert)
-    if (std::isfinite(v)) m = std::max(m, v);
+    if (v > m && v < INFINITY) m = v;
   return m;
 }
 
@@ -2542,7 +2541,7 @@ int dppr_views_solve(pprviz_ctx *ctx, int32_t nviews, const pprviz_graph *const 
           const int64_t gv = std::min<int64_t>(ld, views[v]->n - g0);
           for (int64_t q = 0; q < gv; ++q) {
             const double cq = views[v]->h_deg[(size_t)(g0 + q)] * l1h[(size_t)(w * 2) * ld + q] / alpha;
-            if (std::isfinite(cq)) cmax = std::max(cmax, cq);  // (as finite_max)
+            if (cq > cmax && cq < INFINITY) cmax = cq;  // (as finite_max)
           }
         }
         return PPRVIZ_OK;
