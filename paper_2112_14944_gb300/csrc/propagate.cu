@@ -1054,19 +1054,36 @@ int64_t choose_group_f32(int64_t n, int32_t k) {
   return choose_group(n, k, sizeof(float));
 }
 
-// Level-l DPPR, more than 64 supernodes and a state beyond L2: narrow groups
-// (k_sweep_nw) where they are the faster ones, as 64 columns, or on large graphs
-// as 32 where that pads less. A whole call at 32 / 64 / 128 columns, 128
-// supernodes, 10 edges per node: 45,000 nodes 3.5 / 2.0 / 1.75 ms, 60,000
-// 3.8 / 2.3 / 2.3, 100,000 4.6 / 3.4 / 4.0 (30 edges per node 7.8 / 6.0 / 6.2),
-// 2M 85 / 88 / 100; 200 supernodes: 100,000 nodes of 30 edges 13.4 / 11.8 / 11.9,
-// 200,000 of 10 13.0 / 15.2 / 16.5, 2M 150 / 176 / 203. Weighted, 128 supernodes:
-// 100,000 nodes of 30 edges 9.1 / 7.2 / 6.5, 300,000 of 10 15.5 / 13.7 / 13.8,
-// 2M 105 / 99 / 101.
+// Level-l DPPR, more than 64 supernodes and a state beyond L2: the width by the
+// columns that a call computes at it (whole groups) and what a column costs. A
+// call of 128 supernodes at 32 / 64 / 128 columns (ms), 10 edges per node (30 in
+// brackets), where all three compute 128:
+//                 unweighted                        weighted                        directed
+//   50,000   3.8 / 2.0 / 1.9 (5.3/3.3/3.0)     3.9 / 2.2 / 2.0 (5.8/3.7/3.2)     7.0 / 3.9 / 4.1
+//   70,000   4.0 / 2.6 / 2.9 (6.0/4.3/4.2)     4.2 / 2.9 / 3.0 (6.9/4.9/4.5)     7.1 / 4.6 / 6.1
+//  100,000   4.6 / 3.4 / 4.0 (7.7/6.0/6.0)     5.2 / 3.9 / 4.2 (8.8/7.2/6.4)     8.3 / 6.5 / 8.8
+//  150,000   6.0 / 5.5 / 6.1 (10.6/9.2/9.6)    7.0 / 6.4 / 6.3 (13/10.7/10)     11.5 / 13.2 / 14.3
+//  300,000  11.9 /11.3 /12.6 (20/19/22)       15.2 /13.1 /13.0 (26/22.5/22.6)   27.3 / 26.6 / 26.8
+// and fewer where a narrow group pads less: 70 supernodes (96 / 128 / 128 columns)
+// on 150,000 nodes 4.5 / 5.4 / 6.0, weighted 5.2 / 6.4 / 6.4, directed 8.2 / 11.8 /
+// 13.1; 200 (224 / 256 / 256) on 2M 150 / 176 / 203.
 int64_t level_group(const pprviz_graph *g, int32_t nsup) {
-  const int64_t ld = choose_group_f32(g->n, nsup);
-  if (ld != kChunk || g->n < (pull_weighted(g) ? 300000 : 100000)) return ld;
-  return g->n >= 200000 && (nsup + 31) / 32 % 2 ? 32 : 64;
+  const int64_t n = g->n, ld = choose_group_f32(n, nsup);
+  if (ld != kChunk || state_fits(n, kChunk) || (n < 60000 && !g->directed)) return ld;
+  auto columns = [nsup](int64_t w) { return (double)((nsup + w - 1) / w * w); };
+  // what a column costs at 32 against 64, and at 64 against 128
+  double r32, r64 = 0.95;
+  if (g->directed) {
+    r32 = n < 80000 ? 1.5 : n < 110000 ? 1.25 : n < 250000 ? 0.95 : 1.03;
+  } else if (g->weighted) {
+    const bool dense = (double)g->nnz > 15.0 * (double)n;
+    r32 = n < 110000 ? 1.35 : n < 140000 ? 1.2 : 1.08;
+    r64 = dense ? 1.1 : n < 140000 ? 0.95 : 1.0;
+  } else {
+    r32 = n < 110000 ? 1.35 : n < 140000 ? 1.18 : 1.07;
+  }
+  const double c32 = r32 * r64 * columns(32), c64 = r64 * columns(64), c128 = columns(128);
+  return c32 < c64 ? (c32 < c128 ? 32 : 128) : (c64 < c128 ? 64 : 128);
 }
 
 // A wave of batched views (see k_sweep): the state covers the union-graph

@@ -9,17 +9,21 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,nsup,weighted,group", [
-    (43000, 70, False, 128), (45000, 96, False, 128), (99999, 70, False, 128), (100001, 70, False, 64),
-    (200001, 70, False, 32), (200001, 100, False, 64), (200001, 100, True, 128), (300001, 130, True, 32),
+@pytest.mark.parametrize("n,nsup,kind,group", [
+    (43000, 70, "unweighted", 128), (45000, 96, "unweighted", 128), (70001, 70, "unweighted", 64),
+    (130001, 70, "unweighted", 32), (200001, 100, "unweighted", 64), (45000, 96, "weighted", 128),
+    (200001, 100, "weighted", 128), (300001, 130, "weighted", 32), (43000, 70, "directed", 128),
+    (50001, 96, "directed", 64), (150001, 100, "directed", 32),
 ])
-def test_level_group_width(n, nsup, weighted, group):
+def test_level_group_width(n, nsup, kind, group):
     import paper_2112_14944_gb300 as P
     g = synth.chung_lu(n, 4, 2.5, seed=3)
-    if weighted:  # symmetric weights from the pair
+    if kind == "weighted":  # symmetric weights from the pair
         u, v = np.repeat(np.arange(n), np.diff(g.row_ptr)), g.col.astype(np.int64)
         w = (0.5 + ((np.minimum(u, v) * 7919 + np.maximum(u, v) * 104729) % 997) / 997.0).astype(np.float32)
         g = synth.Graph(n, g.row_ptr, g.col, w)
+    if kind == "directed":
+        g = synth.directed_from(g, seed=4)
     c = P.Context(0)
     try:
         G = c.upload_graph(g)
