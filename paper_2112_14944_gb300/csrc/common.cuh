@@ -66,6 +66,14 @@ enum Slot {
   WS_COUNT
 };
 
+// Times (ms) of one sweep and one residual pass at 32, 64 and 128 columns, by
+// graph size class (tuned_shape in propagate.cu).
+struct NarrowTimes {
+  uint64_t key;
+  float sweep[3], residual[3];
+  int res_blocks;  // the residual's CTA count at 128 columns
+};
+
 }  // namespace pprviz
 
 struct pprviz_ctx {
@@ -100,6 +108,7 @@ struct pprviz_ctx {
   int launches = 0;  // kernels launched in the current call
   // source-group widths chosen by the sweep autotuner, by graph size class
   std::vector<std::pair<uint64_t, int64_t>> tuned_groups;
+  std::vector<pprviz::NarrowTimes> tuned_narrow;
 };
 
 struct pprviz_graph {

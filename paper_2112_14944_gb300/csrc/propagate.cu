@@ -1355,10 +1355,17 @@ int launch_residual(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const in
 // lengths of n, nnz and k, weighted or not), kept in the context so that its
 // cost (a few milliseconds) is paid on the first call of each class:
 //  * the source-group width G: candidates 128, 256, ... up to the width whose
-//    ~3 live [n][G] buffers fill ~64 MB of L2 (choose_group), and 32 and 64
-//    where not even 128 columns fit; each runs three timed Chebyshev sweeps on
-//    the graph (after one untimed), and the width with the least time for all
-//    k sources wins;
+//    ~3 live [n][G] buffers fill ~64 MB of L2 (choose_group); each runs three
+//    timed Chebyshev sweeps on the graph (after one untimed), and the width
+//    with the least time for all k sources wins;
+//  * where not even 128 columns fit, 32, 64 and 128: three timed sweeps and one
+//    timed residual pass each, kept by n and nnz in quarter octaves for all k
+//    (70,000 and 100,000 nodes choose differently). A group costs about 2 k1 sweeps
+//    (k1: the main solve's, for this call's alpha and graph), two residual
+//    passes and its host waits, and a narrower width has to win by 1 %: a
+//    residual pass takes as long as its longest row (0.33 ms at 32 columns, 0.36
+//    at 128 on 85,000 nodes of 30 weighted edges), so by the sweeps alone such a
+//    graph took 32 columns, 8.4 ms for 200 sources against 5.2 with 128;
 //  * then, at that width, the residual's CTA count (608 .. 4,864 in all): three
 //    timed residual passes with a low part each, the fastest wins.
 // The values of the state do not change the work of either kernel, so both
@@ -1368,17 +1375,44 @@ struct TunedShape {
   int res_blocks;
 };
 
-TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *status) {
+constexpr int64_t kNarrowWidths[3] = {32, 64, 128};
+
+// the width for k sources from a class's times; a state beyond L2 pays for the
+// right-hand side of the refinement's sweeps too, which the timed ones do not read
+int64_t narrow_group(const NarrowTimes &t, int64_t n, int32_t k, int k1) {
+  double cost[3];
+  for (int i = 0; i < 3; ++i) {
+    const int64_t groups = (k + kNarrowWidths[i] - 1) / kNarrowWidths[i];
+    const double sweep = t.sweep[i] * (state_fits(n, kNarrowWidths[i]) ? 1.0 : 1.08);
+    cost[i] = (double)groups * (2.0 * k1 * sweep + 2.0 * t.residual[i] + 0.03);
+  }
+  const int b = cost[0] < cost[1] ? 0 : 1;
+  return cost[b] < 0.99 * cost[2] ? kNarrowWidths[b] : kNarrowWidths[2];
+}
+
+// k1: sweeps of the main solve
+TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int k1, int *status) {
   *status = PPRVIZ_OK;
   auto bits = [](uint64_t x) { int b = 0; while (x) { ++b; x >>= 1; } return (uint64_t)b; };
   const uint64_t key = (bits((uint64_t)g->n) << 40) | (bits((uint64_t)g->nnz) << 32) | (bits((uint64_t)k) << 8) |
                        (g->weighted ? 1u : 0u) | (g->directed ? 2u : 0u);
   const int64_t gmax = choose_group_f32(g->n, k);
   if (gmax < kChunk) return TunedShape{gmax, 1216};  // one narrow group
+  const bool narrow = gmax == kChunk && !state_fits(g->n, kChunk);
+  // the narrow widths' class: quarter octaves of n and nnz, any k
+  auto quarter = [&bits](uint64_t x) { const uint64_t b = bits(x); return 4 * b + (b > 2 ? (x >> (b - 3)) & 3 : 0); };
+  const uint64_t nkey = (quarter((uint64_t)g->n) << 40) | (quarter((uint64_t)g->nnz) << 8) | (key & 3);
+  if (narrow)
+    for (const NarrowTimes &t : ctx->tuned_narrow)
+      if (t.key == nkey) return TunedShape{narrow_group(t, g->n, k, k1), t.res_blocks};
+  NarrowTimes times{nkey, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, 0};
   for (const auto &e : ctx->tuned_groups)
-    if (e.first == key) return TunedShape{e.second >> 16, (int)(e.second & 0xFFFF)};
+    if (e.first == key) {
+      if (!narrow) return TunedShape{e.second >> 16, (int)(e.second & 0xFFFF)};
+      times.res_blocks = (int)(e.second & 0xFFFF);  // tuned for a graph of this class
+    }
   std::vector<int64_t> cands;
-  if (gmax == kChunk && !state_fits(g->n, kChunk)) cands = {32, 64};
+  if (narrow) cands = {32, 64};
   for (int64_t c = kChunk; c < gmax; c *= 2) cands.push_back(c);
   cands.push_back(gmax);
   int64_t best = gmax;
@@ -1393,7 +1427,7 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
     }
     double best_score = 0.0;
     int st = PPRVIZ_OK;
-    for (int64_t G : cands) {
+    for (const int64_t &G : cands) {
       if (cands.size() == 1) break;
       const size_t bytes = sizeof(float) * (size_t)(g->n * G);
       if ((st = ws_ensure(ctx, WS_Y0, bytes)) != PPRVIZ_OK) break;
@@ -1417,6 +1451,23 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
         st = cuda_err(ctx, ce, "autotuner timing");
         break;
       }
+      if (narrow) {  // one residual pass, after one untimed
+        const int slot = (int)(&G - cands.data());
+        times.sweep[slot] = ms / 3.0f;
+        if ((st = ws_ensure(ctx, WS_CERT, 2 * sizeof(double) * (size_t)G)) != PPRVIZ_OK) break;
+        for (int rep = 0; rep < 2 && st == PPRVIZ_OK; ++rep) {
+          if (rep == 1) cudaEventRecord(e0, ctx->stream);
+          st = launch_residual<float, false>(ctx, g, G, src, ya, nullptr, nullptr, ctx->ws[WS_CERT].as<double>(), 0.15);
+        }
+        if (st != PPRVIZ_OK) break;
+        cudaEventRecord(e1, ctx->stream);
+        if ((ce = cudaEventSynchronize(e1)) != cudaSuccess ||
+            (ce = cudaEventElapsedTime(&times.residual[slot], e0, e1)) != cudaSuccess) {
+          st = cuda_err(ctx, ce, "autotuner timing");
+          break;
+        }
+        continue;
+      }
       const double score = (double)ms * (double)((k + G - 1) / G);
       if (best_score == 0.0 || score < best_score) {
         best_score = score;
@@ -1425,7 +1476,9 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
     }
     // the residual's CTA count at the chosen width (only where its state fits in L2)
     const bool fits_l2 = (double)g->n * (double)best * 8.0 <= 64.0 * 1024 * 1024;
-    if (st == PPRVIZ_OK && fits_l2 && g->n >= 8 * 608) {
+    if (times.res_blocks) {
+      best_res = times.res_blocks;
+    } else if (st == PPRVIZ_OK && fits_l2 && g->n >= 8 * 608) {
       const size_t bytes = sizeof(float) * (size_t)(g->n * best);
       if (st == PPRVIZ_OK) st = ws_ensure(ctx, WS_Y0, bytes);
       if (st == PPRVIZ_OK) st = ws_ensure(ctx, WS_Y1, bytes);
@@ -1467,7 +1520,12 @@ TunedShape tuned_shape(pprviz_ctx *ctx, const pprviz_graph *g, int32_t k, int *s
       return TunedShape{gmax, 1216};
     }
   }
-  ctx->tuned_groups.push_back({key, (best << 16) | best_res});
+  if (!times.res_blocks) ctx->tuned_groups.push_back({key, (best << 16) | best_res});
+  if (narrow) {
+    times.res_blocks = best_res;
+    ctx->tuned_narrow.push_back(times);
+    best = narrow_group(times, g->n, k, k1);
+  }
   return TunedShape{best, best_res};
 }
 
@@ -1635,37 +1693,10 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
     dense = dense_prepare(ctx, g) == PPRVIZ_OK;
     if (!dense) ctx->err.clear();
   }
-  int64_t ld = 0;
-  int res_blocks = 1216;
-  if (dense) {
-    ld = dense_group(k);
-  } else if (fp64) {
-    ld = choose_group(g->n, k, elem);
-  } else {
-    int ts = PPRVIZ_OK;
-    const TunedShape sh = tuned_shape(ctx, g, k, &ts);
-    PPRVIZ_TRY(ts);
-    ld = sh.group;
-    res_blocks = sh.res_blocks;
-  }
-  const size_t sbytes = elem * (size_t)(g->n * ld);
   const double c = 1.0 - alpha;
-  PPRVIZ_TRY(ws_ensure(ctx, WS_Y0, sbytes));
-  PPRVIZ_TRY(ws_ensure(ctx, WS_Y1, sbytes));
-  if (!fp64) {
-    PPRVIZ_TRY(ws_ensure(ctx, WS_Y2, sbytes));
-    PPRVIZ_TRY(ws_ensure(ctx, WS_Y3, sbytes));
-    PPRVIZ_TRY(ws_ensure(ctx, WS_RHS, sbytes));
-  }
-  PPRVIZ_TRY(ws_ensure(ctx, WS_SRC, sizeof(int32_t) * (size_t)ld));
-  PPRVIZ_TRY(ws_ensure(ctx, WS_CERT, 2 * sizeof(double) * (size_t)ld));
-  int32_t *src = ctx->ws[WS_SRC].as<int32_t>();
-  double *l1 = ctx->ws[WS_CERT].as<double>();
   // deflated sweeps (FP32): component roots and the spectral bound of the graph
   bool defl = false;
   double bsp = 1.0;
-  int32_t *csrc = nullptr;
-  double *kappa = nullptr;
   // a directed walk is not reversible: its spectrum is complex, so the FP32
   // path runs power sweeps (the Chebyshev weights with an interval of width 0)
   // instead of Chebyshev sweeps, from a start that carries the dominant mode
@@ -1679,6 +1710,39 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
     defl = g->spec_deflate;
     bsp = defl ? g->spec_b : 1.0;
   }
+  // rate of the iterated modes on [1 - delta, 1 + delta] (power sweeps: c)
+  auto rate = [power, &prate](double delta) { return power ? prate : (delta > 1e-12 ? chebyshev_rate(delta) : 0.0); };
+  auto sweeps_for = [](double factor, double r) {  // K with 2 r^K <= factor
+    return r > 0.0 ? (int)ceil(log(0.5 * factor) / log(r)) : 1;
+  };
+  int64_t ld = 0;
+  int res_blocks = 1216;
+  if (dense) {
+    ld = dense_group(k);
+  } else if (fp64) {
+    ld = choose_group(g->n, k, elem);
+  } else {
+    int ts = PPRVIZ_OK;
+    const int k1 = sweeps_for(1e-5, perron ? c * g->per_b : rate(power ? 0.0 : c * bsp));
+    const TunedShape sh = tuned_shape(ctx, g, k, k1, &ts);
+    PPRVIZ_TRY(ts);
+    ld = sh.group;
+    res_blocks = sh.res_blocks;
+  }
+  const size_t sbytes = elem * (size_t)(g->n * ld);
+  PPRVIZ_TRY(ws_ensure(ctx, WS_Y0, sbytes));
+  PPRVIZ_TRY(ws_ensure(ctx, WS_Y1, sbytes));
+  if (!fp64) {
+    PPRVIZ_TRY(ws_ensure(ctx, WS_Y2, sbytes));
+    PPRVIZ_TRY(ws_ensure(ctx, WS_Y3, sbytes));
+    PPRVIZ_TRY(ws_ensure(ctx, WS_RHS, sbytes));
+  }
+  PPRVIZ_TRY(ws_ensure(ctx, WS_SRC, sizeof(int32_t) * (size_t)ld));
+  PPRVIZ_TRY(ws_ensure(ctx, WS_CERT, 2 * sizeof(double) * (size_t)ld));
+  int32_t *src = ctx->ws[WS_SRC].as<int32_t>();
+  double *l1 = ctx->ws[WS_CERT].as<double>();
+  int32_t *csrc = nullptr;
+  double *kappa = nullptr;
   if (!fp64) {
     PPRVIZ_TRY(ws_ensure(ctx, WS_CSRC, sizeof(int32_t) * (size_t)ld));
     PPRVIZ_TRY(ws_ensure(ctx, WS_KAPPA, sizeof(double) * (size_t)ld));
@@ -1698,11 +1762,6 @@ int dppr_solve(pprviz_ctx *ctx, const pprviz_graph *g, const int32_t *view_d,
   std::vector<int32_t> srch((size_t)ld);
   std::vector<double> cert;
   bool not_converged = false;
-  // rate of the iterated modes on [1 - delta, 1 + delta] (power sweeps: c)
-  auto rate = [power, &prate](double delta) { return power ? prate : (delta > 1e-12 ? chebyshev_rate(delta) : 0.0); };
-  auto sweeps_for = [](double factor, double r) {  // K with 2 r^K <= factor
-    return r > 0.0 ? (int)ceil(log(0.5 * factor) / log(r)) : 1;
-  };
   // the compensated FP32 residual resolves certificates down to ~1e-9; below
   // that the neighbour sums are accumulated in FP64
   const bool exact_res = eps < 1e-9;
