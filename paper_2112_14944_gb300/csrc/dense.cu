@@ -667,7 +667,7 @@ static int dsweep_tf32(pprviz_ctx *ctx, const pprviz_graph *g, int64_t ld, const
   const int64_t mw = (g->n + 127) / 128 * 128;
   const dim3 grid((unsigned)(ld / NT), (unsigned)(mw / dtc::TM));
   const uint64_t limit_ns = 2000000000ull;  // bounded waits: 2 s
-  const int withhold = ctx->expire_here() ? 0 : -1;
+  const int withhold = g->dense_nw / dtc::KC > C::NST && ctx->expire_here() ? 0 : -1;
   PPRVIZ_PROF(ctx, PPRVIZ_K_SWEEP);
   k_dsweep_ws<NT, RHS><<<grid, dws::THREADS, C::SMEM, ctx->stream>>>(
       g->n, g->dense_nw, ld, g->dense.as<float>(), g->invdw_f.as<float>(), src, rhs, ycur, yold, yold,

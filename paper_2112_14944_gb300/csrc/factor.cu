@@ -1093,7 +1093,7 @@ static int spd_inverse(pprviz_ctx *ctx, int32_t kp, T *A, T *work, int *err) {
     int nsm = 0;
     PPRVIZ_CUDA(ctx, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     const uint64_t limit_ns = 2000000000ull;  // bounded waits: 2 s
-    int withhold = ctx->expire_here() ? 0 : -1;  // consumed by the first main trailing launch
+    int withhold = nblk > 1 && ctx->expire_here() ? 0 : -1;  // consumed by the first main trailing launch
     PPRVIZ_PROF(ctx, PPRVIZ_K_FACTOR);
     float *Af = (float *)A;
     k_fac_diag128<<<1, DIAG128_THREADS, 0, ctx->stream>>>(kp, 0, Af, (float *)P[0]);

@@ -1355,7 +1355,7 @@ int resident_updates(pprviz_ctx *ctx, int32_t k, int32_t kp, int iters, const fl
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int withhold = ctx->expire_here() ? 1 : 0;
+  const int withhold = grid > 1 && ctx->expire_here() ? 1 : 0;
   PPRVIZ_PROF(ctx, PPRVIZ_K_LY);
   const cudaError_t e =
       cudaLaunchKernelEx(&cfg, kernel, k, kp, kq, nrows, iters, W1, M, X, B, bar, err, limit_ns, withhold);

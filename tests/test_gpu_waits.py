@@ -47,6 +47,23 @@ def test_resident_layout_barrier(ctx, k):
     expires(ctx, 2, lambda: ctx.layout(delta, x0, 3, P.FP32))
 
 
+def test_launches_without_a_wait_are_not_counted(ctx):
+    """One pivot block and one CTA wait for nobody: the aid passes over them."""
+    import paper_2112_14944_gb300 as P
+    from paper_2112_14944_gb300 import _binding as B
+    small, large = np.full((4, 4), 3.0, np.float32), np.full((300, 300), 3.0, np.float32)
+    np.fill_diagonal(small, 0)
+    np.fill_diagonal(large, 0)
+    x4, x300 = synth.uniform_x0(4, seed=1), synth.uniform_x0(300, seed=1)
+    good = ctx.layout(small, x4, 2, P.FP32)[0]
+    B.pprviz_test_expire_wait(ctx.h)
+    B.pprviz_test_expire_wait(ctx.h)
+    assert np.array_equal(ctx.layout(small, x4, 2, P.FP32)[0], good)
+    with pytest.raises(P.PPRVizError) as ei:
+        ctx.layout(large, x300, 2, P.FP32)
+    assert ei.value.status == B.PPRVIZ_E_TIMEOUT
+
+
 @pytest.mark.parametrize("columns", [128, 300])  # 128- and 256-wide tiles
 @pytest.mark.parametrize("sweep", [1, 3])
 def test_tensor_core_sweep(ctx, columns, sweep):
